@@ -6,31 +6,36 @@
 //   a in [0, p) is centred to s in [-(p-1)/2, (p-1)/2] and split exactly as
 //   s = 256 h + l with l in [-128, 127], h in [-128, 128].  Every digit is an
 //   exact fp16 value and every digit product is an integer of magnitude at
-//   most 2^14, so 1024 of them sum to at most 2^24: exact in an fp32
-//   accumulator.  A and B digits therefore go through tcgen05.mma kind::f16
-//   with fp32 accumulation in TMEM, and every 1024 terms (the exact chunk,
-//   Eq. (1) read with m = 24 for the fp32 significand) the four digit-product
-//   accumulators are recombined as hh*2^16 + (hl + lh)*2^8 + ll in int64,
-//   reduced mod p, and summed as residues.  Nothing is approximated.
-//   Roles per CTA (one CTA per SM, persistent over (tile, chunk) units):
-//     warp 0      TMA-loads uint32 A boxes (two 64-deep k-blocks per slot)
-//                 from HBM into a ring of shared-memory slots (a prepared A:
-//                 bulk-copies its 8-bit digit planes, one k-block per slot)
-//     warp 1      owns TMEM and issues the MMAs (one thread)
-//     warp 2      bulk-copies the pre-split B digit tiles (own ring)
-//     warps 3-10  read a landed A box into registers, centre and split it,
-//                 and write the two fp16 digit tiles in place over it
-//                 (128-byte-swizzled, K-major), the same 32 KiB per k-block
-//                 (a prepared A: widen its 8-bit digits to the same tiles)
-//     warps 11-14 drain the accumulators (tcgen05.ld), recombine, reduce
-//   B's digits are stacked [hi | lo] along N (N = 128 per MMA), so one MMA
-//   per A digit yields both products with that digit; the two MMAs of a K
-//   step accumulate into separate TMEM columns (two independent chains).
-//   Units of one output tile may be split over several CTAs: each adds its
-//   residue sums for the tile into a column-major u32 workspace (coalesced
-//   atomics, one transaction per column and warp), and a small kernel behind
-//   this one reduces the sums mod p, writes C through a shared-memory
-//   transpose and clears the workspace.
+//   most 2^14.  The digit products go through tcgen05.mma kind::f16 into fp32
+//   accumulators in TMEM, three per output: hh, hl + lh and ll.  The middle
+//   one takes two products per term, so 512 terms sum to at most 2^24: exact
+//   (Eq. (1) read with m = 24 for the fp32 significand).  After each such
+//   chunk the accumulators are recombined as (hh 256 + (hl + lh)) 256 + ll mod
+//   p and added to the output's residue sum.  Nothing is approximated.
+//
+//   A work unit is one 128-row tile of A times one K range of at most 512
+//   terms (eight 64-deep k-blocks) of one 64-column tile of B.  Units are
+//   ordered with the row tiles innermost and split evenly over one persistent
+//   CTA per SM, so a CTA works through many row tiles against the same K
+//   range: that range's B digits (128 KiB) stay in shared memory and are made
+//   once per range, and A alone streams.  A's digits go to TMEM, from where
+//   the MMAs read them: shared memory sees only B, and the rest of its 256 KiB
+//   per SM stays L1, which is where loads in flight land.  Roles per CTA:
+//     warps 0-7    load A with 16-byte loads, 24 in flight per thread (96 KiB
+//                  per SM), centre and split the words in registers and store
+//                  the fp16 digits (tcgen05.st) to one of two TMEM slots.  No
+//                  warp waits for another: slots pass through mbarriers alone
+//     warps 8-15   drain the accumulators (tcgen05.ld), recombine, reduce and
+//                  add the residues to the partial sums
+//     warp 16      owns TMEM and issues the MMAs (one thread)
+//     warp 17      bulk-copies B's digit tiles, split once by a small kernel
+//                  before this one, each as soon as the MMAs of the K range
+//                  before have read its place for the last time
+//   Each output meets the partial sums of its K ranges in a column-major u32
+//   workspace (coalesced atomics, one transaction per column and warp), and a
+//   small kernel behind this one reduces the sums mod p, writes C through a
+//   shared-memory transpose and clears the workspace; a product with a single
+//   K range writes C directly.
 //
 // Larger moduli on the tensor cores (p > 65791): the exact integer products
 // sum_t A[i][t] B[t][j] are below k (p-1)^2, so they are fixed by their
@@ -42,8 +47,6 @@
 //
 // CUDA-core path (any p <= 2^32-1): shared-memory tiled product with the
 // per-thread unreduced accumulators of the dot-product kernels.
-#include <cuda.h>
-#include <cudaTypedefs.h>
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -59,78 +62,85 @@ namespace blk {
 constexpr int BM = 128;            // rows per tile (MMA M)
 constexpr int BK = 64;             // K per k-block: one 128-byte swizzle row of fp16
 constexpr int NT = 64;             // output columns per n-tile
-constexpr int MMA_N = 2 * NT;      // hi and lo digits of B stacked along N
-constexpr int KC = 16;             // k-blocks per exact chunk (1024 terms)
-constexpr int A_TILE_BYTES = BM * BK * 4;                     // 32 KiB of uint32 per k-block
-constexpr int A_DIGIT_BYTES = BM * BK * 2;                    // 16 KiB per digit
+constexpr int MMA_N = 2 * NT;      // low and high digits of B stacked along N
+constexpr int RK = 8;              // k-blocks per K range at most: 512 terms, the exact chunk
 constexpr int B_TILE_BYTES = MMA_N * BK * 2;                  // 16 KiB
-static_assert(A_TILE_BYTES == 2 * A_DIGIT_BYTES, "in-place conversion needs equal sizes");
-constexpr int CONV_WARPS = 8;
-constexpr int EPI_WARPS = 4;
-constexpr int W_APROD = 0, W_MMA = 1, W_BPROD = 2, W_CONV0 = 3, W_EPI0 = W_CONV0 + CONV_WARPS;
-constexpr int THREADS = 32 * (W_EPI0 + EPI_WARPS);            // 480
-constexpr uint32_t TMEM_COLS = 512;   // 2 accumulator sets x 2 digits x 128 columns
+// A's digits live in TMEM: two slots of one k-block each
+constexpr int SLOTS = 2;
+constexpr uint32_t SLOT_COLS = 64;                            // 32 columns per digit
+constexpr uint32_t ACC_COLS = 3 * NT;                         // ll, middle, hh
+constexpr uint32_t A_COL0 = 2 * ACC_COLS;                     // behind two accumulator sets
+constexpr int CONV_WARPS = 8, EPI_WARPS = 8;
+constexpr int W_EPI0 = CONV_WARPS, W_MMA = CONV_WARPS + EPI_WARPS, W_BPROD = W_MMA + 1;
+constexpr int THREADS = 32 * (W_MMA + 4);                     // 640: two warps of the last group idle
+// registers per thread: 96 at launch, then shared out by role (warpgroups)
+constexpr int REGS_LAUNCH = 96, REGS_CONV = 152, REGS_EPI = 64, REGS_MMA = 48;
+static_assert(REGS_LAUNCH * THREADS == 32 * (REGS_CONV * CONV_WARPS + REGS_EPI * EPI_WARPS + REGS_MMA * 4),
+              "the roles' registers are exactly those the block is launched with");
+static_assert(REGS_LAUNCH * THREADS <= 65536, "one CTA per SM");
+static_assert(W_EPI0 % 4 == 0, "an epilogue warp reads the TMEM lanes of its index modulo 4");
+constexpr uint32_t TMEM_COLS = 512;
+static_assert(A_COL0 + SLOTS * SLOT_COLS == TMEM_COLS, "accumulators and A digits fill TMEM");
 constexpr uint64_t WAIT_NS = 2000000000ull;   // bounded waits: 2 s
 constexpr uint32_t IDESC = ptx::idesc_f16_f32(BM, MMA_N);
+constexpr uint32_t IDESC_HALF = ptx::idesc_f16_f32(BM, NT);
+// terms of one launch: 2^24 / 512 partial sums below p <= 65791, and one more
+// (the sums of earlier launches, folded below p), stay below 2^32
+constexpr uint64_t SLAB_K = 1ull << 24;
 
-// Pipeline depths: SLOTS shared-memory slots of KBB k-blocks of A each, and
-// BSTAGES B digit tiles.  A slot receives a uint32 box (TMA) that the
-// converter warps turn into fp16 digit tiles in place, or, for a prepared A,
-// a tile of 8-bit digit planes (bulk copy) that they widen in place.  The
-// uint32 path measured fastest with three two-k-block slots (longer TMA row
-// bursts) and two B stages; the prepared path with five one-k-block slots
-// and four B stages.
-template <int SLOTS_, int BSTAGES_, int KBB_>
-struct Pipe {
-    static constexpr int SLOTS = SLOTS_, BSTAGES = BSTAGES_, KBB = KBB_;
-    static constexpr int SLOT_BYTES = KBB * A_TILE_BYTES;
-    struct Bars {
-        uint64_t a_full[SLOTS];    // A tile landed (1 arrival + tx bytes)
-        uint64_t conv[SLOTS];      // digits written in place (one arrival per converter warp)
-        uint64_t a_empty[SLOTS];   // MMAs reading the digits completed (tcgen05.commit)
-        uint64_t full_b[BSTAGES];  // B digit tile landed (1 arrival + tx bytes)
-        uint64_t empty_b[BSTAGES]; // MMAs reading the B tile completed (tcgen05.commit)
-        uint64_t acc_full[2];      // accumulator set ready (tcgen05.commit)
-        uint64_t acc_empty[2];     // accumulator set drained (one arrival per epilogue warp)
-        uint64_t drain;            // all MMAs issued by this CTA completed
-        uint32_t tmem_base;
-        uint32_t abort;
-    };
-    static constexpr size_t SMEM_BYTES = 1024 /*alignment slack*/ + (size_t)SLOTS * SLOT_BYTES +
-                                         (size_t)BSTAGES * B_TILE_BYTES + 1024;
-    static_assert(sizeof(Bars) <= 1024, "barriers fit their reserve");
-    static_assert(SMEM_BYTES <= 232448, "shared memory per block");
+struct Bars {
+    uint64_t conv[SLOTS];      // digits of a slot written (one arrival per converter warp)
+    uint64_t a_empty[SLOTS];   // MMAs reading the slot completed (tcgen05.commit)
+    uint64_t b_full[RK];       // B digit tile landed (1 arrival + tx bytes)
+    uint64_t b_empty[RK];      // last MMAs reading the tile completed (tcgen05.commit)
+    uint64_t acc_full[2];      // accumulator set ready (tcgen05.commit)
+    uint64_t acc_empty[2];     // accumulator set drained (one arrival per epilogue warp)
+    uint64_t drain;            // all MMAs issued by this CTA completed
+    uint32_t tmem_base;
+    uint32_t abort;
 };
-using PipeU32 = Pipe<3, 2, 2>;    // uint32 A, converted in place
-using PipePrep = Pipe<5, 4, 1>;   // prepared A: 8-bit digit planes, widened in place
-static_assert(PipePrep::KBB == 1, "one prepared tile per slot");
+constexpr size_t SMEM_BYTES = 1024 /*alignment slack*/ + (size_t)RK * B_TILE_BYTES + 1024;
+static_assert(sizeof(Bars) <= 1024, "barriers fit their reserve");
+static_assert(SMEM_BYTES <= 232448, "shared memory per block");
 
-// Prepared A (gfp_block_prepare): per (m-tile, k-block) two planes of 8-bit
-// digits, high then low, each 128 rows x 64 K, row-major, every digit stored
-// with a bias of 128.  A residue a of p <= 65536 is represented by s = a or
-// a - p in [-32896, 32639] (s = a when a <= min((p-1)/2, 32639)), split as
+// How A arrives: uint32 rows that 16-byte loads can take, uint32 rows of any
+// alignment, or prepared 8-bit digit planes.
+enum AMode : int { A_VEC = 0, A_ANY = 1, A_PREP = 2 };
+
+// Prepared A (gfp_block_prepare): per (m-tile, k-block) the 8-bit digits of
+// 128 rows x 64 K, in the order the converter lanes of the product take them:
+// for each of the eight converter warps 1 KiB of high and 1 KiB of low
+// digits, 16 bytes a lane at a time (AWords), every digit stored with a bias of 128.  A
+// residue a of p <= 65536 is represented by s = a or a - p in
+// [-32896, 32639] (s = a when a <= min((p-1)/2, 32639)), split as
 // s = 256 h + l with h, l in [-128, 127]: u = s + 32896 in [0, 65535] holds
 // h + 128 in its high byte and l + 128 in its low byte.  Every digit is still
-// at most 128 in magnitude, so the 1024-term fp32 chunks stay exact.
-constexpr int A8_PLANE_BYTES = BM * BK;           // 8 KiB per digit plane
-constexpr int A8_TILE_BYTES = 2 * A8_PLANE_BYTES; // 16 KiB per (m-tile, k-block)
+// at most 128 in magnitude, so the 512-term fp32 chunks stay exact.
+constexpr int A8_TILE_BYTES = 2 * BM * BK;        // 16 KiB per (m-tile, k-block)
 constexpr uint32_t DIGIT8_MAX_P = 65536;
 
 struct Args {
-    CUtensorMap tmap_a;       // A as a 2-D uint32 tensor {k, m}, box {BK*KBB, BM} (uint32 pipe), zero fill
-    uint64_t m, k, nb;
+    uint64_t m, k, nb;        // k: terms of this launch
+    const uint32_t *A;
+    uint64_t lda;
+    const uint8_t *Aimg;      // prepared A: [m_tiles][img_kblocks] tiles of A8_TILE_BYTES
+    uint32_t img_kblocks, img_kb0;   // k-blocks of the whole image, first one of this launch
     const uint8_t *Bimg;      // [n_tiles][kblocks] tiles of B_TILE_BYTES
-    const uint8_t *Aimg;      // prepared A: [m_tiles][kblocks] tiles of A8_TILE_BYTES (PREP)
     uint32_t *C;
     uint64_t ldc;
     uint32_t *Cacc;           // (n_tiles*NT) x m u32 partial residue sums, column-major: the
                               // entry of row i, column j at j*m + i (zero outside calls)
     uint32_t *err;            // bit 0: a bounded wait expired
-    Mod mod;
-    uint64_t off;             // multiple of p >= 2^41 making recombined values non-negative
-    uint32_t pre_magic;       // floor(2^32 / p) for the input reduction of the residue passes
-    uint32_t half;            // (p-1)/2
-    uint32_t m_tiles, n_tiles, kblocks, chunks;
+    uint32_t p, half;         // half = (p-1)/2
+    uint32_t magic;           // floor(2^32 / p)
+    int32_t smagic;           // the same, at most 2^31 - 1
+    uint32_t magic47;         // floor(2^47 / p) of a residue-pass modulus (p > 65000)
+    uint32_t direct;          // one K range: residues go to C, not to the workspace
+    uint32_t m_tiles, n_tiles, kblocks;
+    uint32_t ranges, r_base, r_rem;   // K ranges of r_base k-blocks, the first r_rem one more
+    uint32_t bsets;           // K ranges whose B tiles fit the RK tiles at once,
+    uint32_t bset_tiles;      // the distance between their tiles
+    uint32_t edge_m, edge_k;  // last row tile, last k-block where ragged (else none: ~0)
     uint64_t units;
 };
 
@@ -154,6 +164,15 @@ __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, volatile
             }
         }
     }
+}
+
+// The same for a converged warp: every lane polls (a lone polling lane adds
+// the cost of leaving and rejoining the warp, 506 against 318 cycles for a
+// hand-over of 16 warps to one and back), and all lanes agree on the result.
+__device__ __forceinline__ bool wait_bar_warp(uint32_t bar, uint32_t parity, volatile uint32_t *abort,
+                                              uint32_t *err)
+{
+    return __all_sync(0xffffffffu, wait_bar(bar, parity, abort, err));
 }
 
 // Failure-detection self test: one thread waits on an mbarrier that nothing
@@ -184,151 +203,225 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatil
     return __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
 }
 
-struct UnitPos {
-    uint32_t nt, mt, c, kb0, kb1;
-};
-
-__device__ __forceinline__ UnitPos unit_pos(const Args &a, uint64_t u)
-{
-    UnitPos q;
-    q.c = (uint32_t)(u % a.chunks);
-    const uint64_t tile = u / a.chunks;
-    q.mt = (uint32_t)(tile % a.m_tiles);
-    q.nt = (uint32_t)(tile / a.m_tiles);
-    q.kb0 = q.c * KC;
-    q.kb1 = min(q.kb0 + (uint32_t)KC, a.kblocks);
-    return q;
-}
-
-// Centre two residues and split each into balanced 8-bit digits, returned
-// as packed fp16 pairs (element 0 in the low half).  With u = s + 32896, where
-// s in [-32895, 32895] is the centred residue, the digits of s = 256 h + l are
-// l = (u & 255) - 128 and h = (u >> 8) - 128.  The fp16 encoding of 1536 + d
-// for an integer |d| <= 512 is the 16-bit integer 0x6600 + d (exponent of
-// [1024, 2048), unit spacing), so a byte permute plus one integer add builds
-// 1536 + d for both lanes and one exact fp16 subtraction leaves d.
-__device__ __forceinline__ void split_pair(uint32_t a0, uint32_t a1, uint32_t p, uint32_t half,
-                                           uint32_t &hi2, uint32_t &lo2)
-{
-    const uint32_t u0 = a0 + 32896u - (a0 > half ? p : 0u);
-    const uint32_t u1 = a1 + 32896u - (a1 > half ? p : 0u);
-    const uint32_t lo_bits = __byte_perm(u0, u1, 0x3430) + 0x65806580u;   // [u0 & 255, u1 & 255]
-    const uint32_t hi_bits = __byte_perm(u0, u1, 0x6521) + 0x65806580u;   // [u0 >> 8, u1 >> 8]
-    const __half2 bias = __halves2half2(__ushort_as_half(0x6600), __ushort_as_half(0x6600));
-    const __half2 lo = __hsub2(*reinterpret_cast<const __half2 *>(&lo_bits), bias);
-    const __half2 hi = __hsub2(*reinterpret_cast<const __half2 *>(&hi_bits), bias);
-    lo2 = *reinterpret_cast<const uint32_t *>(&lo);
-    hi2 = *reinterpret_cast<const uint32_t *>(&hi);
-}
-
-// Converter thread ct (0..255) handles 8 chunks of 4 consecutive K of one row.
-// load_tile copies them from the landed uint32 tile (row-major, 256 bytes per
-// row) into registers; once every converter thread has done so, store_digits
-// overwrites the same 32 KiB with the two 128-byte-swizzled K-major fp16
-// digit tiles (high digits first).
-struct ARegs {
-    uint4 v[8];
-};
-
-// sub-tile `sub` of a slot holding KBB k-blocks (row stride BK*4*KBB bytes)
-template <int KBB>
-__device__ __forceinline__ void load_tile(const uint8_t *slot, int sub, int ct, ARegs &r)
-{
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int q = ct + 256 * i;
-        const int row = q >> 4, c4 = q & 15;
-        r.v[i] = *reinterpret_cast<const uint4 *>(slot + row * (BK * 4 * KBB) + sub * (BK * 4) + c4 * 16);
+// Walks a CTA's units in order: row tiles innermost, then K ranges, then
+// column tiles.
+struct Walk {
+    uint32_t mt, rg, nt;
+    uint32_t kb0, kbs;   // first k-block and number of k-blocks of the K range
+    uint32_t left;       // units not finished, the current one included
+    __device__ __forceinline__ void range(const Args &a)
+    {
+        kb0 = rg * a.r_base + min(rg, a.r_rem);
+        kbs = a.r_base + (rg < a.r_rem ? 1u : 0u);
     }
+    __device__ __forceinline__ void start(const Args &a, uint64_t u0, uint64_t u1)
+    {
+        left = (uint32_t)(u1 - u0);
+        mt = (uint32_t)(u0 % a.m_tiles);
+        const uint64_t t = u0 / a.m_tiles;
+        rg = (uint32_t)(t % a.ranges);
+        nt = (uint32_t)(t / a.ranges);
+        range(a);
+    }
+    // to the next unit; true when its K range or column tile is another one
+    __device__ __forceinline__ bool next(const Args &a)
+    {
+        --left;
+        if (++mt < a.m_tiles) return false;
+        mt = 0;
+        if (++rg == a.ranges) {
+            rg = 0;
+            ++nt;
+        }
+        range(a);
+        return true;
+    }
+};
+
+// Two values u = s + 32896 (s the representative, in [-32896, 32895]) to the
+// balanced 8-bit digits l = (u & 255) - 128 and h = (u >> 8) - 128 of
+// s = 256 h + l, as packed fp16 pairs (element 0 in the low half).  The fp16
+// encoding of 1024 + b for an integer 0 <= b <= 256 is the 16-bit integer
+// 0x6400 + b, so with U_BIAS added to u (0x64 in its two upper bytes; u = 2^16
+// and above carries into the lower of them, as 0x6400 + 256 wants it) one byte
+// permute builds 1024 + b for both lanes and one exact fp16 subtraction of
+// 1152 leaves the digits.
+constexpr uint32_t U_BIAS = 0x64640000u + 32896u;
+
+__device__ __forceinline__ uint32_t sub_half2(uint32_t x, uint32_t half_bits)
+{
+    const __half2 b = __halves2half2(__ushort_as_half((unsigned short)half_bits),
+                                     __ushort_as_half((unsigned short)half_bits));
+    const __half2 r = __hsub2(*reinterpret_cast<const __half2 *>(&x), b);
+    return *reinterpret_cast<const uint32_t *>(&r);
+}
+
+__device__ __forceinline__ void split_u(uint32_t u0, uint32_t u1, uint32_t &hi2, uint32_t &lo2)
+{
+    lo2 = sub_half2(__byte_perm(u0, u1, 0x7430), 0x6480u);   // bytes 0 and 3 of each
+    hi2 = sub_half2(__byte_perm(u0, u1, 0x6521), 0x6480u);   // bytes 1 and 2 of each
 }
 
 // a mod p for any 32-bit a and p <= 65791: q = floor(a * floor(2^32/p) / 2^32)
 // is floor(a/p) or one less, so one conditional subtraction finishes it
 __device__ __forceinline__ uint32_t reduce_small(uint32_t a, uint32_t p, uint32_t magic)
 {
-    uint32_t r = a - __umulhi(a, magic) * p;
-    return r >= p ? r - p : r;
+    const uint32_t r = a - __umulhi(a, magic) * p;
+    return min(r, r - p);
+}
+
+// u = s + U_BIAS for the centred representative s of a residue a < p
+__device__ __forceinline__ uint32_t centre_u(uint32_t a, const Args &g)
+{
+    return a + (a > g.half ? U_BIAS - g.p : U_BIAS);
+}
+
+// u = s + U_BIAS with s = a (mod p) for any 32-bit a and a residue-pass modulus
+// 65000 < p < 65536: q = a / p rounded to nearest from the quotient to 15
+// fractional bits.  That quotient is low by less than two units of 2^-15
+// (magic47 by less than one part in 2^31, the multiply-high by less than one
+// unit), so |s| <= p/2 + 2 p / 32768 < 32896 - 100.
+__device__ __forceinline__ uint32_t reduce_u(uint32_t a, const Args &g)
+{
+    const uint32_t q = (__umulhi(a, g.magic47) + 16384u) >> 15;
+    return a + U_BIAS - q * g.p;
 }
 
 template <bool PRE>
-__device__ __forceinline__ void store_digits(const Args &a, const ARegs &r, uint8_t *stage, int ct)
+__device__ __forceinline__ void split4(const uint4 &w, const Args &a, uint32_t &hi01, uint32_t &hi23,
+                                       uint32_t &lo01, uint32_t &lo23)
 {
-    uint8_t *th = stage;                    // high digits
-    uint8_t *tl = stage + A_DIGIT_BYTES;    // low digits
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int q = ct + 256 * i;
-        const int row = q >> 4, c4 = q & 15;
-        uint32_t h01, l01, h23, l23;
-        uint4 w = r.v[i];
-        if (PRE) {
-            w.x = reduce_small(w.x, a.mod.p, a.pre_magic);
-            w.y = reduce_small(w.y, a.mod.p, a.pre_magic);
-            w.z = reduce_small(w.z, a.mod.p, a.pre_magic);
-            w.w = reduce_small(w.w, a.mod.p, a.pre_magic);
+    const uint32_t u0 = PRE ? reduce_u(w.x, a) : centre_u(w.x, a);
+    const uint32_t u1 = PRE ? reduce_u(w.y, a) : centre_u(w.y, a);
+    const uint32_t u2 = PRE ? reduce_u(w.z, a) : centre_u(w.z, a);
+    const uint32_t u3 = PRE ? reduce_u(w.w, a) : centre_u(w.w, a);
+    split_u(u0, u1, hi01, lo01);
+    split_u(u2, u3, hi23, lo23);
+}
+
+// Four biased 8-bit digits to fp16 pairs: a byte b under 0x64 is 1024 + b
+__device__ __forceinline__ void widen4(uint32_t w, uint32_t &d01, uint32_t &d23)
+{
+    d01 = sub_half2(__byte_perm(w, 0x64646464u, 0x4140), 0x6480u);
+    d23 = sub_half2(__byte_perm(w, 0x64646464u, 0x4342), 0x6480u);
+}
+
+// What one converter lane holds of a k-block of A.  Warp w writes the TMEM
+// lanes (rows) 32 (w mod 4) + 16 (w / 4) .. + 15; with the 16x256b store shape
+// lane l holds, per 16 K, four consecutive K (l mod 4) of rows l / 4 and
+// l / 4 + 8.  v[i] are those pieces: K group i / 2, row l / 4 + 8 (i mod 2); for
+// uint32 A 16 bytes each (the four groups of a row are 256 consecutive bytes),
+// for a prepared A the four bytes of one word: v[0], v[1] the high digits of K
+// groups 0, 1 and 2, 3, v[2], v[3] the low ones.  Rows and columns outside the
+// matrix are zero.
+template <int MODE>
+struct AWords {
+    uint4 v[MODE == A_PREP ? 4 : 8];
+};
+
+// Runs ahead of the conversion: where the next k-block's words are.
+template <int MODE>
+struct ALoads {
+    Walk w;
+    uint32_t j;           // k-block within the K range
+    const uint8_t *src;   // this lane's first piece of that k-block
+    __device__ __forceinline__ void locate(const Args &a, int warp, int lane)
+    {
+        j = 0;
+        if constexpr (MODE == A_PREP) {
+            src = a.Aimg + ((uint64_t)w.mt * a.img_kblocks + a.img_kb0 + w.kb0) * A8_TILE_BYTES + warp * 2048 +
+                  lane * 16;
+        } else {
+            const uint64_t row = (uint64_t)w.mt * BM + (warp & 3) * 32 + (warp >> 2) * 16 + (lane >> 2);
+            const uint64_t col = (uint64_t)w.kb0 * BK + (lane & 3) * 4;
+            src = reinterpret_cast<const uint8_t *>(a.A + row * a.lda + col);
         }
-        split_pair(w.x, w.y, a.mod.p, a.half, h01, l01);
-        split_pair(w.z, w.w, a.mod.p, a.half, h23, l23);
-        // 128-byte swizzle: 16-byte chunk j of row r sits at chunk j ^ (r & 7)
-        const int j = c4 >> 1, halfsel = c4 & 1;
-        const uint32_t off = (uint32_t)row * 128u + ((uint32_t)(j ^ (row & 7)) << 4) + (halfsel << 3);
-        *reinterpret_cast<uint2 *>(th + off) = make_uint2(h01, h23);
-        *reinterpret_cast<uint2 *>(tl + off) = make_uint2(l01, l23);
     }
-}
-
-// A prepared tile's 16-byte chunk c of 1024 (thread ct takes c = ct + 256 i):
-// plane c / 512, row (c / 4) mod 128, K columns 16 (c mod 4) .. + 15.  Its
-// 16 biased bytes become 16 fp16 digits: the fp16 encoding of 1408 + b for a
-// byte b is the 16-bit integer 0x6580 + b, and one exact subtraction of 1536
-// leaves b - 128.  The two 8-digit halves land at their 128-byte-swizzled
-// places of the plane's fp16 tile (high digits at slot offset 0, low at
-// A_DIGIT_BYTES), the layout the MMAs read.
-__device__ __forceinline__ void widen_store(uint8_t *slot, int c, uint4 w)
-{
-    const int d = c >> 9, row = (c >> 2) & 127, j = c & 3;
-    const __half2 bias = __halves2half2(__ushort_as_half(0x6600), __ushort_as_half(0x6600));
-    const uint32_t in[4] = {w.x, w.y, w.z, w.w};
-    uint32_t o[8];
+    // to the next k-block; the last one of the CTA is its own successor, so that
+    // the loads need no condition and write straight to their registers
+    __device__ __forceinline__ void step(const Args &a, int warp, int lane)
+    {
+        if (++j < w.kbs) {
+            src += MODE == A_PREP ? A8_TILE_BYTES : BK * 4;
+        } else if (w.left > 1) {
+            w.next(a);
+            locate(a, warp, lane);
+        } else {
+            --j;
+        }
+    }
+    __device__ __forceinline__ void load(const Args &a, int warp, int lane, AWords<MODE> &r) const
+    {
+        if constexpr (MODE == A_PREP) {
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        const uint32_t b01 = __byte_perm(in[e], 0u, 0x4140) + 0x65806580u;   // bytes 0, 1
-        const uint32_t b23 = __byte_perm(in[e], 0u, 0x4342) + 0x65806580u;   // bytes 2, 3
-        const __half2 h01 = __hsub2(*reinterpret_cast<const __half2 *>(&b01), bias);
-        const __half2 h23 = __hsub2(*reinterpret_cast<const __half2 *>(&b23), bias);
-        o[2 * e] = *reinterpret_cast<const uint32_t *>(&h01);
-        o[2 * e + 1] = *reinterpret_cast<const uint32_t *>(&h23);
+            for (int i = 0; i < 4; ++i) ptx::ld_stream4(r.v[i], src + i * 512);
+        } else if (w.mt != a.edge_m && w.kb0 + j != a.edge_k) {
+            const uint8_t *src8 = src + 32 * a.lda;   // eight rows further
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const uint8_t *q = ((i & 1) ? src8 : src) + (i >> 1) * 64;
+                if constexpr (MODE == A_VEC) {
+                    ptx::ld_stream4(r.v[i], q);
+                } else {
+                    const uint32_t *q1 = reinterpret_cast<const uint32_t *>(q);
+                    ptx::ld_if(r.v[i].x, q1, true);
+                    ptx::ld_if(r.v[i].y, q1 + 1, true);
+                    ptx::ld_if(r.v[i].z, q1 + 2, true);
+                    ptx::ld_if(r.v[i].w, q1 + 3, true);
+                }
+            }
+        } else {
+            const uint64_t row = (uint64_t)w.mt * BM + (warp & 3) * 32 + (warp >> 2) * 16 + (lane >> 2);
+            const uint64_t col = (uint64_t)(w.kb0 + j) * BK + (lane & 3) * 4;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const uint32_t *q = reinterpret_cast<const uint32_t *>(src + (i & 1) * 32 * a.lda + (i >> 1) * 64);
+                const uint64_t c = col + (i >> 1) * 16;
+                // columns of this piece inside A
+                const uint64_t n = row + 8 * (i & 1) < a.m && c < a.k ? a.k - c : 0;
+                r.v[i] = make_uint4(0u, 0u, 0u, 0u);
+                ptx::ld_if(r.v[i].x, q, n > 0);
+                ptx::ld_if(r.v[i].y, q + 1, n > 1);
+                ptx::ld_if(r.v[i].z, q + 2, n > 2);
+                ptx::ld_if(r.v[i].w, q + 3, n > 3);
+            }
+        }
     }
-    uint8_t *tile = slot + (size_t)d * A_DIGIT_BYTES;
-    const uint32_t r7 = (uint32_t)(row & 7), base = (uint32_t)row * 128u;
-    *reinterpret_cast<uint4 *>(tile + base + (((uint32_t)(2 * j) ^ r7) << 4)) = make_uint4(o[0], o[1], o[2], o[3]);
-    *reinterpret_cast<uint4 *>(tile + base + (((uint32_t)(2 * j + 1) ^ r7) << 4)) = make_uint4(o[4], o[5], o[6], o[7]);
-}
+};
 
-// (x + y) mod p for x, y < p: the per-thread sums of chunk residues stay
-// below p however many chunks a long K holds, and the u32 partial sums that
-// meet in the workspace then add at most one such sum per contributing CTA
-__device__ __forceinline__ uint32_t add_mod(uint32_t x, uint32_t y, uint32_t p)
+// Splits (or widens) the lane's words into the digits of its 16 rows x 64 K,
+// in the order of the 16x256b store
+template <int MODE, bool PRE>
+__device__ __forceinline__ void convert_a(const Args &a, const AWords<MODE> &r, uint32_t (&hi)[16],
+                                          uint32_t (&lo)[16])
 {
-    const uint32_t t = x + y;
-    return t >= p ? t - p : t;
+    if constexpr (MODE == A_PREP) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            widen4(r.v[i].x, hi[8 * i], hi[8 * i + 1]);
+            widen4(r.v[i].y, hi[8 * i + 2], hi[8 * i + 3]);
+            widen4(r.v[i].z, hi[8 * i + 4], hi[8 * i + 5]);
+            widen4(r.v[i].w, hi[8 * i + 6], hi[8 * i + 7]);
+            widen4(r.v[2 + i].x, lo[8 * i], lo[8 * i + 1]);
+            widen4(r.v[2 + i].y, lo[8 * i + 2], lo[8 * i + 3]);
+            widen4(r.v[2 + i].z, lo[8 * i + 4], lo[8 * i + 5]);
+            widen4(r.v[2 + i].w, lo[8 * i + 6], lo[8 * i + 7]);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            split4<PRE>(r.v[i], a, hi[2 * i], hi[2 * i + 1], lo[2 * i], lo[2 * i + 1]);
+    }
 }
 
-// PRE: reduce each input modulo p while splitting it (the residue passes).
-// PREP: A arrives prepared, as 8-bit digit planes (k_block_prep_a); the
-// producer bulk-copies a 16 KiB tile into the upper half of a slot and the
-// converter warps widen it in place into the two fp16 digit tiles.
-template <bool PRE, bool PREP, class P>
+// PRE: reduce each entry of A modulo p while splitting it (the residue passes).
+template <int MODE, bool PRE>
 __global__ void __launch_bounds__(THREADS, 1) k_block_tc(const __grid_constant__ Args a)
 {
-    constexpr int SLOTS = P::SLOTS, BSTAGES = P::BSTAGES, KBB = P::KBB;
-    constexpr int SLOT_BYTES = P::SLOT_BYTES;
-    using Bars = typename P::Bars;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t *slot_mem = smem;                                  // SLOTS A slots
-    uint8_t *bst = smem + (size_t)SLOTS * SLOT_BYTES;          // BSTAGES B digit tiles
-    Bars *bars = reinterpret_cast<Bars *>(bst + (size_t)BSTAGES * B_TILE_BYTES);
+    uint8_t *btiles = smem;                                    // RK digit tiles of B
+    Bars *bars = reinterpret_cast<Bars *>(btiles + (size_t)RK * B_TILE_BYTES);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     const uint64_t u0 = a.units * blockIdx.x / gridDim.x;
@@ -336,13 +429,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_block_tc(const __grid_constant__
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < SLOTS; ++s) {
-            ptx::mbar_init(ptx::smem_u32(&bars->a_full[s]), 1);
             ptx::mbar_init(ptx::smem_u32(&bars->conv[s]), CONV_WARPS);
             ptx::mbar_init(ptx::smem_u32(&bars->a_empty[s]), 1);
         }
-        for (int s = 0; s < BSTAGES; ++s) {
-            ptx::mbar_init(ptx::smem_u32(&bars->full_b[s]), 1);
-            ptx::mbar_init(ptx::smem_u32(&bars->empty_b[s]), 1);
+        for (int t = 0; t < RK; ++t) {
+            ptx::mbar_init(ptx::smem_u32(&bars->b_full[t]), 1);
+            ptx::mbar_init(ptx::smem_u32(&bars->b_empty[t]), 1);
         }
         for (int b = 0; b < 2; ++b) {
             ptx::mbar_init(ptx::smem_u32(&bars->acc_full[b]), 1);
@@ -361,133 +453,107 @@ __global__ void __launch_bounds__(THREADS, 1) k_block_tc(const __grid_constant__
     ptx::tc_fence_after();
     const uint32_t tmem = bars->tmem_base;
     volatile uint32_t *abort = &bars->abort;
+    // Programmatic dependent launch: this grid may be placed while the previous
+    // kernel of the stream, the one that makes B's digits or reduces the partial
+    // sums of the pass before, is still running.  What came before that kernel
+    // is complete (it waited for it), so A may be read at once; the roles that
+    // touch B's digits or the partial sums wait for it.
 
-    if (warp == W_APROD) {
-        // ---------------- producer: uint32 A tiles (TMA) into free slots ----------------
-        if (lane == 0) {
-            int armed[SLOTS];
-            for (int s = 0; s < SLOTS; ++s) armed[s] = -1;
-            uint32_t si = 0;   // slot sequence number
-            bool ok = true;
-            if (!PREP) ptx::prefetch_tensormap(&a.tmap_a);
-            for (uint64_t u = u0; u < u1 && ok; ++u) {
-                const UnitPos q = unit_pos(a, u);
-                for (uint32_t kb = q.kb0; kb < q.kb1; kb += KBB, ++si) {
-                    const uint32_t s = si % SLOTS, round = si / SLOTS;
-                    if (round > 0 &&
-                        !wait_bar(ptx::smem_u32(&bars->a_empty[s]), (round - 1) & 1, abort, a.err)) {
-                        ok = false;
-                        break;
-                    }
-                    const uint32_t fb = ptx::smem_u32(&bars->a_full[s]);
-                    if (PREP) {
-                        // one prepared tile, into the slot's upper half
-                        ptx::mbar_arrive_expect_tx(fb, A8_TILE_BYTES);
-                        ptx::bulk_g2s(ptx::smem_u32(slot_mem + (size_t)s * SLOT_BYTES + A_DIGIT_BYTES),
-                                      a.Aimg + ((uint64_t)q.mt * a.kblocks + kb) * A8_TILE_BYTES,
-                                      A8_TILE_BYTES, fb);
-                    } else {
-                        ptx::mbar_arrive_expect_tx(fb, SLOT_BYTES);
-                        ptx::tma_load_2d(ptx::smem_u32(slot_mem + (size_t)s * SLOT_BYTES), &a.tmap_a,
-                                         (int)(kb * BK), (int)(q.mt * BM), fb);
-                    }
-                    armed[s] = (int)round;
-                }
-            }
-            // copies already issued must land before the CTA can exit
-            for (int s = 0; s < SLOTS; ++s) {
-                if (armed[s] < 0) continue;
-                const uint32_t fb = ptx::smem_u32(&bars->a_full[s]);
-                const uint64_t t0 = ptx::globaltimer();
-                while (!ptx::mbar_try_wait(fb, armed[s] & 1) && ptx::globaltimer() - t0 < WAIT_NS) {
-                }
-            }
+    if (warp < CONV_WARPS) {
+        // ---------------- converters: A to fp16 digits ----------------
+        ptx::regs_inc<REGS_CONV>();
+        // k-blocks of A in flight in registers: 64 KiB per SM
+        constexpr int D = MODE == A_PREP ? 4 : 2;
+        AWords<MODE> buf[D];
+        ALoads<MODE> ld;
+        ld.w.start(a, u0, u1);
+        ld.locate(a, warp, lane);
+        Walk w = ld.w;
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+            ld.load(a, warp, lane, buf[d]);
+            ld.step(a, warp, lane);
         }
-    } else if (warp == W_BPROD) {
-        // ---------------- producer: B digit tiles (bulk copies from the prepared image) ----------------
-        if (lane == 0) {
-            // the image is written by the B-digit kernel launched just before
-            // this one (programmatic dependent launch): the only read of its
-            // output, so the only role that waits for it; A's copies, barrier
-            // set-up and TMEM allocation overlap its run
-            asm volatile("griddepcontrol.wait;" ::: "memory");
-            int armed[BSTAGES];
-            for (int s = 0; s < BSTAGES; ++s) armed[s] = -1;
-            uint32_t it = 0;
-            bool ok = true;
-            for (uint64_t u = u0; u < u1 && ok; ++u) {
-                const UnitPos q = unit_pos(a, u);
-                for (uint32_t kb = q.kb0; kb < q.kb1; ++kb, ++it) {
-                    const uint32_t s = it % BSTAGES, round = it / BSTAGES;
-                    if (round > 0 &&
-                        !wait_bar(ptx::smem_u32(&bars->empty_b[s]), (round - 1) & 1, abort, a.err)) {
-                        ok = false;
-                        break;
-                    }
-                    const uint32_t fb = ptx::smem_u32(&bars->full_b[s]);
-                    ptx::mbar_arrive_expect_tx(fb, B_TILE_BYTES);
-                    ptx::bulk_g2s(ptx::smem_u32(bst + (size_t)s * B_TILE_BYTES),
-                                  a.Bimg + ((uint64_t)q.nt * a.kblocks + kb) * B_TILE_BYTES,
-                                  B_TILE_BYTES, fb);
-                    armed[s] = (int)round;
+        const uint32_t tslot = tmem + A_COL0 + ((uint32_t)((warp & 3) * 32 + (warp >> 2) * 16) << 16);
+        const uint32_t bar_empty = ptx::smem_u32(&bars->a_empty[0]), bar_conv = ptx::smem_u32(&bars->conv[0]);
+        uint32_t j = 0, s = 0, ph = 1;   // k-block within the K range, slot
+        bool run = true;
+        while (run) {
+#pragma unroll
+            for (int d = 0; d < D; ++d) {
+                uint32_t hi[16], lo[16];
+                convert_a<MODE, PRE>(a, buf[d], hi, lo);
+                ld.load(a, warp, lane, buf[d]);
+                ld.step(a, warp, lane);
+                if (!w.left || !wait_bar_warp(bar_empty + s * 8u, ph, abort, a.err)) {
+                    run = false;
+                    break;
                 }
-            }
-            for (int s = 0; s < BSTAGES; ++s) {
-                if (armed[s] < 0) continue;
-                const uint32_t fb = ptx::smem_u32(&bars->full_b[s]);
-                const uint64_t t0 = ptx::globaltimer();
-                while (!ptx::mbar_try_wait(fb, armed[s] & 1) && ptx::globaltimer() - t0 < WAIT_NS) {
+                ptx::tc_fence_after();
+                ptx::tmem_st_16x256b_x4(tslot + s * SLOT_COLS, hi);
+                ptx::tmem_st_16x256b_x4(tslot + s * SLOT_COLS + SLOT_COLS / 2, lo);
+                ptx::tmem_st_wait();
+                ptx::tc_fence_before();
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(bar_conv + s * 8u);
+                s ^= 1u;
+                if (s == 0) ph ^= 1u;
+                if (++j == w.kbs) {
+                    j = 0;
+                    w.next(a);
                 }
             }
         }
     } else if (warp == W_MMA) {
         // ---------------- MMA issue (one thread) ----------------
+        ptx::regs_dec<REGS_MMA>();
         if (lane == 0) {
-            uint32_t it = 0, si = 0;
-            bool ok = true;
-            uint64_t idx = 0;
-            for (uint64_t u = u0; u < u1 && ok; ++u, ++idx) {
-                const UnitPos q = unit_pos(a, u);
-                const uint32_t b = (uint32_t)(idx & 1), use = (uint32_t)(idx >> 1);
-                if (use > 0 &&
-                    !wait_bar(ptx::smem_u32(&bars->acc_empty[b]), (use - 1) & 1, abort, a.err)) {
-                    ok = false;
-                    break;
-                }
+            Walk w;
+            w.start(a, u0, u1);
+            uint32_t s = 0, ph = 0, bset = 0, used = 0, b = 0, bph = 1;
+            bool ok = true, fresh = true;   // fresh: the K range's first unit
+            while (w.left && ok) {
+                // the accumulator set was drained by the unit before the last
+                if (!wait_bar(ptx::smem_u32(&bars->acc_empty[b]), bph, abort, a.err)) break;
                 ptx::tc_fence_after();
-                const uint32_t d_hi = tmem + b * 256u;         // A high digit x [B hi | B lo]
-                const uint32_t d_lo = tmem + b * 256u + 128u;  // A low digit  x [B hi | B lo]
-                for (uint32_t kb = q.kb0; kb < q.kb1; ++kb, ++it) {
-                    const uint32_t sub = (kb - q.kb0) % KBB;
-                    const uint32_t s = si % SLOTS, round = si / SLOTS;
-                    const uint32_t sb = it % BSTAGES, roundb = it / BSTAGES;
-                    // the slot's fp16 digits: converted or widened in place
-                    if (!wait_bar(ptx::smem_u32(&bars->full_b[sb]), roundb & 1, abort, a.err) ||
-                        (sub == 0 && !wait_bar(ptx::smem_u32(&bars->conv[s]), round & 1, abort, a.err))) {
-                        ok = false;
-                        break;
+                const uint32_t d_lo = tmem + b * ACC_COLS;   // A low digit x [B lo | B hi]: ll, lh
+                const uint32_t d_hi = d_lo + NT;             // A high digit x [B lo | B hi]: hl, hh
+                const bool final = w.left == 1 || w.mt + 1 == a.m_tiles;   // the K range's last unit
+                uint32_t t = bset * a.bset_tiles;
+                uint64_t db = ptx::sdesc_k_sw128(ptx::smem_u32(btiles + t * B_TILE_BYTES));
+                for (uint32_t j = 0; j < w.kbs; ++j, ++t, db += B_TILE_BYTES >> 4) {
+                    ok = wait_bar(ptx::smem_u32(&bars->conv[s]), ph, abort, a.err);
+                    if (ok && fresh) {
+                        ok = wait_bar(ptx::smem_u32(&bars->b_full[t]), (used >> t) & 1u, abort, a.err);
+                        used ^= 1u << t;
                     }
+                    if (!ok) break;
                     ptx::tc_fence_after();
-                    const uint32_t base =
-                        ptx::smem_u32(slot_mem + (size_t)s * SLOT_BYTES + (size_t)sub * A_TILE_BYTES);
-                    const uint64_t dah = ptx::sdesc_k_sw128(base);
-                    const uint64_t dal = ptx::sdesc_k_sw128(base + A_DIGIT_BYTES);
-                    const uint64_t db = ptx::sdesc_k_sw128(ptx::smem_u32(bst + (size_t)sb * B_TILE_BYTES));
+                    const uint32_t ah = tmem + A_COL0 + s * SLOT_COLS, al = ah + SLOT_COLS / 2;
 #pragma unroll
-                    for (int kk = 0; kk < BK / 16; ++kk) {
-                        const uint32_t acc = (kb > q.kb0 || kk > 0) ? 1u : 0u;
-                        // advance 16 fp16 (32 bytes) along K inside the swizzle atom
-                        ptx::mma_f16(d_hi, dah + 2 * kk, db + 2 * kk, IDESC, acc);
-                        ptx::mma_f16(d_lo, dal + 2 * kk, db + 2 * kk, IDESC, acc);
+                    for (uint32_t kk = 0; kk < 4; ++kk) {
+                        // 16 K: eight TMEM columns of A, 32 bytes of B inside the swizzle atom
+                        const uint32_t acc = (j > 0 || kk > 0) ? 1u : 0u;
+                        ptx::mma_f16_ts(d_lo, al + 8 * kk, db + 2 * kk, IDESC, acc);
+                        if (acc) {
+                            ptx::mma_f16_ts(d_hi, ah + 8 * kk, db + 2 * kk, IDESC, 1u);
+                        } else {
+                            // the middle columns already hold lh; hh starts from zero
+                            ptx::mma_f16_ts(d_hi, ah, db, IDESC_HALF, 1u);
+                            ptx::mma_f16_ts(d_hi + NT, ah, db + ((64 * 128) >> 4), IDESC_HALF, 0u);
+                        }
                     }
-                    ptx::mma_commit(ptx::smem_u32(&bars->empty_b[sb]));
-                    if (sub == KBB - 1 || kb + 1 == q.kb1) {   // last k-block of this slot
-                        ptx::mma_commit(ptx::smem_u32(&bars->a_empty[s]));
-                        ++si;
-                    }
+                    ptx::mma_commit(ptx::smem_u32(&bars->a_empty[s]));
+                    if (final) ptx::mma_commit(ptx::smem_u32(&bars->b_empty[t]));
+                    s ^= 1u;
+                    if (s == 0) ph ^= 1u;
                 }
                 if (!ok) break;
                 ptx::mma_commit(ptx::smem_u32(&bars->acc_full[b]));
+                b ^= 1u;
+                if (b == 0) bph ^= 1u;
+                fresh = w.next(a);
+                if (fresh && ++bset == a.bsets) bset = 0;
             }
             // every MMA issued by this CTA has completed before TMEM is freed
             ptx::mma_commit(ptx::smem_u32(&bars->drain));
@@ -496,130 +562,106 @@ __global__ void __launch_bounds__(THREADS, 1) k_block_tc(const __grid_constant__
                    ptx::globaltimer() - t0 < WAIT_NS) {
             }
         }
-    } else if (PREP && warp < W_EPI0) {
-        // ---------------- converters: 8-bit digit planes -> fp16 digit tiles, in place ----------------
-        const int ct = threadIdx.x - 32 * W_CONV0;   // 0..255
-        uint32_t si = 0;
-        for (uint64_t u = u0; u < u1; ++u) {
-            const UnitPos q = unit_pos(a, u);
+    } else if (warp > W_MMA) {
+        // ---------------- B digit tiles, once per K range (bulk copies) ----------------
+        ptx::regs_dec<REGS_MMA>();
+        if (warp == W_BPROD && lane == 0) {
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            Walk w;
+            w.start(a, u0, u1);
+            uint32_t bset = 0, used = 0, landing = 0;   // bit t: tile t's phase; tiles copied to
             bool ok = true;
-            for (uint32_t kb = q.kb0; kb < q.kb1; ++kb, ++si) {
-                const uint32_t s = si % SLOTS, round = si / SLOTS;
-                const bool got = warp_wait(ptx::smem_u32(&bars->a_full[s]), round & 1, abort, a.err);
-                // every converter warp reads its chunks before any overwrites them
-                if (ptx::bar_red_or<2, CONV_WARPS * 32>(!got || *abort != 0)) {
-                    ok = false;
-                    break;
+            while (w.left && ok) {
+                for (uint32_t j = 0; j < w.kbs; ++j) {
+                    const uint32_t t = bset * a.bset_tiles + j, bit = 1u << t;
+                    // free once the last unit of the range before has read it
+                    ok = wait_bar(ptx::smem_u32(&bars->b_empty[t]), used & bit ? 0u : 1u, abort, a.err);
+                    if (!ok) break;
+                    used ^= bit;
+                    landing |= bit;
+                    const uint32_t fb = ptx::smem_u32(&bars->b_full[t]);
+                    ptx::mbar_arrive_expect_tx(fb, B_TILE_BYTES);
+                    ptx::bulk_g2s(ptx::smem_u32(btiles + t * B_TILE_BYTES),
+                                  a.Bimg + ((uint64_t)w.nt * a.kblocks + w.kb0 + j) * B_TILE_BYTES, B_TILE_BYTES,
+                                  fb);
                 }
-                uint8_t *slot = slot_mem + (size_t)s * SLOT_BYTES;
-                const uint4 *src = reinterpret_cast<const uint4 *>(slot + A_DIGIT_BYTES);
-                uint4 w[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) w[i] = src[ct + 256 * i];
-                asm volatile("bar.sync 2, %0;" ::"n"(CONV_WARPS * 32) : "memory");
-#pragma unroll
-                for (int i = 0; i < 4; ++i) widen_store(slot, ct + 256 * i, w[i]);
-                ptx::fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&bars->conv[s]));
-            }
-            if (!ok) break;
-        }
-    } else if (warp < W_EPI0) {
-        // ---------------- converters: uint32 tiles -> centred fp16 digits, in place ----------------
-        const int ct = threadIdx.x - 32 * W_CONV0;   // 0..255
-        uint32_t si = 0;
-        for (uint64_t u = u0; u < u1; ++u) {
-            const UnitPos q = unit_pos(a, u);
-            bool ok = true;
-            for (uint32_t kb = q.kb0; kb < q.kb1; kb += KBB, ++si) {
-                const uint32_t s = si % SLOTS, round = si / SLOTS;
-                const bool got = warp_wait(ptx::smem_u32(&bars->a_full[s]), round & 1, abort, a.err);
-                // all converter warps read the box before any overwrites it; decide together
-                if (ptx::bar_red_or<2, CONV_WARPS * 32>(!got || *abort != 0)) {
-                    ok = false;
-                    break;
+                if (++bset == a.bsets) bset = 0;
+                while (w.left && !w.next(a)) {
                 }
-                uint8_t *slot = slot_mem + (size_t)s * SLOT_BYTES;
-                const uint32_t nsub = min((uint32_t)KBB, q.kb1 - kb);
-                ARegs r[KBB];
-#pragma unroll
-                for (int sub = 0; sub < KBB; ++sub)
-                    if ((uint32_t)sub < nsub) load_tile<KBB>(slot, sub, ct, r[sub]);
-                asm volatile("bar.sync 2, %0;" ::"n"(CONV_WARPS * 32) : "memory");
-#pragma unroll
-                for (int sub = 0; sub < KBB; ++sub)
-                    if ((uint32_t)sub < nsub) store_digits<PRE>(a, r[sub], slot + (size_t)sub * A_TILE_BYTES, ct);
-                ptx::fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&bars->conv[s]));
             }
-            if (!ok) break;
+            // copies already issued must land before the CTA can exit
+            for (uint32_t t = 0; t < RK; ++t) {
+                if (!((landing >> t) & 1u)) continue;
+                const uint64_t t0 = ptx::globaltimer();
+                while (!ptx::mbar_try_wait(ptx::smem_u32(&bars->b_full[t]), ((used >> t) & 1u) ^ 1u) &&
+                       ptx::globaltimer() - t0 < WAIT_NS) {
+                }
+            }
         }
     } else {
         // ---------------- epilogue: TMEM -> residues ----------------
+        ptx::regs_dec<REGS_EPI>();
+        asm volatile("griddepcontrol.wait;" ::: "memory");
         const int quarter = warp & 3;               // TMEM lanes 32*quarter .. +31
-        const int row_in_tile = quarter * 32 + lane;
-        const uint32_t lane_bits = (uint32_t)(quarter * 32) << 16;
-        uint32_t res[NT];
-#pragma unroll
-        for (int j = 0; j < NT; ++j) res[j] = 0;
-        uint64_t idx = 0;
-        for (uint64_t u = u0; u < u1; ++u, ++idx) {
-            const UnitPos q = unit_pos(a, u);
-            const uint32_t b = (uint32_t)(idx & 1), use = (uint32_t)(idx >> 1);
-            const bool got = warp_wait(ptx::smem_u32(&bars->acc_full[b]), use & 1, abort, a.err);
-            // decide together: the epilogue warps meet at named barriers below
-            if (ptx::bar_red_or<1, EPI_WARPS * 32>(!got || *abort != 0)) break;
+        const uint32_t c_first = (uint32_t)((warp - W_EPI0) >> 2) * 32u;   // this warp's 32 columns
+        const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + c_first;
+        Walk w;
+        w.start(a, u0, u1);
+        uint32_t b = 0, ph = 0;
+        while (w.left && wait_bar_warp(ptx::smem_u32(&bars->acc_full[b]), ph, abort, a.err)) {
             ptx::tc_fence_after();
-            const uint32_t d_hi = tmem + lane_bits + b * 256u;
-            const uint32_t d_lo = d_hi + 128u;
-#pragma unroll
-            for (int g = 0; g < NT / 8; ++g) {
-                uint32_t hh[8], hl[8], lh[8], ll[8];
-                ptx::tmem_ld8(d_hi + g * 8, hh);
-                ptx::tmem_ld8(d_hi + NT + g * 8, hl);
-                ptx::tmem_ld8(d_lo + g * 8, lh);
-                ptx::tmem_ld8(d_lo + NT + g * 8, ll);
+            const uint64_t grow = (uint64_t)w.mt * BM + quarter * 32 + lane;
+            const uint64_t col0 = (uint64_t)w.nt * NT + c_first;
+            // columns of this warp's 32 that exist (none for a row outside)
+            const int ncols = grow < a.m && col0 < a.nb ? (int)min(a.nb - col0, (uint64_t)32) : 0;
+            uint32_t *dst = a.direct ? a.C + grow * a.ldc + col0 : a.Cacc + col0 * a.m + grow;
+            const uint64_t step = a.direct ? 1 : a.m;
+#pragma unroll 1
+            for (int g = 0; g < 32; g += 8) {
+                uint32_t hh[8], md[8], ll[8];
+                ptx::tmem_ld8(taddr + b * ACC_COLS + g, ll);
+                ptx::tmem_ld8(taddr + b * ACC_COLS + NT + g, md);
+                ptx::tmem_ld8(taddr + b * ACC_COLS + 2 * NT + g, hh);
                 ptx::tmem_ld_wait();
+                if (g == 24) {
+                    ptx::tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&bars->acc_empty[b]));
+                }
+                // Horner's rule modulo p in 32 bits, t - floor(t smagic / 2^32) p:
+                // every accumulator is at most 2^24 in magnitude, so |t| stays
+                // below 2^26, the quotient is that of t / p but for less than
+                // |t| / 2^32 < 1/64, and the remainder lies in (-p/64, p + p/64);
+                // adding p and taking it off again where the result stays
+                // non-negative leaves [0, p + p/64]
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    const long long vhh = __float2int_rn(__uint_as_float(hh[j]));
-                    const long long vx = (long long)__float2int_rn(__uint_as_float(hl[j])) +
-                                         (long long)__float2int_rn(__uint_as_float(lh[j]));
-                    const long long vll = __float2int_rn(__uint_as_float(ll[j]));
-                    const long long v = vhh * 65536ll + vx * 256ll + vll;
-                    res[g * 8 + j] = add_mod(res[g * 8 + j], reduce64((uint64_t)(v + (long long)a.off), a.mod),
-                                             a.mod.p);
+                    const int p = (int)a.p;
+                    int t = __float2int_rn(__uint_as_float(hh[j]));
+                    t -= __mulhi(t, a.smagic) * p;
+                    t = t * 256 + __float2int_rn(__uint_as_float(md[j]));
+                    t -= __mulhi(t, a.smagic) * p;
+                    t = t * 256 + __float2int_rn(__uint_as_float(ll[j]));
+                    t -= __mulhi(t, a.smagic) * p;
+                    hh[j] = min((uint32_t)t, (uint32_t)(t + p));
+                }
+                if (a.direct) {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        if (g + j < ncols) dst[g + j] = min(hh[j], hh[j] - a.p);
+                } else {
+                    // column-major partial sums: the 32 lanes of a warp
+                    // (consecutive rows) add to 128 consecutive bytes
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        if (g + j < ncols) atomicAdd(dst, hh[j]);
+                        dst += step;
+                    }
                 }
             }
-            ptx::tc_fence_before();
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&bars->acc_empty[b]));
-            // end of this CTA's run of units on the output tile?
-            bool flush = (u + 1 == u1);
-            if (!flush) {
-                const UnitPos nq = unit_pos(a, u + 1);
-                flush = (nq.mt != q.mt) || (nq.nt != q.nt);
-            }
-            if (flush) {
-                // column-major partial sums: the 32 lanes of a warp (consecutive
-                // rows) add to 128 consecutive bytes, one L2 transaction per
-                // column; k_block_finish reduces them into C after this kernel
-                const uint64_t grow = (uint64_t)q.mt * BM + row_in_tile;
-                const uint64_t col0 = (uint64_t)q.nt * NT;
-                if (grow < a.m) {
-#pragma unroll
-                    for (int j = 0; j < NT; ++j)
-                        if (col0 + j < a.nb) atomicAdd(&a.Cacc[(col0 + j) * a.m + grow], res[j]);
-                }
-#pragma unroll
-                for (int j = 0; j < NT; ++j) res[j] = 0;
-                // the epilogue warps meet after a flush: without this barrier the
-                // compiler carries the flush into the next unit's drain and the
-                // kernel spills about 440 bytes per thread at 128 registers
-                asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32));
-            }
+            b ^= 1u;
+            if (b == 0) ph ^= 1u;
+            w.next(a);
         }
         // the kernel that reduces the partial sums may be launched now (it
         // waits for this grid to complete before reading them)
@@ -634,6 +676,64 @@ __global__ void __launch_bounds__(THREADS, 1) k_block_tc(const __grid_constant__
     }
 }
 
+// B (k x nb, row-major) -> per (modulus, n-tile, k-block) tiles of 128 rows x
+// 64 K fp16 digits in the 128-byte swizzled K-major layout: rows 0..63 hold the
+// low digits of output columns nt*64 + r, rows 64..127 the high digits.  One
+// pass over B serves every residue pass.
+struct PrepB {
+    uint32_t n;                        // moduli; one: B's entries are already below it
+    uint32_t p[RNS_MAX], magic[RNS_MAX];
+};
+constexpr int PREPB_THREADS = 256;
+__global__ void __launch_bounds__(PREPB_THREADS)
+    k_block_prep_b(const uint32_t *__restrict__ B, uint64_t ldb, uint64_t k, uint64_t nb, uint32_t kblocks,
+                   const __grid_constant__ PrepB pb, uint8_t *img)
+{
+    // everything before this kernel is complete from here on, so the product
+    // kernel may be placed (it waits for this grid where it reads the tiles)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const uint32_t tile = blockIdx.x;            // nt * kblocks + kb
+    const uint32_t nt = tile / kblocks, kb = tile % kblocks;
+    constexpr int PER = 64 * 8 / PREPB_THREADS;  // (column, 8 K) items of a thread
+    uint32_t v[PER][8];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int t = threadIdx.x + i * PREPB_THREADS;
+        // consecutive threads: consecutive columns of one row of B
+        const uint64_t col = (uint64_t)nt * NT + (t & 63), k0 = (uint64_t)kb * BK + (t >> 6) * 8;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[i][e] = (col < nb && k0 + e < k) ? __ldg(B + (k0 + e) * ldb + col) : 0u;
+    }
+    for (uint32_t l = 0; l < pb.n; ++l) {
+        const uint32_t p = pb.p[l], half = (p - 1) / 2;
+        uint8_t *out = img + ((uint64_t)l * gridDim.x + tile) * B_TILE_BYTES;
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            const int t = threadIdx.x + i * PREPB_THREADS;
+            uint32_t u[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const uint32_t b = pb.n > 1 ? reduce_small(v[i][e], p, pb.magic[l]) : v[i][e];
+                u[e] = b + (b > half ? U_BIAS - p : U_BIAS);
+            }
+            uint4 h, lo;
+            split_u(u[0], u[1], h.x, lo.x);
+            split_u(u[2], u[3], h.y, lo.y);
+            split_u(u[4], u[5], h.z, lo.z);
+            split_u(u[6], u[7], h.w, lo.w);
+            // 128-byte swizzle: 16-byte chunk j of row r sits at chunk j ^ (r & 7)
+            const int row = t & 63, j = t >> 6;
+            const uint32_t off = (uint32_t)row * 128u + ((uint32_t)(j ^ (row & 7)) << 4);
+            *reinterpret_cast<uint4 *>(out + off) = lo;
+            *reinterpret_cast<uint4 *>(out + 64 * 128 + off) = h;
+        }
+    }
+}
+
+// Partial sums to residues: C = sums mod p (and the sums back to zero), or,
+// with C null, the sums themselves reduced below p in place (between the
+// launches of a product with more than SLAB_K terms).
 constexpr int FIN_THREADS = 512;
 __global__ void __launch_bounds__(FIN_THREADS)
     k_block_finish(uint32_t *__restrict__ Cacc, uint64_t m, uint64_t nb, uint32_t *__restrict__ C,
@@ -641,6 +741,8 @@ __global__ void __launch_bounds__(FIN_THREADS)
 {
     __shared__ uint32_t t[NT][BM + 1];   // [column][row], padded against bank conflicts
     constexpr int PER = NT * BM / FIN_THREADS;
+    // the next product of the stream may be placed now; it waits for this grid
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const uint64_t r0 = (uint64_t)blockIdx.x * BM, c0 = (uint64_t)blockIdx.y * NT;
     // all of a thread's loads are issued before any is used or cleared (one
@@ -655,9 +757,11 @@ __global__ void __launch_bounds__(FIN_THREADS)
 #pragma unroll
     for (int e = 0; e < PER; ++e) {
         const int i = threadIdx.x + e * FIN_THREADS, c = i / BM, r = i % BM;
-        if (r0 + r < m && c0 + c < nb) __stcg(&Cacc[(c0 + c) * m + r0 + r], 0u);
-        t[c][r] = reduce_small(v[e], p, magic);   // the sums are below 2^32
+        v[e] = reduce_small(v[e], p, magic);   // the sums are below 2^32
+        if (r0 + r < m && c0 + c < nb) __stcg(&Cacc[(c0 + c) * m + r0 + r], C ? 0u : v[e]);
+        t[c][r] = v[e];
     }
+    if (!C) return;
     __syncthreads();
     for (int i = threadIdx.x; i < NT * BM; i += FIN_THREADS) {
         const int r = i / NT, c = i % NT;   // consecutive threads: consecutive columns of one row
@@ -665,70 +769,50 @@ __global__ void __launch_bounds__(FIN_THREADS)
     }
 }
 
-
-// B (k x nb, row-major) -> per (n-tile, k-block) tiles of 128 rows x 64 K
-// fp16 digits in the 128-byte swizzled K-major layout: rows 0..63 hold the
-// high digits of output columns nt*64 + r, rows 64..127 the low digits.
-__global__ void k_block_prep_b(const uint32_t *B, uint64_t ldb, uint64_t k, uint64_t nb, Mod mod,
-                               uint32_t half, uint32_t kblocks, int pre, uint8_t *img)
-{
-    // the product kernel that follows may be placed now (it waits for this
-    // grid only where it reads the image)
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const uint32_t tile = blockIdx.x;            // nt * kblocks + kb
-    const uint32_t nt = tile / kblocks, kb = tile % kblocks;
-    uint8_t *out = img + (uint64_t)tile * B_TILE_BYTES;
-    for (int t = threadIdx.x; t < 64 * 8; t += blockDim.x) {
-        const int col = t >> 3, j = t & 7;       // output column within the tile, 16-byte chunk
-        const uint64_t gcol = (uint64_t)nt * NT + col;
-        uint32_t v[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const uint64_t gk = (uint64_t)kb * BK + j * 8 + e;
-            v[e] = (gk < k && gcol < nb) ? B[gk * ldb + gcol] : 0u;
-            if (pre) v[e] %= mod.p;
-        }
-        uint4 wh, wl;
-        split_pair(v[0], v[1], mod.p, half, wh.x, wl.x);
-        split_pair(v[2], v[3], mod.p, half, wh.y, wl.y);
-        split_pair(v[4], v[5], mod.p, half, wh.z, wl.z);
-        split_pair(v[6], v[7], mod.p, half, wh.w, wl.w);
-        const int rh = col, rl = col + 64;
-        *reinterpret_cast<uint4 *>(out + rh * 128 + ((j ^ (rh & 7)) << 4)) = wh;
-        *reinterpret_cast<uint4 *>(out + rl * 128 + ((j ^ (rl & 7)) << 4)) = wl;
-    }
-}
-
 // A (m x k, row-major uint32 residues, leading dimension lda) -> prepared
-// tiles for one modulus p <= 65536: per (m-tile, k-block) the two 8-bit digit
-// planes described at A8_TILE_BYTES.  Entries outside the matrix are 0
-// (bytes 0x80, 0x80).  With pre != 0 each entry is first reduced modulo p (a
-// residue pass).  Thread q of a tile handles 4 consecutive K of one row.
-__global__ void __launch_bounds__(256)
-    k_block_prep_a(const uint32_t *__restrict__ A, uint64_t lda, uint64_t m, uint64_t k, Mod mod,
-                   uint32_t pre_magic, int pre, uint32_t kblocks, uint8_t *img)
+// tiles for one modulus p <= 65536 (A8_TILE_BYTES): thread t of a tile writes
+// the 32 high and 32 low digits that converter lane t of the product reads.
+// Entries outside the matrix are 0 (bytes 0x80, 0x80).  With pre != 0 each
+// entry is first reduced modulo p (a residue pass).
+__global__ void __launch_bounds__(32 * CONV_WARPS)
+    k_block_prep_a(const uint32_t *__restrict__ A, uint64_t lda, uint64_t m, uint64_t k, uint32_t p,
+                   uint32_t magic, int pre, int vec, uint32_t kblocks, uint8_t *img)
 {
     const uint64_t tile = blockIdx.x;   // mt * kblocks + kb
-    const uint64_t mt = tile / kblocks, kb = tile % kblocks;
-    uint8_t *hi = img + tile * A8_TILE_BYTES;
-    uint8_t *lo = hi + A8_PLANE_BYTES;
-    const uint32_t p = mod.p;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint64_t row = tile / kblocks * BM + (warp & 3) * 32 + (warp >> 2) * 16 + (lane >> 2);
+    const uint64_t col = tile % kblocks * BK + (lane & 3) * 4;
     const uint32_t thr = min((p - 1) / 2, 32639u);   // largest residue kept as itself
-    for (int q = threadIdx.x; q < BM * 16; q += blockDim.x) {
-        const int row = q >> 4, c4 = q & 15;
-        const uint64_t gr = mt * BM + row, gk = kb * BK + (uint64_t)c4 * 4;
-        uint32_t hb = 0, lb = 0;
+    uint4 w[8];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            uint32_t v = (gr < m && gk + e < k) ? __ldg(A + gr * lda + gk + e) : 0u;
-            if (pre) v = reduce_small(v, p, pre_magic);
-            const uint32_t u = v + 32896u - (v > thr ? p : 0u);   // in [0, 65535]
-            hb |= (u >> 8) << (8 * e);
-            lb |= (u & 255u) << (8 * e);
-        }
-        *reinterpret_cast<uint32_t *>(hi + row * BK + c4 * 4) = hb;
-        *reinterpret_cast<uint32_t *>(lo + row * BK + c4 * 4) = lb;
+    for (int i = 0; i < 8; ++i) {
+        const uint64_t r = row + 8 * (i & 1), c = col + (i >> 1) * 16;
+        const uint32_t *q = A + r * lda + c;
+        const uint64_t n = r < m && c < k ? k - c : 0;
+        if (vec && n >= 4)
+            w[i] = __ldcs(reinterpret_cast<const uint4 *>(q));
+        else
+            w[i] = make_uint4(n > 0 ? __ldg(q) : 0u, n > 1 ? __ldg(q + 1) : 0u, n > 2 ? __ldg(q + 2) : 0u,
+                              n > 3 ? __ldg(q + 3) : 0u);
     }
+    uint32_t hb[8], lb[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const uint32_t e[4] = {w[i].x, w[i].y, w[i].z, w[i].w};
+        hb[i] = lb[i] = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t v = pre ? reduce_small(e[j], p, magic) : e[j];
+            const uint32_t u = v + 32896u - (v > thr ? p : 0u);   // in [0, 65535]
+            hb[i] |= (u >> 8) << (8 * j);
+            lb[i] |= (u & 255u) << (8 * j);
+        }
+    }
+    uint8_t *out = img + tile * A8_TILE_BYTES + warp * 2048 + lane * 16;
+    *reinterpret_cast<uint4 *>(out) = make_uint4(hb[0], hb[1], hb[2], hb[3]);
+    *reinterpret_cast<uint4 *>(out + 512) = make_uint4(hb[4], hb[5], hb[6], hb[7]);
+    *reinterpret_cast<uint4 *>(out + 1024) = make_uint4(lb[0], lb[1], lb[2], lb[3]);
+    *reinterpret_cast<uint4 *>(out + 1536) = make_uint4(lb[4], lb[5], lb[6], lb[7]);
 }
 
 // x mod m for x < 2^40 and m < 2^17, minv = floor((2^64 - 1) / m): the
@@ -901,43 +985,18 @@ bool block_rns_plan(uint32_t p, uint64_t k, RnsConst *rc)
     return true;
 }
 
-size_t block_tc_bimg_bytes(uint64_t k, uint64_t nb)
+size_t block_tc_workspace_bytes(uint64_t m, uint64_t nb)
 {
-    const uint64_t kblocks = (k + blk::BK - 1) / blk::BK;
     const uint64_t n_tiles = (nb + blk::NT - 1) / blk::NT;
-    return (n_tiles * kblocks * (uint64_t)blk::B_TILE_BYTES + 255) & ~(size_t)255;
+    return 256 /* error flag */ + ((m * n_tiles * blk::NT * 4 + 255) & ~(size_t)255);
 }
 
-size_t block_tc_workspace_bytes(uint64_t m, uint64_t k, uint64_t nb)
+size_t block_tc_bimg_bytes(uint64_t k, uint64_t nb, int n_mod)
 {
-    const uint64_t kblocks = (k + blk::BK - 1) / blk::BK;
+    const bool cut = k > blk::SLAB_K;   // residue passes then make their tiles one after the other
+    const uint64_t kblocks = (std::min<uint64_t>(k, blk::SLAB_K) + blk::BK - 1) / blk::BK;
     const uint64_t n_tiles = (nb + blk::NT - 1) / blk::NT;
-    size_t b = n_tiles * kblocks * (uint64_t)blk::B_TILE_BYTES;
-    b = (b + 255) & ~(size_t)255;
-    b += ((m * n_tiles * blk::NT * 4 + 255) & ~(size_t)255);
-    b += 256;   // error flag
-    return b;
-}
-
-uint32_t *block_tc_err_flag(void *ws, uint64_t m, uint64_t k, uint64_t nb)
-{
-    return (uint32_t *)((uint8_t *)ws + block_tc_workspace_bytes(m, k, nb) - 256);
-}
-
-static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
-{
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
-                                             &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = (PFN_cuTensorMapEncodeTiled_v12000)p;
-    }
-    return fn;
+    return n_tiles * kblocks * (uint64_t)blk::B_TILE_BYTES * (cut ? (n_mod > 1 ? 2 : 1) : n_mod);
 }
 
 size_t block_prep_a_bytes(uint64_t m, uint64_t k)
@@ -955,108 +1014,144 @@ cudaError_t launch_block_prep_a(const Mod &mod, uint64_t m, uint64_t k, const ui
     if (m_tiles * kblocks == 0) return cudaSuccess;
     if (m_tiles * kblocks > 0x7FFFFFFFull) return cudaErrorInvalidValue;
     if (mod.p > DIGIT8_MAX_P) return cudaErrorInvalidValue;
-    k_block_prep_a<<<(unsigned)(m_tiles * kblocks), 256, 0, s>>>(
-        A, lda, m, k, mod, (uint32_t)((1ull << 32) / mod.p), reduce_inputs ? 1 : 0, (uint32_t)kblocks,
-        img);
+    k_block_prep_a<<<(unsigned)(m_tiles * kblocks), 32 * CONV_WARPS, 0, s>>>(
+        A, lda, m, k, mod.p, (uint32_t)((1ull << 32) / mod.p), reduce_inputs ? 1 : 0,
+        block_tc_layout_ok(A, lda) ? 1 : 0, (uint32_t)kblocks, img);
     return cudaGetLastError();
 }
 
-cudaError_t launch_block_tc(const Mod &mod, uint64_t m, uint64_t k, uint64_t nb, const uint32_t *A,
-                            uint64_t lda, const uint32_t *B, uint64_t ldb, uint32_t *C, uint64_t ldc,
-                            void *ws, int sm_count, cudaStream_t s, int *launches, bool reduce_inputs,
-                            const uint8_t *Aimg)
+// K ranges of a product with `tiles` output tiles and `kblocks` k-blocks on
+// `sms` CTAs: at least enough for the exact chunk of RK k-blocks, more where
+// units would not fill the CTAs or would leave them uneven.  A unit costs its
+// k-blocks plus its drain; the CTA with the most units sets the time.
+static uint32_t block_ranges(uint64_t tiles, uint32_t kblocks, int sms)
+{
+    const uint32_t lo = (kblocks + blk::RK - 1) / blk::RK;
+    uint32_t best = lo;
+    double best_cost = 0;
+    for (uint32_t r = lo; r <= kblocks && r <= 8 * lo; ++r) {
+        const double per_cta = (double)((tiles * r + sms - 1) / (uint64_t)sms);
+        const double cost = per_cta * ((double)((kblocks + r - 1) / r) + 1.5);
+        if (r == lo || cost < 0.97 * best_cost) {
+            best = r;
+            best_cost = cost;
+        }
+        if (tiles * r > 8 * (uint64_t)sms) break;
+    }
+    return best;
+}
+
+// One product (n_mod = 1: modulus mods[0]; C = A B mod it) or all residue
+// passes (n_mod moduli; pass l writes the dense m x nb matrix C + l m nb).
+cudaError_t launch_block_tc(const uint32_t *mods, int n_mod, uint64_t m, uint64_t k, uint64_t nb,
+                            const uint32_t *A, uint64_t lda, const uint32_t *B, uint64_t ldb, uint32_t *C,
+                            uint64_t ldc, const BlockScratch &sc, int sm_count, cudaStream_t s,
+                            int *launches, const uint8_t *Aimg, size_t img_bytes)
 {
     using namespace blk;
+    typedef void (*Kernel)(const Args);
+    static const Kernel kernels[5] = {k_block_tc<A_VEC, false>, k_block_tc<A_VEC, true>,
+                                      k_block_tc<A_ANY, false>, k_block_tc<A_ANY, true>,
+                                      k_block_tc<A_PREP, false>};
     static bool attr = false;
     if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_block_tc<false, false, PipeU32>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)PipeU32::SMEM_BYTES);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_block_tc<true, false, PipeU32>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PipeU32::SMEM_BYTES);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_block_tc<false, true, PipePrep>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PipePrep::SMEM_BYTES);
-        if (e != cudaSuccess) return e;
+        for (Kernel f : kernels) {
+            cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)SMEM_BYTES);
+            // the rest of the 256 KiB stays L1: the loads in flight land there
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 58);
+            if (e != cudaSuccess) return e;
+        }
         attr = true;
     }
+    const bool reduce = n_mod > 1;
+    // prepared digits: 16-byte aligned tiles of a device allocation
+    if (Aimg && (((uintptr_t)Aimg) & 15u)) return cudaErrorInvalidValue;
+    const Kernel kernel = Aimg ? kernels[4] : kernels[(block_tc_layout_ok(A, lda) ? 0 : 2) + (reduce ? 1 : 0)];
+    if ((nb + NT - 1) / NT > 65535) return cudaErrorInvalidValue;   // grid y of the finishing kernel
     Args a;
     memset(&a, 0, sizeof a);
-    if (Aimg) {
-        // prepared digits (16-byte aligned tiles of a device allocation): no tensor map
-        if (((uintptr_t)Aimg) & 15u) return cudaErrorInvalidValue;
-        a.Aimg = Aimg;
-    } else {
-        PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
-        if (!encode) return cudaErrorNotSupported;
-        // A: innermost dimension k (elements), then m rows lda*4 bytes apart
-        const cuuint64_t gdim[2] = {(cuuint64_t)k, (cuuint64_t)m};
-        const cuuint64_t gstride[1] = {(cuuint64_t)lda * 4};
-        const cuuint32_t box[2] = {(cuuint32_t)(BK * PipeU32::KBB), (cuuint32_t)BM};
-        const cuuint32_t estride[2] = {1, 1};
-        if (encode(&a.tmap_a, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, (void *)A, gdim, gstride, box, estride,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return cudaErrorInvalidValue;
-    }
     a.m = m;
-    a.k = k;
     a.nb = nb;
-    a.C = C;
-    a.ldc = ldc;
-    a.mod = mod;
-    a.half = (mod.p - 1) / 2;
-    a.kblocks = (uint32_t)((k + BK - 1) / BK);
+    a.lda = lda;
+    a.img_kblocks = (uint32_t)((k + BK - 1) / BK);
+    a.err = (uint32_t *)sc.ws;
+    a.Cacc = (uint32_t *)((uint8_t *)sc.ws + 256);
     a.n_tiles = (uint32_t)((nb + NT - 1) / NT);
     a.m_tiles = (uint32_t)((m + BM - 1) / BM);
-    a.chunks = (a.kblocks + KC - 1) / KC;
-    a.units = (uint64_t)a.n_tiles * a.m_tiles * a.chunks;
-    if (a.n_tiles > 65535) return cudaErrorInvalidValue;   // grid y of the finishing kernel
-    const uint64_t two41 = 1ull << 41;
-    a.off = (two41 / mod.p + 1) * (uint64_t)mod.p;
-    a.pre_magic = (uint32_t)((1ull << 32) / mod.p);
-    uint8_t *w = (uint8_t *)ws;
-    size_t o = (size_t)a.n_tiles * a.kblocks * B_TILE_BYTES;
-    o = (o + 255) & ~(size_t)255;
-    a.Bimg = w;
-    a.Cacc = (uint32_t *)(w + o);
-    o += ((m * a.n_tiles * NT * 4 + 255) & ~(size_t)255);
-    a.err = (uint32_t *)(w + o);
-    k_block_prep_b<<<a.n_tiles * a.kblocks, 256, 0, s>>>(B, ldb, k, nb, mod, a.half, a.kblocks,
-                                                         reduce_inputs ? 1 : 0, (uint8_t *)a.Bimg);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    const uint64_t grid = std::min<uint64_t>(a.units, (uint64_t)sm_count);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(THREADS);
-    cfg.stream = s;
+    a.edge_m = m % BM ? a.m_tiles - 1 : ~0u;
+    const uint64_t tiles = (uint64_t)a.m_tiles * a.n_tiles;
     cudaLaunchAttribute pdl[1];
     pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     pdl[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = pdl;
-    cfg.numAttrs = 1;
-    if (Aimg) {   // the image already holds the residues of this pass's modulus
-        cfg.dynamicSmemBytes = PipePrep::SMEM_BYTES;
-        e = cudaLaunchKernelEx(&cfg, k_block_tc<false, true, PipePrep>, a);
-    } else if (reduce_inputs) {
-        cfg.dynamicSmemBytes = PipeU32::SMEM_BYTES;
-        e = cudaLaunchKernelEx(&cfg, k_block_tc<true, false, PipeU32>, a);
-    } else {
-        cfg.dynamicSmemBytes = PipeU32::SMEM_BYTES;
-        e = cudaLaunchKernelEx(&cfg, k_block_tc<false, false, PipeU32>, a);
-    }
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t fcfg = {};
+    cudaLaunchConfig_t bcfg = {}, cfg = {}, fcfg = {};
+    bcfg.blockDim = dim3(PREPB_THREADS);
+    cfg.blockDim = dim3(THREADS);
+    cfg.dynamicSmemBytes = SMEM_BYTES;
     fcfg.gridDim = dim3(a.m_tiles, a.n_tiles);
     fcfg.blockDim = dim3(FIN_THREADS);
-    fcfg.stream = s;
-    fcfg.attrs = pdl;
-    fcfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&fcfg, k_block_finish, a.Cacc, m, nb, C, ldc, mod.p, a.pre_magic);
-    if (e != cudaSuccess) return e;
-    *launches += 3;
+    bcfg.stream = cfg.stream = fcfg.stream = s;
+    bcfg.attrs = cfg.attrs = fcfg.attrs = pdl;
+    bcfg.numAttrs = cfg.numAttrs = fcfg.numAttrs = 1;
+    PrepB pb;
+    memset(&pb, 0, sizeof pb);
+    for (int l0 = 0; l0 < n_mod; l0 += k > SLAB_K ? 1 : n_mod) {
+        // all moduli of a product in one launch set; one at a time where K is cut
+        const int l1 = k > SLAB_K ? l0 + 1 : n_mod;
+        for (uint64_t k0 = 0; k0 < k; k0 += SLAB_K) {
+            a.k = std::min<uint64_t>(SLAB_K, k - k0);
+            const bool last = k - k0 <= SLAB_K;
+            a.A = A ? A + k0 : nullptr;
+            a.img_kb0 = (uint32_t)(k0 / BK);
+            a.kblocks = (uint32_t)((a.k + BK - 1) / BK);
+            a.ranges = block_ranges(tiles, a.kblocks, sm_count);
+            a.r_base = a.kblocks / a.ranges;
+            a.r_rem = a.kblocks % a.ranges;
+            a.bsets = RK / (a.r_base + (a.r_rem ? 1 : 0));
+            a.bset_tiles = RK / a.bsets;
+            a.edge_k = a.k % BK ? a.kblocks - 1 : ~0u;
+            a.units = tiles * a.ranges;
+            a.direct = a.ranges == 1 && k <= SLAB_K ? 1 : 0;
+            const uint32_t btiles = a.n_tiles * a.kblocks;
+            pb.n = (uint32_t)(l1 - l0);
+            for (int l = l0; l < l1; ++l) {
+                pb.p[l - l0] = mods[l];
+                pb.magic[l - l0] = (uint32_t)((1ull << 32) / mods[l]);
+            }
+            if (reduce && pb.n == 1) {   // the tiles of one residue modulus still need the reduction
+                pb.n = 2;
+                pb.p[1] = pb.p[0];
+                pb.magic[1] = pb.magic[0];
+            }
+            bcfg.gridDim = dim3(btiles);
+            cudaError_t e = cudaLaunchKernelEx(&bcfg, k_block_prep_b, B + k0 * ldb, ldb, a.k, nb, a.kblocks, pb,
+                                               sc.bimg);
+            if (e != cudaSuccess) return e;
+            ++*launches;
+            cfg.gridDim = dim3((unsigned)std::min<uint64_t>(a.units, (uint64_t)sm_count));
+            for (int l = l0; l < l1; ++l) {
+                const uint32_t p = mods[l];
+                a.p = p;
+                a.half = (p - 1) / 2;
+                a.magic = (uint32_t)((1ull << 32) / p);
+                a.smagic = (int32_t)std::min<uint64_t>((1ull << 32) / p, 0x7FFFFFFFull);
+                a.magic47 = reduce ? (uint32_t)((1ull << 47) / p) : 0;
+                a.C = C + (reduce ? (uint64_t)l * m * nb : 0);
+                a.ldc = ldc;
+                a.Aimg = Aimg ? Aimg + (size_t)l * img_bytes : nullptr;
+                a.Bimg = sc.bimg + (uint64_t)(l - l0) * btiles * B_TILE_BYTES;
+                e = cudaLaunchKernelEx(&cfg, kernel, a);
+                if (e != cudaSuccess) return e;
+                ++*launches;
+                if (a.direct) continue;
+                e = cudaLaunchKernelEx(&fcfg, k_block_finish, a.Cacc, m, nb, last ? a.C : (uint32_t *)nullptr,
+                                       ldc, p, a.magic);
+                if (e != cudaSuccess) return e;
+                ++*launches;
+            }
+        }
+    }
     return cudaGetLastError();
 }
 

@@ -126,7 +126,7 @@ constexpr uint32_t BLOCK_TC_MAX_P = 65791;
 // most 65536, so that every residue has two 8-bit balanced digits.
 constexpr uint32_t RNS_PRIME_MAX = 65536;
 bool block_tc_eligible(uint32_t p, const uint32_t *A, uint64_t lda);
-// A's layout suits the tensor-core kernel (TMA: 16-byte base, rows 16-byte apart)
+// A's layout suits 16-byte loads (16-byte base, rows a multiple of 16 bytes apart)
 bool block_tc_layout_ok(const uint32_t *A, uint64_t lda);
 
 // Residue-number-system constants of a large-p tensor-core block product:
@@ -146,18 +146,25 @@ struct RnsConst {
 bool block_rns_plan(uint32_t p, uint64_t k, RnsConst *rc);
 cudaError_t launch_block_crt(const uint32_t *R, uint64_t m, uint64_t nb, uint32_t *C, uint64_t ldc,
                              const RnsConst &rc, int sm_count, cudaStream_t s);
-size_t block_tc_workspace_bytes(uint64_t m, uint64_t k, uint64_t nb);
-size_t block_tc_bimg_bytes(uint64_t k, uint64_t nb);   // the rest must be zero at launch
-cudaError_t launch_block_tc(const Mod &mod, uint64_t m, uint64_t k, uint64_t nb, const uint32_t *A,
-                            uint64_t lda, const uint32_t *B, uint64_t ldb, uint32_t *C, uint64_t ldc,
-                            void *ws, int sm_count, cudaStream_t s, int *launches,
-                            bool reduce_inputs = false, const uint8_t *Aimg = nullptr);
+// error flag and partial sums; all zero at launch, and again after it
+size_t block_tc_workspace_bytes(uint64_t m, uint64_t nb);
+size_t block_tc_bimg_bytes(uint64_t k, uint64_t nb, int n_mod);
+struct BlockScratch {
+    void *ws;        // block_tc_workspace_bytes, zero; the error flag is its first word
+    uint8_t *bimg;   // block_tc_bimg_bytes: B's digit tiles
+};
+// n_mod = 1: C = A B mod mods[0].  More: the residue passes, A and B reduced
+// modulo each; pass l writes the dense m x nb matrix C + l m nb (ldc = nb).
+cudaError_t launch_block_tc(const uint32_t *mods, int n_mod, uint64_t m, uint64_t k, uint64_t nb,
+                            const uint32_t *A, uint64_t lda, const uint32_t *B, uint64_t ldb, uint32_t *C,
+                            uint64_t ldc, const BlockScratch &sc, int sm_count, cudaStream_t s,
+                            int *launches, const uint8_t *Aimg = nullptr, size_t img_bytes = 0);
 // Prepared A: digit image of A for one modulus (block_prep_a_bytes(m, k)
-// bytes), consumed by launch_block_tc through Aimg (A and lda then unused).
+// bytes), consumed by launch_block_tc through Aimg (A and lda then unused; pass
+// l reads the image at l img_bytes).
 size_t block_prep_a_bytes(uint64_t m, uint64_t k);
 cudaError_t launch_block_prep_a(const Mod &mod, uint64_t m, uint64_t k, const uint32_t *A,
                                 uint64_t lda, bool reduce_inputs, uint8_t *img, cudaStream_t s);
-uint32_t *block_tc_err_flag(void *ws, uint64_t m, uint64_t k, uint64_t nb);
 // Runs the bounded-wait self test; *status_bits gets the device error word.
 cudaError_t wait_selftest(uint64_t limit_ns, cudaStream_t s, uint32_t *status_bits);
 cudaError_t launch_block_cc(Repr r, const Mod &mod, uint64_t kbound, uint64_t m, uint64_t k,
@@ -211,11 +218,13 @@ struct gfp_ctx {
     uint32_t *stage_out = nullptr;
     size_t stage_out_elems = 0;
 
-    // block-product workspace (B digit image, column-major partial sums,
-    // error flag); zero outside calls except the B image; grown on demand
+    // block-product workspace (error flag, column-major partial sums), zero
+    // outside calls, B's digit tiles, and the residue matrices of the passes of
+    // a large modulus; all grown on demand
     void *blk_ws = nullptr;
     size_t blk_ws_bytes = 0;
-    uint64_t blk_m = 0, blk_k = 0, blk_nb = 0;   // shape whose error flag is live
+    void *blk_bimg = nullptr, *blk_res = nullptr;
+    size_t blk_bimg_bytes = 0, blk_res_bytes = 0;
 
     // tuned plan: (p, lg_n) -> entry
     std::map<std::pair<uint32_t, uint32_t>, gfp_plan_entry> plan;

@@ -457,6 +457,8 @@ GFP_API gfp_status gfp_context_destroy(gfp_ctx *ctx)
     if (ctx->stage) cudaFree(ctx->stage);
     if (ctx->stage_out) cudaFree(ctx->stage_out);
     if (ctx->blk_ws) cudaFree(ctx->blk_ws);
+    if (ctx->blk_bimg) cudaFree(ctx->blk_bimg);
+    if (ctx->blk_res) cudaFree(ctx->blk_res);
     delete ctx;
     return GFP_OK;
 }
@@ -770,30 +772,57 @@ static int block_sms(const gfp_ctx *ctx)
     return (ctx->blk_sms > 0 && ctx->blk_sms < ctx->sm_count) ? ctx->blk_sms : ctx->sm_count;
 }
 
-// Block-product workspace of the context for shape (m, k, nb) followed by
-// `passes` residue matrices (m x nb uint32 each); the caller holds ctx->mu.
-static gfp_status ensure_block_ws(gfp_ctx *ctx, uint64_t m, uint64_t k, uint64_t nb, int passes,
-                                  cudaStream_t s)
+// Grows one buffer of the block product to `need` bytes; the old one may still
+// be read by work in flight.
+static gfp_status grow_block_buffer(void **buf, size_t *have, size_t need, bool zero)
 {
-    const size_t tc_need = block_tc_workspace_bytes(m, k, nb);
-    const size_t need = tc_need + (size_t)passes * m * nb * 4;
-    if (need > ctx->blk_ws_bytes) {
-        GFP_CUDA_TRY(cudaDeviceSynchronize());
-        if (ctx->blk_ws) cudaFree(ctx->blk_ws);
-        ctx->blk_ws = nullptr;
-        ctx->blk_ws_bytes = 0;
-        if (cudaMalloc(&ctx->blk_ws, need) != cudaSuccess) return GFP_ERR_NOMEM;
-        GFP_CUDA_TRY(cudaMemset(ctx->blk_ws, 0, need));
-        ctx->blk_ws_bytes = need;
+    if (need <= *have) return GFP_OK;
+    GFP_CUDA_TRY(cudaDeviceSynchronize());
+    if (*buf) cudaFree(*buf);
+    *buf = nullptr;
+    *have = 0;
+    if (cudaMalloc(buf, need) != cudaSuccess) {
+        *buf = nullptr;
+        return GFP_ERR_NOMEM;
     }
-    if (m != ctx->blk_m || k != ctx->blk_k || nb != ctx->blk_nb) {
-        // the partial-sum region moves with the shape: clear it
-        const size_t z = block_tc_bimg_bytes(k, nb);
-        GFP_CUDA_TRY(cudaMemsetAsync((uint8_t *)ctx->blk_ws + z, 0, tc_need - z, s));
-        ctx->blk_m = m;
-        ctx->blk_k = k;
-        ctx->blk_nb = nb;
+    if (zero) GFP_CUDA_TRY(cudaMemset(*buf, 0, need));
+    *have = need;
+    return GFP_OK;
+}
+
+// Block-product buffers of the context for an m x k by k x nb product with
+// n_mod moduli (the residue matrices of the passes where there are several);
+// the caller holds ctx->mu.
+static gfp_status ensure_block_ws(gfp_ctx *ctx, uint64_t m, uint64_t k, uint64_t nb, int n_mod)
+{
+    gfp_status st = grow_block_buffer(&ctx->blk_ws, &ctx->blk_ws_bytes, block_tc_workspace_bytes(m, nb), true);
+    if (st == GFP_OK)
+        st = grow_block_buffer(&ctx->blk_bimg, &ctx->blk_bimg_bytes, block_tc_bimg_bytes(k, nb, n_mod), false);
+    if (st == GFP_OK && n_mod > 1)
+        st = grow_block_buffer(&ctx->blk_res, &ctx->blk_res_bytes, (size_t)n_mod * m * nb * 4, false);
+    return st;
+}
+
+// The tensor-core product through the context's buffers: one modulus directly,
+// several as residue passes recombined modulo rc.p.
+static gfp_status run_block_tc(gfp_ctx *ctx, uint32_t p, const RnsConst *rc, uint64_t m, uint64_t k, uint64_t nb,
+                               const uint32_t *A, uint64_t lda, const uint32_t *B, uint64_t ldb, uint32_t *C,
+                               uint64_t ldc, const uint8_t *Aimg, size_t img_bytes, cudaStream_t s)
+{
+    std::lock_guard<std::mutex> g(ctx->mu);
+    const int n_mod = rc ? rc->L : 1;
+    const gfp_status st = ensure_block_ws(ctx, m, k, nb, n_mod);
+    if (st != GFP_OK) return st;
+    const BlockScratch sc{ctx->blk_ws, (uint8_t *)ctx->blk_bimg};
+    uint32_t *R = (uint32_t *)ctx->blk_res;
+    int launches = 0;
+    GFP_CUDA_TRY(launch_block_tc(rc ? rc->mod : &p, n_mod, m, k, nb, A, lda, B, ldb, n_mod > 1 ? R : C,
+                                 n_mod > 1 ? nb : ldc, sc, block_sms(ctx), s, &launches, Aimg, img_bytes));
+    if (n_mod > 1) {
+        GFP_CUDA_TRY(launch_block_crt(R, m, nb, C, ldc, *rc, ctx->sm_count, s));
+        ++launches;
     }
+    ctx->launches += launches;
     return GFP_OK;
 }
 
@@ -812,8 +841,10 @@ GFP_API gfp_status gfp_matmul_block(gfp_ctx *ctx, uint32_t p, uint64_t m, uint64
         return GFP_OK;
     }
     // tensor cores: directly for p <= 65791, through residues modulo small
-    // primes (one pass each, then a Garner recombination) above that
-    const bool layout_ok = block_tc_layout_ok(A, lda);
+    // primes (one pass each, then a Garner recombination) above that.  Forcing
+    // them asks for a layout that 16-byte loads take; the automatic choice also
+    // uses them for other layouts, with 4-byte loads
+    const bool layout_ok = ctx->forced == GFP_REPR_AUTO || block_tc_layout_ok(A, lda);
     RnsConst rc;
     const bool direct_ok = layout_ok && p <= BLOCK_TC_MAX_P;
     bool rns_ok = layout_ok && p > BLOCK_TC_MAX_P && block_rns_plan(p, k, &rc);
@@ -847,26 +878,7 @@ GFP_API gfp_status gfp_matmul_block(gfp_ctx *ctx, uint32_t p, uint64_t m, uint64
         ctx->launches++;
         return GFP_OK;
     }
-    std::lock_guard<std::mutex> g(ctx->mu);
-    const size_t tc_need = block_tc_workspace_bytes(m, k, nb);
-    {
-        const gfp_status st = ensure_block_ws(ctx, m, k, nb, rns_ok ? rc.L : 0, s);
-        if (st != GFP_OK) return st;
-    }
-    int launches = 0;
-    if (!rns_ok) {
-        GFP_CUDA_TRY(launch_block_tc(mod, m, k, nb, A, lda, B, ldb, C, ldc, ctx->blk_ws, block_sms(ctx),
-                                     s, &launches));
-    } else {
-        uint32_t *R = (uint32_t *)((uint8_t *)ctx->blk_ws + tc_need);
-        for (int l = 0; l < rc.L; ++l)
-            GFP_CUDA_TRY(launch_block_tc(make_mod(rc.mod[l]), m, k, nb, A, lda, B, ldb, R + (size_t)l * m * nb,
-                                         nb, ctx->blk_ws, block_sms(ctx), s, &launches, true));
-        GFP_CUDA_TRY(launch_block_crt(R, m, nb, C, ldc, rc, ctx->sm_count, s));
-        ++launches;
-    }
-    ctx->launches += launches;
-    return GFP_OK;
+    return run_block_tc(ctx, p, rns_ok ? &rc : nullptr, m, k, nb, A, lda, B, ldb, C, ldc, nullptr, 0, s);
 }
 
 // A prepared once for repeated block products: its tensor-core digit
@@ -959,25 +971,8 @@ GFP_API gfp_status gfp_matmul_block_prepared(gfp_ctx *ctx, const gfp_block_prep 
         const gfp_status st = check_range_rows(ctx, B, k, nb, ldb, pp->p, s);
         if (st != GFP_OK) return st;
     }
-    std::lock_guard<std::mutex> g(ctx->mu);
-    const gfp_status st = ensure_block_ws(ctx, m, k, nb, pp->passes > 1 ? pp->passes : 0, s);
-    if (st != GFP_OK) return st;
-    int launches = 0;
-    const uint8_t *img = (const uint8_t *)pp->mem;
-    if (pp->passes == 1) {
-        GFP_CUDA_TRY(launch_block_tc(make_mod(pp->p), m, k, nb, nullptr, 0, B, ldb, C, ldc,
-                                     ctx->blk_ws, block_sms(ctx), s, &launches, false, img));
-    } else {
-        uint32_t *R = (uint32_t *)((uint8_t *)ctx->blk_ws + block_tc_workspace_bytes(m, k, nb));
-        for (int l = 0; l < pp->passes; ++l)
-            GFP_CUDA_TRY(launch_block_tc(make_mod(pp->rc.mod[l]), m, k, nb, nullptr, 0, B, ldb,
-                                         R + (size_t)l * m * nb, nb, ctx->blk_ws, block_sms(ctx), s,
-                                         &launches, true, img + pp->per * l));
-        GFP_CUDA_TRY(launch_block_crt(R, m, nb, C, ldc, pp->rc, ctx->sm_count, s));
-        ++launches;
-    }
-    ctx->launches += launches;
-    return GFP_OK;
+    return run_block_tc(ctx, pp->p, pp->passes > 1 ? &pp->rc : nullptr, m, k, nb, nullptr, 0, B, ldb, C, ldc,
+                        (const uint8_t *)pp->mem, pp->per, s);
 }
 
 GFP_API gfp_status gfp_matmul_block_csr(gfp_ctx *ctx, uint32_t p, uint64_t m, uint64_t k,
@@ -1029,9 +1024,8 @@ GFP_API gfp_status gfp_context_check(gfp_ctx *ctx)
     // device-side checks (GFP_DEVICE_CHECKS builds; always 0 otherwise)
     const uint32_t dbits = csr_check_bits() | dot_check_bits();
     if (!ctx->blk_ws) return dbits ? GFP_ERR_INVALID : GFP_OK;
-    uint32_t *flag = block_tc_err_flag(ctx->blk_ws, ctx->blk_m, ctx->blk_k, ctx->blk_nb);
     uint32_t h = 0;
-    GFP_CUDA_TRY(cudaMemcpy(&h, flag, 4, cudaMemcpyDeviceToHost));
+    GFP_CUDA_TRY(cudaMemcpy(&h, ctx->blk_ws, 4, cudaMemcpyDeviceToHost));   // the error flag
     if (h) {
         GFP_CUDA_TRY(cudaMemset(ctx->blk_ws, 0, ctx->blk_ws_bytes));
         return GFP_ERR_TIMEOUT;
