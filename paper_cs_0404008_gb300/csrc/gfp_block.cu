@@ -21,14 +21,15 @@
 //   once per range, and A alone streams.  A's digits go to TMEM, from where
 //   the MMAs read them: shared memory sees only B, and the rest of its 256 KiB
 //   per SM stays L1, which is where loads in flight land.  Roles per CTA:
-//     warps 0-7    load A with 16-byte loads, 24 in flight per thread (96 KiB
-//                  per SM), centre and split the words in registers and store
-//                  the fp16 digits (tcgen05.st) to one of two TMEM slots.  No
-//                  warp waits for another: slots pass through mbarriers alone
-//     warps 8-15   drain the accumulators (tcgen05.ld), recombine, reduce and
+//     warps 0-15   load A with 16-byte loads (64 KiB in flight per SM), centre
+//                  and split the words in registers and store the fp16 digits
+//                  (tcgen05.st) to TMEM: two groups of eight warps with a slot
+//                  each take alternate k-blocks.  No warp waits for another:
+//                  slots pass through mbarriers alone
+//     warps 16-23  drain the accumulators (tcgen05.ld), recombine, reduce and
 //                  add the residues to the partial sums
-//     warp 16      owns TMEM and issues the MMAs (one thread)
-//     warp 17      bulk-copies B's digit tiles, split once by a small kernel
+//     warp 24      owns TMEM and issues the MMAs
+//     warp 25      bulk-copies B's digit tiles, split once by a small kernel
 //                  before this one, each as soon as the MMAs of the K range
 //                  before have read its place for the last time
 //   Each output meets the partial sums of its K ranges in a column-major u32
@@ -70,12 +71,14 @@ constexpr int SLOTS = 2;
 constexpr uint32_t SLOT_COLS = 64;                            // 32 columns per digit
 constexpr uint32_t ACC_COLS = 3 * NT;                         // ll, middle, hh
 constexpr uint32_t A_COL0 = 2 * ACC_COLS;                     // behind two accumulator sets
-constexpr int CONV_WARPS = 8, EPI_WARPS = 8;
-constexpr int W_EPI0 = CONV_WARPS, W_MMA = CONV_WARPS + EPI_WARPS, W_BPROD = W_MMA + 1;
-constexpr int THREADS = 32 * (W_MMA + 4);                     // 640: two warps of the last group idle
-// registers per thread: 96 at launch, then shared out by role (warpgroups)
-constexpr int REGS_LAUNCH = 96, REGS_CONV = 152, REGS_EPI = 64, REGS_MMA = 48;
-static_assert(REGS_LAUNCH * THREADS == 32 * (REGS_CONV * CONV_WARPS + REGS_EPI * EPI_WARPS + REGS_MMA * 4),
+constexpr int CONV_GROUPS = 2, CONV_WARPS = 8, EPI_WARPS = 8;   // converter warps of a group
+constexpr int W_EPI0 = CONV_GROUPS * CONV_WARPS, W_MMA = W_EPI0 + EPI_WARPS, W_BPROD = W_MMA + 1;
+static_assert(CONV_GROUPS == SLOTS, "each group has a slot of its own");
+constexpr int THREADS = 32 * (W_MMA + 4);                     // 896: two warps of the last group idle
+// registers per thread: 72 at launch, then shared out by role (warpgroups)
+constexpr int REGS_LAUNCH = 72, REGS_CONV = 88, REGS_EPI = 56, REGS_MMA = 40;
+static_assert(REGS_LAUNCH * THREADS ==
+                  32 * (REGS_CONV * CONV_GROUPS * CONV_WARPS + REGS_EPI * EPI_WARPS + REGS_MMA * 4),
               "the roles' registers are exactly those the block is launched with");
 static_assert(REGS_LAUNCH * THREADS <= 65536, "one CTA per SM");
 static_assert(W_EPI0 % 4 == 0, "an epilogue warp reads the TMEM lanes of its index modulo 4");
@@ -325,30 +328,36 @@ struct ALoads {
     Walk w;
     uint32_t j;           // k-block within the K range
     const uint8_t *src;   // this lane's first piece of that k-block
+    bool end;             // no k-block left
+    static constexpr uint32_t STRIDE = MODE == A_PREP ? A8_TILE_BYTES : BK * 4;
     __device__ __forceinline__ void locate(const Args &a, int warp, int lane)
     {
-        j = 0;
         if constexpr (MODE == A_PREP) {
-            src = a.Aimg + ((uint64_t)w.mt * a.img_kblocks + a.img_kb0 + w.kb0) * A8_TILE_BYTES + warp * 2048 +
+            src = a.Aimg + ((uint64_t)w.mt * a.img_kblocks + a.img_kb0 + w.kb0 + j) * A8_TILE_BYTES + warp * 2048 +
                   lane * 16;
         } else {
             const uint64_t row = (uint64_t)w.mt * BM + (warp & 3) * 32 + (warp >> 2) * 16 + (lane >> 2);
-            const uint64_t col = (uint64_t)w.kb0 * BK + (lane & 3) * 4;
+            const uint64_t col = (uint64_t)(w.kb0 + j) * BK + (lane & 3) * 4;
             src = reinterpret_cast<const uint8_t *>(a.A + row * a.lda + col);
         }
     }
-    // to the next k-block; the last one of the CTA is its own successor, so that
-    // the loads need no condition and write straight to their registers
-    __device__ __forceinline__ void step(const Args &a, int warp, int lane)
+    // n k-blocks on
+    __device__ __forceinline__ void advance(const Args &a, int warp, int lane, uint32_t n)
     {
-        if (++j < w.kbs) {
-            src += MODE == A_PREP ? A8_TILE_BYTES : BK * 4;
-        } else if (w.left > 1) {
-            w.next(a);
-            locate(a, warp, lane);
-        } else {
-            --j;
+        j += n;
+        if (j < w.kbs) {
+            src += n * STRIDE;
+            return;
         }
+        do {
+            j -= w.kbs;
+            if (w.left <= 1) {
+                end = true;
+                return;
+            }
+            w.next(a);
+        } while (j >= w.kbs);
+        locate(a, warp, lane);
     }
     __device__ __forceinline__ void load(const Args &a, int warp, int lane, AWords<MODE> &r) const
     {
@@ -422,7 +431,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_block_tc(const __grid_constant__
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t *btiles = smem;                                    // RK digit tiles of B
     Bars *bars = reinterpret_cast<Bars *>(btiles + (size_t)RK * B_TILE_BYTES);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // one lane's value for the whole warp: the compiler may then keep what
+    // depends on it in uniform registers, where tcgen05 takes its addresses from
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
 
     const uint64_t u0 = a.units * blockIdx.x / gridDim.x;
     const uint64_t u1 = a.units * (blockIdx.x + 1) / gridDim.x;
@@ -459,109 +470,128 @@ __global__ void __launch_bounds__(THREADS, 1) k_block_tc(const __grid_constant__
     // is complete (it waited for it), so A may be read at once; the roles that
     // touch B's digits or the partial sums wait for it.
 
-    if (warp < CONV_WARPS) {
+    if (warp < W_EPI0) {
         // ---------------- converters: A to fp16 digits ----------------
         ptx::regs_inc<REGS_CONV>();
-        // k-blocks of A in flight in registers: 64 KiB per SM
-        constexpr int D = MODE == A_PREP ? 4 : 2;
+        // each group takes every second k-block: while one waits for its slot's
+        // MMAs the other converts
+        const int group = warp / CONV_WARPS, gw = warp % CONV_WARPS;
+        // k-blocks in flight in registers: 64 KiB per SM over both groups
+        constexpr int D = MODE == A_PREP ? 2 : 1;
         AWords<MODE> buf[D];
         ALoads<MODE> ld;
         ld.w.start(a, u0, u1);
-        ld.locate(a, warp, lane);
-        Walk w = ld.w;
+        ld.j = 0;
+        ld.end = false;
+        ld.locate(a, gw, lane);
+        if (group) ld.advance(a, gw, lane, 1);
+        uint32_t loaded = 0;
 #pragma unroll
         for (int d = 0; d < D; ++d) {
-            ld.load(a, warp, lane, buf[d]);
-            ld.step(a, warp, lane);
+            if (!ld.end) {
+                ld.load(a, gw, lane, buf[d]);
+                ld.advance(a, gw, lane, CONV_GROUPS);
+                ++loaded;
+            }
         }
-        const uint32_t tslot = tmem + A_COL0 + ((uint32_t)((warp & 3) * 32 + (warp >> 2) * 16) << 16);
-        const uint32_t bar_empty = ptx::smem_u32(&bars->a_empty[0]), bar_conv = ptx::smem_u32(&bars->conv[0]);
-        uint32_t j = 0, s = 0, ph = 1;   // k-block within the K range, slot
+        const uint32_t tslot = tmem + A_COL0 + (uint32_t)group * SLOT_COLS +
+                               ((uint32_t)((gw & 3) * 32 + (gw >> 2) * 16) << 16);
+        const uint32_t bar_empty = ptx::smem_u32(&bars->a_empty[group]), bar_conv = ptx::smem_u32(&bars->conv[group]);
+        uint32_t ph = 1;
         bool run = true;
         while (run) {
 #pragma unroll
             for (int d = 0; d < D; ++d) {
+                if (loaded == 0) {
+                    run = false;
+                    break;
+                }
                 uint32_t hi[16], lo[16];
                 convert_a<MODE, PRE>(a, buf[d], hi, lo);
-                ld.load(a, warp, lane, buf[d]);
-                ld.step(a, warp, lane);
-                if (!w.left || !wait_bar_warp(bar_empty + s * 8u, ph, abort, a.err)) {
+                if (!ld.end) {
+                    ld.load(a, gw, lane, buf[d]);
+                    ld.advance(a, gw, lane, CONV_GROUPS);
+                } else {
+                    --loaded;
+                }
+                if (!wait_bar_warp(bar_empty, ph, abort, a.err)) {
                     run = false;
                     break;
                 }
                 ptx::tc_fence_after();
-                ptx::tmem_st_16x256b_x4(tslot + s * SLOT_COLS, hi);
-                ptx::tmem_st_16x256b_x4(tslot + s * SLOT_COLS + SLOT_COLS / 2, lo);
+                ptx::tmem_st_16x256b_x4(tslot, hi);
+                ptx::tmem_st_16x256b_x4(tslot + SLOT_COLS / 2, lo);
                 ptx::tmem_st_wait();
                 ptx::tc_fence_before();
                 __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(bar_conv + s * 8u);
-                s ^= 1u;
-                if (s == 0) ph ^= 1u;
-                if (++j == w.kbs) {
-                    j = 0;
-                    w.next(a);
-                }
+                if (lane == 0) ptx::mbar_arrive(bar_conv);
+                ph ^= 1u;
             }
         }
     } else if (warp == W_MMA) {
-        // ---------------- MMA issue (one thread) ----------------
+        // ---------------- MMA issue ----------------
+        // The whole warp walks the loop, so that addresses and descriptors stay
+        // in uniform registers, and one elected lane issues: with a lone lane in
+        // the loop every operand of every MMA was moved there first, and the
+        // eight MMAs of a k-block took 750-1000 cycles to issue against the 503
+        // they need
         ptx::regs_dec<REGS_MMA>();
-        if (lane == 0) {
-            Walk w;
-            w.start(a, u0, u1);
-            uint32_t s = 0, ph = 0, bset = 0, used = 0, b = 0, bph = 1;
-            bool ok = true, fresh = true;   // fresh: the K range's first unit
-            while (w.left && ok) {
-                // the accumulator set was drained by the unit before the last
-                if (!wait_bar(ptx::smem_u32(&bars->acc_empty[b]), bph, abort, a.err)) break;
-                ptx::tc_fence_after();
-                const uint32_t d_lo = tmem + b * ACC_COLS;   // A low digit x [B lo | B hi]: ll, lh
-                const uint32_t d_hi = d_lo + NT;             // A high digit x [B lo | B hi]: hl, hh
-                const bool final = w.left == 1 || w.mt + 1 == a.m_tiles;   // the K range's last unit
-                uint32_t t = bset * a.bset_tiles;
-                uint64_t db = ptx::sdesc_k_sw128(ptx::smem_u32(btiles + t * B_TILE_BYTES));
-                for (uint32_t j = 0; j < w.kbs; ++j, ++t, db += B_TILE_BYTES >> 4) {
-                    ok = wait_bar(ptx::smem_u32(&bars->conv[s]), ph, abort, a.err);
-                    if (ok && fresh) {
-                        ok = wait_bar(ptx::smem_u32(&bars->b_full[t]), (used >> t) & 1u, abort, a.err);
-                        used ^= 1u << t;
-                    }
-                    if (!ok) break;
-                    ptx::tc_fence_after();
-                    const uint32_t ah = tmem + A_COL0 + s * SLOT_COLS, al = ah + SLOT_COLS / 2;
-#pragma unroll
-                    for (uint32_t kk = 0; kk < 4; ++kk) {
-                        // 16 K: eight TMEM columns of A, 32 bytes of B inside the swizzle atom
-                        const uint32_t acc = (j > 0 || kk > 0) ? 1u : 0u;
-                        ptx::mma_f16_ts(d_lo, al + 8 * kk, db + 2 * kk, IDESC, acc);
-                        if (acc) {
-                            ptx::mma_f16_ts(d_hi, ah + 8 * kk, db + 2 * kk, IDESC, 1u);
-                        } else {
-                            // the middle columns already hold lh; hh starts from zero
-                            ptx::mma_f16_ts(d_hi, ah, db, IDESC_HALF, 1u);
-                            ptx::mma_f16_ts(d_hi + NT, ah, db + ((64 * 128) >> 4), IDESC_HALF, 0u);
-                        }
-                    }
-                    ptx::mma_commit(ptx::smem_u32(&bars->a_empty[s]));
-                    if (final) ptx::mma_commit(ptx::smem_u32(&bars->b_empty[t]));
-                    s ^= 1u;
-                    if (s == 0) ph ^= 1u;
+        const uint32_t lead = ptx::elect_one();
+        Walk w;
+        w.start(a, u0, u1);
+        uint32_t s = 0, ph = 0, bset = 0, used = 0, b = 0, bph = 1;
+        bool ok = true, fresh = true;   // fresh: the K range's first unit
+        while (w.left && ok) {
+            // the accumulator set was drained by the unit before the last
+            if (!wait_bar_warp(ptx::smem_u32(&bars->acc_empty[b]), bph, abort, a.err)) break;
+            ptx::tc_fence_after();
+            const uint32_t d_lo = tmem + b * ACC_COLS;   // A low digit x [B lo | B hi]: ll, lh
+            const uint32_t d_hi = d_lo + NT;             // A high digit x [B lo | B hi]: hl, hh
+            const bool final = w.left == 1 || w.mt + 1 == a.m_tiles;   // the K range's last unit
+            uint32_t t = bset * a.bset_tiles;
+            uint64_t db = ptx::sdesc_k_sw128(ptx::smem_u32(btiles + t * B_TILE_BYTES));
+            for (uint32_t j = 0; j < w.kbs; ++j, ++t, db += B_TILE_BYTES >> 4) {
+                ok = wait_bar_warp(ptx::smem_u32(&bars->conv[s]), ph, abort, a.err);
+                if (ok && fresh) {
+                    ok = wait_bar_warp(ptx::smem_u32(&bars->b_full[t]), (used >> t) & 1u, abort, a.err);
+                    used ^= 1u << t;
                 }
                 if (!ok) break;
-                ptx::mma_commit(ptx::smem_u32(&bars->acc_full[b]));
-                b ^= 1u;
-                if (b == 0) bph ^= 1u;
-                fresh = w.next(a);
-                if (fresh && ++bset == a.bsets) bset = 0;
+                ptx::tc_fence_after();
+                const uint32_t ah = tmem + A_COL0 + s * SLOT_COLS, al = ah + SLOT_COLS / 2;
+                // 16 K: eight TMEM columns of A, 32 bytes of B inside the swizzle atom
+                if (j == 0) {
+                    // the middle columns then hold lh; hh starts from zero
+                    ptx::mma_f16_ts(lead, d_lo, al, db, IDESC, 0u);
+                    ptx::mma_f16_ts(lead, d_hi, ah, db, IDESC_HALF, 1u);
+                    ptx::mma_f16_ts(lead, d_hi + NT, ah, db + ((64 * 128) >> 4), IDESC_HALF, 0u);
+                } else {
+                    ptx::mma_f16_ts(lead, d_lo, al, db, IDESC, 1u);
+                    ptx::mma_f16_ts(lead, d_hi, ah, db, IDESC, 1u);
+                }
+#pragma unroll
+                for (uint32_t kk = 1; kk < 4; ++kk) {
+                    ptx::mma_f16_ts(lead, d_lo, al + 8 * kk, db + 2 * kk, IDESC, 1u);
+                    ptx::mma_f16_ts(lead, d_hi, ah + 8 * kk, db + 2 * kk, IDESC, 1u);
+                }
+                ptx::mma_commit(lead, ptx::smem_u32(&bars->a_empty[s]));
+                if (final) ptx::mma_commit(lead, ptx::smem_u32(&bars->b_empty[t]));
+                s ^= 1u;
+                if (s == 0) ph ^= 1u;
             }
-            // every MMA issued by this CTA has completed before TMEM is freed
-            ptx::mma_commit(ptx::smem_u32(&bars->drain));
-            const uint64_t t0 = ptx::globaltimer();
-            while (!ptx::mbar_try_wait(ptx::smem_u32(&bars->drain), 0) &&
-                   ptx::globaltimer() - t0 < WAIT_NS) {
-            }
+            if (!ok) break;
+            ptx::mma_commit(lead, ptx::smem_u32(&bars->acc_full[b]));
+            b ^= 1u;
+            if (b == 0) bph ^= 1u;
+            fresh = w.next(a);
+            if (fresh && ++bset == a.bsets) bset = 0;
         }
+        // every MMA issued by this CTA has completed before TMEM is freed
+        ptx::mma_commit(lead, ptx::smem_u32(&bars->drain));
+        const uint64_t t0 = ptx::globaltimer();
+        while (!ptx::mbar_try_wait(ptx::smem_u32(&bars->drain), 0) && ptx::globaltimer() - t0 < WAIT_NS) {
+        }
+        __syncwarp();
     } else if (warp > W_MMA) {
         // ---------------- B digit tiles, once per K range (bulk copies) ----------------
         ptx::regs_dec<REGS_MMA>();

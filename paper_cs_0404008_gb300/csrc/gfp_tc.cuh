@@ -81,6 +81,18 @@ __device__ __forceinline__ void ld_if(uint32_t &v, const uint32_t *p, bool on)
                  : "l"(p), "r"((uint32_t)on));
 }
 
+// 1 in one lane of a converged warp, 0 in the others
+__device__ __forceinline__ uint32_t elect_one()
+{
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(r));
+    return r;
+}
+
 // ---- registers of a warpgroup ----
 template <int N>
 __device__ __forceinline__ void regs_inc()
@@ -114,14 +126,16 @@ __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::
 
 // D[tmem] (+)= A[tmem] * B[smem]^T: lane = row of A, each 32-bit column two
 // consecutive K (the lower one in the low half)
-__device__ __forceinline__ void mma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
+// (issued by the lane whose `lead` is not 0)
+__device__ __forceinline__ void mma_f16_ts(uint32_t lead, uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
                                            uint32_t idesc, uint32_t accumulate)
 {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
+        "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(lead)
         : "memory");
 }
 // 16 lanes x 32 columns of 32-bit values: thread i of the warp writes, for each
@@ -137,11 +151,16 @@ __device__ __forceinline__ void tmem_st_16x256b_x4(uint32_t taddr, const uint32_
         : "memory");
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-// arrive on an mbarrier once all previously issued tcgen05.mma have completed
-__device__ __forceinline__ void mma_commit(uint32_t bar)
+// arrive on an mbarrier once all tcgen05.mma the lane issued have completed
+// (the lane whose `lead` is not 0)
+__device__ __forceinline__ void mma_commit(uint32_t lead, uint32_t bar)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-                 : "memory");
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "setp.ne.b32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar),
+        "r"(lead)
+        : "memory");
 }
 // 32 lanes x 8 columns of 32-bit values; thread i of the warp gets lane (base + i)
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8])
