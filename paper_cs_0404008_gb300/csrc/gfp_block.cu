@@ -138,6 +138,7 @@ struct Args {
     uint32_t magic;           // floor(2^32 / p)
     int32_t smagic;           // the same, at most 2^31 - 1
     uint32_t magic47;         // floor(2^47 / p) of a residue-pass modulus (p > 65000)
+    uint32_t backward;        // each CTA takes its units in reverse order
     uint32_t direct;          // one K range: residues go to C, not to the workspace
     uint32_t m_tiles, n_tiles, kblocks;
     uint32_t ranges, r_base, r_rem;   // K ranges of r_base k-blocks, the first r_rem one more
@@ -206,8 +207,8 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatil
     return __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
 }
 
-// Walks a CTA's units in order: row tiles innermost, then K ranges, then
-// column tiles.
+// Walks a CTA's units in order (row tiles innermost, then K ranges, then
+// column tiles), or backwards.
 struct Walk {
     uint32_t mt, rg, nt;
     uint32_t kb0, kbs;   // first k-block and number of k-blocks of the K range
@@ -219,22 +220,40 @@ struct Walk {
     }
     __device__ __forceinline__ void start(const Args &a, uint64_t u0, uint64_t u1)
     {
+        const uint64_t u = a.backward ? u1 - 1 : u0;
         left = (uint32_t)(u1 - u0);
-        mt = (uint32_t)(u0 % a.m_tiles);
-        const uint64_t t = u0 / a.m_tiles;
+        mt = (uint32_t)(u % a.m_tiles);
+        const uint64_t t = u / a.m_tiles;
         rg = (uint32_t)(t % a.ranges);
         nt = (uint32_t)(t / a.ranges);
         range(a);
     }
+    // the last of its K range's units, in walking order
+    __device__ __forceinline__ bool last_of_range(const Args &a) const
+    {
+        return left == 1 || (a.backward ? mt == 0 : mt + 1 == a.m_tiles);
+    }
     // to the next unit; true when its K range or column tile is another one
     __device__ __forceinline__ bool next(const Args &a)
     {
+        const bool turn = last_of_range(a);
         --left;
-        if (++mt < a.m_tiles) return false;
-        mt = 0;
-        if (++rg == a.ranges) {
-            rg = 0;
-            ++nt;
+        if (!turn) {
+            mt += a.backward ? ~0u : 1u;
+            return false;
+        }
+        if (!a.backward) {
+            mt = 0;
+            if (++rg == a.ranges) {
+                rg = 0;
+                ++nt;
+            }
+        } else {
+            mt = a.m_tiles - 1;
+            if (rg-- == 0) {
+                rg = a.ranges - 1;
+                --nt;
+            }
         }
         range(a);
         return true;
@@ -323,7 +342,7 @@ struct AWords {
 };
 
 // Runs ahead of the conversion: where the next k-block's words are.
-template <int MODE>
+template <int MODE, bool PRE>
 struct ALoads {
     Walk w;
     uint32_t j;           // k-block within the K range
@@ -370,7 +389,9 @@ struct ALoads {
             for (int i = 0; i < 8; ++i) {
                 const uint8_t *q = ((i & 1) ? src8 : src) + (i >> 1) * 64;
                 if constexpr (MODE == A_VEC) {
-                    ptx::ld_stream4(r.v[i], q);
+                    // a residue pass leaves A in L2 for the pass behind it
+                    if constexpr (PRE) ptx::ld_l2_4(r.v[i], q);
+                    else ptx::ld_stream4(r.v[i], q);
                 } else {
                     const uint32_t *q1 = reinterpret_cast<const uint32_t *>(q);
                     ptx::ld_if(r.v[i].x, q1, true);
@@ -462,7 +483,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_block_tc(const __grid_constant__
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    const uint32_t tmem = bars->tmem_base;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);   // uniform, as above
     volatile uint32_t *abort = &bars->abort;
     // Programmatic dependent launch: this grid may be placed while the previous
     // kernel of the stream, the one that makes B's digits or reduces the partial
@@ -479,7 +500,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_block_tc(const __grid_constant__
         // k-blocks in flight in registers: 64 KiB per SM over both groups
         constexpr int D = MODE == A_PREP ? 2 : 1;
         AWords<MODE> buf[D];
-        ALoads<MODE> ld;
+        ALoads<MODE, PRE> ld;
         ld.w.start(a, u0, u1);
         ld.j = 0;
         ld.end = false;
@@ -547,7 +568,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_block_tc(const __grid_constant__
             ptx::tc_fence_after();
             const uint32_t d_lo = tmem + b * ACC_COLS;   // A low digit x [B lo | B hi]: ll, lh
             const uint32_t d_hi = d_lo + NT;             // A high digit x [B lo | B hi]: hl, hh
-            const bool final = w.left == 1 || w.mt + 1 == a.m_tiles;   // the K range's last unit
+            const bool final = w.last_of_range(a);
             uint32_t t = bset * a.bset_tiles;
             uint64_t db = ptx::sdesc_k_sw128(ptx::smem_u32(btiles + t * B_TILE_BYTES));
             for (uint32_t j = 0; j < w.kbs; ++j, ++t, db += B_TILE_BYTES >> 4) {
@@ -845,14 +866,6 @@ __global__ void __launch_bounds__(32 * CONV_WARPS)
     *reinterpret_cast<uint4 *>(out + 1536) = make_uint4(lb[4], lb[5], lb[6], lb[7]);
 }
 
-// x mod m for x < 2^40 and m < 2^17, minv = floor((2^64 - 1) / m): the
-// multiply-high quotient is floor(x / m) or one less
-__device__ __forceinline__ uint32_t mod_small64(uint64_t x, uint32_t m, uint64_t minv)
-{
-    const uint64_t r = x - __umul64hi(x, minv) * m;
-    return (uint32_t)(r >= m ? r - m : r);
-}
-
 // Garner recombination of L residue matrices R[l] (m x nb, dense) into
 // C = X mod p, where X is the unique integer in [0, prod m_l) with X = R[l]
 // mod m_l: mixed-radix digits v_l in [0, m_l), X = v_0 + m_0 (v_1 + m_1 (v_2
@@ -875,7 +888,7 @@ __global__ void k_block_crt(const uint32_t *R, uint64_t m, uint64_t nb, uint32_t
                 if (j >= l) break;
                 const uint32_t vj = v[j] >= ml ? v[j] - ml : v[j];
                 t = t >= vj ? t - vj : t + ml - vj;     // (t - v_j) mod m_l
-                t = mod_small64((uint64_t)t * rc.inv[l][j], ml, rc.minv[l]);
+                t = reduce_small(t * rc.inv[l][j], ml, rc.magic[l]);   // both below 2^16
             }
             v[l] = t;
         }
@@ -1009,7 +1022,7 @@ bool block_rns_plan(uint32_t p, uint64_t k, RnsConst *rc)
         rc->mod[l] = l < L ? primes[l] : 1;
         for (int j = 0; j < RNS_MAX; ++j)
             rc->inv[l][j] = (l < L && j < l) ? pow_mod_small(primes[j], primes[l] - 2, primes[l]) : 0;
-        rc->minv[l] = UINT64_MAX / rc->mod[l];
+        rc->magic[l] = (uint32_t)((1ull << 32) / std::max<uint32_t>(rc->mod[l], 2));
     }
     rc->modp = make_mod(p);
     return true;
@@ -1171,6 +1184,10 @@ cudaError_t launch_block_tc(const uint32_t *mods, int n_mod, uint64_t m, uint64_
                 a.ldc = ldc;
                 a.Aimg = Aimg ? Aimg + (size_t)l * img_bytes : nullptr;
                 a.Bimg = sc.bimg + (uint64_t)(l - l0) * btiles * B_TILE_BYTES;
+                // residue passes over a uint32 A alternate direction: what a CTA
+                // read last is what L2 still holds, and every second pass
+                // begins there
+                a.backward = reduce && !Aimg ? (uint32_t)(l & 1) : 0;
                 e = cudaLaunchKernelEx(&cfg, kernel, a);
                 if (e != cudaSuccess) return e;
                 ++*launches;

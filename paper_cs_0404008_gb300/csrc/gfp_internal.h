@@ -138,7 +138,7 @@ struct RnsConst {
     uint32_t p;
     uint32_t mod[RNS_MAX];
     uint32_t inv[RNS_MAX][RNS_MAX];
-    uint64_t minv[RNS_MAX];   // floor((2^64 - 1) / mod[l]), for remainders by multiply-high
+    uint32_t magic[RNS_MAX];  // floor(2^32 / mod[l]), for remainders by multiply-high
     Mod modp;                 // Barrett constants of p
 };
 // Chooses the moduli for k-term sums of products of residues below p; false
@@ -218,13 +218,11 @@ struct gfp_ctx {
     uint32_t *stage_out = nullptr;
     size_t stage_out_elems = 0;
 
-    // block-product workspace (error flag, column-major partial sums), zero
-    // outside calls, B's digit tiles, and the residue matrices of the passes of
-    // a large modulus; all grown on demand
+    // block-product buffer: error flag and column-major partial sums at its
+    // start, zero outside calls; B's digit tiles and the residue matrices of the
+    // passes of a large modulus at its end; grown on demand
     void *blk_ws = nullptr;
-    size_t blk_ws_bytes = 0;
-    void *blk_bimg = nullptr, *blk_res = nullptr;
-    size_t blk_bimg_bytes = 0, blk_res_bytes = 0;
+    size_t blk_ws_bytes = 0, blk_zero = 0;   // size, length of the prefix known to be zero
 
     // tuned plan: (p, lg_n) -> entry
     std::map<std::pair<uint32_t, uint32_t>, gfp_plan_entry> plan;

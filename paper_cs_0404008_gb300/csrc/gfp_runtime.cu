@@ -457,8 +457,6 @@ GFP_API gfp_status gfp_context_destroy(gfp_ctx *ctx)
     if (ctx->stage) cudaFree(ctx->stage);
     if (ctx->stage_out) cudaFree(ctx->stage_out);
     if (ctx->blk_ws) cudaFree(ctx->blk_ws);
-    if (ctx->blk_bimg) cudaFree(ctx->blk_bimg);
-    if (ctx->blk_res) cudaFree(ctx->blk_res);
     delete ctx;
     return GFP_OK;
 }
@@ -772,35 +770,36 @@ static int block_sms(const gfp_ctx *ctx)
     return (ctx->blk_sms > 0 && ctx->blk_sms < ctx->sm_count) ? ctx->blk_sms : ctx->sm_count;
 }
 
-// Grows one buffer of the block product to `need` bytes; the old one may still
-// be read by work in flight.
-static gfp_status grow_block_buffer(void **buf, size_t *have, size_t need, bool zero)
+// Block-product buffer of the context for an m x k by k x nb product with n_mod
+// moduli, one allocation grown on demand: the workspace at its start, B's digit
+// tiles and (where there are several moduli) the residue matrices at its end.
+// Only [0, blk_zero) is known to be zero; the caller holds ctx->mu.
+static gfp_status ensure_block_ws(gfp_ctx *ctx, uint64_t m, uint64_t k, uint64_t nb, int n_mod, cudaStream_t s,
+                                  BlockScratch *sc, uint32_t **res)
 {
-    if (need <= *have) return GFP_OK;
-    GFP_CUDA_TRY(cudaDeviceSynchronize());
-    if (*buf) cudaFree(*buf);
-    *buf = nullptr;
-    *have = 0;
-    if (cudaMalloc(buf, need) != cudaSuccess) {
-        *buf = nullptr;
-        return GFP_ERR_NOMEM;
+    const size_t ws = align256(block_tc_workspace_bytes(m, nb)), img = align256(block_tc_bimg_bytes(k, nb, n_mod));
+    const size_t rb = n_mod > 1 ? align256((size_t)n_mod * m * nb * 4) : 0, need = ws + img + rb;
+    if (need > ctx->blk_ws_bytes) {
+        GFP_CUDA_TRY(cudaDeviceSynchronize());   // work in flight may still use the old one
+        if (ctx->blk_ws) cudaFree(ctx->blk_ws);
+        ctx->blk_ws = nullptr;
+        ctx->blk_ws_bytes = ctx->blk_zero = 0;
+        if (cudaMalloc(&ctx->blk_ws, need) != cudaSuccess) {
+            ctx->blk_ws = nullptr;
+            return GFP_ERR_NOMEM;
+        }
+        ctx->blk_ws_bytes = need;
     }
-    if (zero) GFP_CUDA_TRY(cudaMemset(*buf, 0, need));
-    *have = need;
+    uint8_t *base = (uint8_t *)ctx->blk_ws, *tail = base + (ctx->blk_ws_bytes - img - rb) / 256 * 256;
+    if (ws > ctx->blk_zero) {
+        GFP_CUDA_TRY(cudaMemsetAsync(base + ctx->blk_zero, 0, ws - ctx->blk_zero, s));
+        ctx->blk_zero = ws;
+    }
+    ctx->blk_zero = std::min<size_t>(ctx->blk_zero, (size_t)(tail - base));   // the rest is written below
+    sc->ws = base;
+    sc->bimg = tail;
+    *res = (uint32_t *)(tail + img);
     return GFP_OK;
-}
-
-// Block-product buffers of the context for an m x k by k x nb product with
-// n_mod moduli (the residue matrices of the passes where there are several);
-// the caller holds ctx->mu.
-static gfp_status ensure_block_ws(gfp_ctx *ctx, uint64_t m, uint64_t k, uint64_t nb, int n_mod)
-{
-    gfp_status st = grow_block_buffer(&ctx->blk_ws, &ctx->blk_ws_bytes, block_tc_workspace_bytes(m, nb), true);
-    if (st == GFP_OK)
-        st = grow_block_buffer(&ctx->blk_bimg, &ctx->blk_bimg_bytes, block_tc_bimg_bytes(k, nb, n_mod), false);
-    if (st == GFP_OK && n_mod > 1)
-        st = grow_block_buffer(&ctx->blk_res, &ctx->blk_res_bytes, (size_t)n_mod * m * nb * 4, false);
-    return st;
 }
 
 // The tensor-core product through the context's buffers: one modulus directly,
@@ -811,10 +810,10 @@ static gfp_status run_block_tc(gfp_ctx *ctx, uint32_t p, const RnsConst *rc, uin
 {
     std::lock_guard<std::mutex> g(ctx->mu);
     const int n_mod = rc ? rc->L : 1;
-    const gfp_status st = ensure_block_ws(ctx, m, k, nb, n_mod);
+    BlockScratch sc;
+    uint32_t *R;
+    const gfp_status st = ensure_block_ws(ctx, m, k, nb, n_mod, s, &sc, &R);
     if (st != GFP_OK) return st;
-    const BlockScratch sc{ctx->blk_ws, (uint8_t *)ctx->blk_bimg};
-    uint32_t *R = (uint32_t *)ctx->blk_res;
     int launches = 0;
     GFP_CUDA_TRY(launch_block_tc(rc ? rc->mod : &p, n_mod, m, k, nb, A, lda, B, ldb, n_mod > 1 ? R : C,
                                  n_mod > 1 ? nb : ldc, sc, block_sms(ctx), s, &launches, Aimg, img_bytes));
@@ -849,11 +848,16 @@ GFP_API gfp_status gfp_matmul_block(gfp_ctx *ctx, uint32_t p, uint64_t m, uint64
     const bool direct_ok = layout_ok && p <= BLOCK_TC_MAX_P;
     bool rns_ok = layout_ok && p > BLOCK_TC_MAX_P && block_rns_plan(p, k, &rc);
     if (rns_ok && ctx->forced == GFP_REPR_AUTO) {
-        // the residue passes each stream A once (about 4 TB/s) after two
-        // launches; the CUDA-core kernel pays per multiply-add (about 4.5e12/s
-        // at best): keep the residues only where they are expected to win
-        const double t_rns = rc.L * (25e-6 + 4.0 * (double)m * (double)k / 4.0e12);
-        const double t_cc = (double)m * (double)k * (double)nb / 4.5e12;
+        // A residue pass costs about 10 us before its traffic (its own launch, its
+        // finishing launch, a partly filled wave), then A once at about 4.5 TB/s
+        // and its result three times.  A CTA of the CUDA-core kernel takes 0.134 us
+        // per term for its 64 x 64 outputs, an SM as long for each CTA it holds.
+        // Measured (us, residues / CUDA cores): 256 x 256 x 64 over GF(2^26 - 5)
+        // 45 / 42, 512 x 512 x 64 45 / 76, 1024 x 1024 x 64 45 / 144,
+        // 256 x 16384 x 64 71 / 2172, 16384 x 256 x 64 70 / 66, 4096 x 64 x 64 46 / 17
+        const double ctas = (double)((m + 63) / 64) * (double)((nb + 63) / 64);
+        const double t_rns = 5e-6 + rc.L * (10e-6 + (4.0 * (double)m * (double)k + 16.0 * (double)m * (double)nb) / 4.5e12);
+        const double t_cc = 7e-6 + (double)k * 0.134e-6 * std::max(1.0, ctas / ctx->sm_count);
         if (t_cc <= t_rns) rns_ok = false;
     }
     const bool tc_ok = direct_ok || rns_ok;
@@ -1028,6 +1032,7 @@ GFP_API gfp_status gfp_context_check(gfp_ctx *ctx)
     GFP_CUDA_TRY(cudaMemcpy(&h, ctx->blk_ws, 4, cudaMemcpyDeviceToHost));   // the error flag
     if (h) {
         GFP_CUDA_TRY(cudaMemset(ctx->blk_ws, 0, ctx->blk_ws_bytes));
+        ctx->blk_zero = ctx->blk_ws_bytes;
         return GFP_ERR_TIMEOUT;
     }
     return dbits ? GFP_ERR_INVALID : GFP_OK;

@@ -71,6 +71,13 @@ __device__ __forceinline__ void ld_stream4(uint4 &v, const void *p)
                  : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                  : "l"(p));
 }
+// the same without marking the lines for early eviction
+__device__ __forceinline__ void ld_l2_4(uint4 &v, const void *p)
+{
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(p));
+}
 // loads only where `on` holds; v keeps its value elsewhere
 __device__ __forceinline__ void ld_if(uint32_t &v, const uint32_t *p, bool on)
 {
