@@ -87,7 +87,7 @@ bool repr_eligible(Repr r, uint32_t p);
 
 // Launch configuration constants of the dot kernels.
 constexpr int DOT_THREADS = 256;
-constexpr int MV_THREADS = 1024;
+constexpr int MV_THREADS = 512;
 
 // Device scratch of one batched execution.
 struct BatchScratch {

@@ -5,14 +5,32 @@
 // Inside a CTA the warps form G groups of W warps: a group works on one row at
 // a time and warp s of the group streams column segment s of that row with
 // 128-bit loads, accumulating unreduced (Section 3 of the paper) and leaving
-// one residue per (row, segment) in shared memory.  After a batch of RB rows
+// one residue per (row, segment) in shared memory.  After a window of rows
 // the CTA sums the W segment residues of each row and writes y.  No atomics,
 // no per-row barrier; A is read exactly once.
+//
+// HBM bound, so what counts is that loads stay in flight.  A warp keeps two
+// batches of U vectors a lane: while it adds one up (and reduces at the end of a
+// row) the next, of the same row or of its next one, is already loading.  A
+// ragged end is part of a batch, not a loop of its own.  64 iterations of
+// 32768^2 over GF(2^31 - 1): 39.1 -> 37.7 ms (7.29 TB/s) against one batch of
+// four vectors in flight in 32 warps; 9001 x 7003 with packed, odd rows: 54.9 ->
+// 41.6 us (6.1 TB/s).  Batches of four or six vectors were slower (70 and 66
+// against 52 us for the latter with a flushed L2): more batches a row.
+//
+// Rows need not be 16-byte aligned.  A row that starts r words past a 16-byte
+// boundary is read as the aligned vectors inside it; x is then kept in shared
+// memory as four planes of every fourth element, so that the four elements a
+// vector multiplies are one conflict-free read each (from a plain x the lanes'
+// words would lie four apart, a four-way bank conflict).  The fewer than four
+// elements before the first and after the last vector are added by themselves.
+#include <algorithm>
+
 #include "gfp_internal.h"
 
 namespace gfp {
 
-constexpr int MV_RB = 64;   // rows per batch (multiple of every group count G)
+constexpr int MV_U = 8;     // vectors a lane loads at a time, two batches in flight
 constexpr int MV_PREFETCH_ROWS = 4;   // rows of A requested into L2 before the dependency wait
 
 // Sum of one uint64 per thread over the CTA, valid in thread 0.
@@ -44,10 +62,24 @@ struct MvProj {
     uint32_t *sout;
 };
 
-template <class Acc, bool XS, int U>
+// Where x is read from: global memory (16-byte aligned, or 4-byte reads),
+// shared memory as it is, or shared memory in four planes for rows of any
+// alignment.
+enum XMode : int { X_GLOBAL = 0, X_SMEM = 1, X_PLANES = 2 };
+
+// One warp's part [c0, c1) of a row; columns are counted from c0.
+struct RowPart {
+    const uint4 *av;   // first 16-byte vector inside it, this lane's
+    uint32_t nv;       // vectors
+    uint32_t head;     // column of the first one
+    uint32_t ecol;     // column of the lane's element outside the vectors, or ~0
+    uint32_t eval;     // that element
+};
+
+template <class Acc, int XM, int U>
 __global__ void __launch_bounds__(MV_THREADS, 1)
     k_matvec(Mod m, uint64_t k, uint64_t rows, uint64_t cols, const uint32_t *__restrict__ A,
-             uint64_t lda, const uint32_t *__restrict__ x, uint32_t *__restrict__ y, int W,
+             uint64_t lda, const uint32_t *__restrict__ x, uint32_t *__restrict__ y, int W, uint32_t window,
              MvProj proj)
 {
     extern __shared__ __align__(16) uint32_t smem[];
@@ -58,74 +90,148 @@ __global__ void __launch_bounds__(MV_THREADS, 1)
     // CTA asks L2 for the first rows it will stream; everything that reads
     // x or writes y comes after the wait.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const uint64_t r_begin = rows * blockIdx.x / gridDim.x;
+    const uint64_t r_end = rows * (blockIdx.x + 1) / gridDim.x;
     {
-        const uint64_t r0 = rows * blockIdx.x / gridDim.x, r1 = rows * (blockIdx.x + 1) / gridDim.x;
         const uint64_t row_bytes = cols * 4;
-        if (threadIdx.x < MV_PREFETCH_ROWS && r0 + threadIdx.x < r1 &&
+        if (threadIdx.x < MV_PREFETCH_ROWS && r_begin + threadIdx.x < r_end &&
             ((((uintptr_t)A) | (lda * 4) | row_bytes) & 15u) == 0 && row_bytes <= 0xFFFFFFF0ull)
-            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(A + (r0 + threadIdx.x) * lda),
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(A + (r_begin + threadIdx.x) * lda),
                          "r"((uint32_t)row_bytes)
                          : "memory");
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     uint32_t *xs = smem;
-    uint32_t *part = smem + (XS ? colsp : 0);
-    const int nw = blockDim.x >> 5, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t plane = (uint32_t)(colsp >> 2);   // words of a plane of x
+    uint32_t *part = smem + (XM != X_GLOBAL ? colsp : 0);
+    const int nw = MV_THREADS / 32, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int G = nw / W, g = w / W, sgm = w % W;
-
-    if (XS) {
-        for (uint64_t j = threadIdx.x; j < colsp; j += blockDim.x) xs[j] = (j < cols) ? x[j] : 0u;
-        __syncthreads();
-    }
-    const uint32_t *xsrc = XS ? xs : x;
-    const bool vec = ((((uintptr_t)A) & 15u) == 0) && (lda % 4 == 0) &&
-                     (XS || ((((uintptr_t)x) & 15u) == 0));
 
     // column segment of this warp: [c0, c1), c0 a multiple of 4
     const uint64_t seg = ((cols + W - 1) / W + 3) & ~3ull;
-    const uint64_t c0 = (uint64_t)sgm * seg;
-    const uint64_t c1 = (c0 + seg < cols) ? c0 + seg : cols;
+    const uint64_t c0 = min((uint64_t)sgm * seg, cols);
+    const uint64_t c1 = min(c0 + seg, cols);
+    // batches that cover any row's part (at least one: it carries the elements outside the vectors)
+    const uint32_t nq = max(1u, (uint32_t)((((c1 - c0) >> 2) + U * 32 - 1) / (U * 32)));
+    // rows that 16-byte loads take as they are (X_GLOBAL: else the plain loop below)
+    const bool vec = XM != X_GLOBAL ||
+                     ((((uintptr_t)A) | (uintptr_t)(lda * 4) | ((uintptr_t)x)) & 15u) == 0;
 
-    const uint64_t r_begin = rows * blockIdx.x / gridDim.x;
-    const uint64_t r_end = rows * (blockIdx.x + 1) / gridDim.x;
-    uint64_t pacc = 0;   // projection partial (sum of residues)
-
-    for (uint64_t rb = r_begin; rb < r_end; rb += MV_RB) {
-        const uint64_t rcount = (r_end - rb < (uint64_t)MV_RB) ? r_end - rb : (uint64_t)MV_RB;
-        for (uint64_t i = g; i < rcount; i += G) {
-            const uint32_t *Ar = A + (rb + i) * lda;
-            Acc acc;
-            acc.init(m, k);
-            if (c0 < c1) {
-                if (vec) {
-                    const uint4 *av = reinterpret_cast<const uint4 *>(Ar + c0);
-                    const uint4 *xv = reinterpret_cast<const uint4 *>(xsrc + c0);
-                    const uint64_t nv = (c1 - c0) >> 2;
-                    uint64_t v = lane;
-                    for (; v + (U - 1) * 32 < nv; v += U * 32) {
-                        uint4 a[U];
+    const uint32_t cs = XM != X_GLOBAL ? (uint32_t)c0 : 0u;   // c0, where x is in shared memory
+    const auto xat = [&](uint32_t j) -> uint32_t {
+        if constexpr (XM == X_PLANES) return xs[(j & 3) * plane + ((cs + j) >> 2)];   // c0 is a multiple of 4
+        else if constexpr (XM == X_SMEM) return xs[cs + j];
+        else return __ldg(x + c0 + j);
+    };
+    const auto locate = [&](uint64_t row, RowPart &p) {
+        const uint32_t *Ar = A + row * lda + c0;
+        const uint32_t len = (uint32_t)(c1 - c0);
+        uint32_t head = 0;   // words before the first boundary
+        if constexpr (XM == X_PLANES) head = min((uint32_t)(-(int)((uintptr_t)Ar >> 2) & 3), len);
+        p.nv = (len - head) >> 2;
+        p.head = head;
+        p.av = reinterpret_cast<const uint4 *>(Ar + head) + lane;
+        const uint32_t after = head + (p.nv << 2);   // first element past the vectors
+        const uint32_t e = (uint32_t)lane < head ? (uint32_t)lane : after + (uint32_t)lane - 4u;
+        const bool has = (uint32_t)lane < head || (lane >= 4 && e < len);
+        p.ecol = has ? e : ~0u;
+        p.eval = has ? __ldcs(Ar + e) : 0u;
+    };
+    const auto load = [&](const RowPart &p, uint32_t q, uint4 (&buf)[U]) {
 #pragma unroll
-                        for (int u = 0; u < U; ++u) a[u] = __ldcs(av + v + u * 32);
+        for (int u = 0; u < U; ++u) {
+            const uint32_t v = q * (U * 32) + u * 32;
+            if (v + lane < p.nv) buf[u] = __ldcs(p.av + v);
+        }
+    };
+    Acc acc;
+    acc.init(m, k);
+    const auto consume = [&](const RowPart &p, uint32_t q, const uint4 (&buf)[U]) {
 #pragma unroll
-                        for (int u = 0; u < U; ++u)
-                            acc.add4(a[u], XS ? xv[v + u * 32] : __ldg(xv + v + u * 32), m);
-                    }
-                    for (; v < nv; v += 32)
-                        acc.add4(__ldcs(av + v), XS ? xv[v] : __ldg(xv + v), m);
-                    const uint64_t j = c0 + (nv << 2) + lane;
-                    if (j < c1) acc.add(__ldcs(Ar + j), XS ? xsrc[j] : __ldg(xsrc + j), m);
+        for (int u = 0; u < U; ++u) {
+            const uint32_t v = q * (U * 32) + u * 32 + lane;
+            if (v < p.nv) {
+                uint4 xv;
+                if constexpr (XM == X_PLANES) {
+                    const uint32_t j = p.head, i = (cs >> 2) + v;   // element e: plane (j + e) mod 4
+                    const uint32_t i1 = i + (j > 2), i2 = i + (j > 1), i3 = i + (j > 0);
+                    xv = make_uint4(xs[j * plane + i], xs[((j + 1) & 3) * plane + i1],
+                                    xs[((j + 2) & 3) * plane + i2], xs[((j + 3) & 3) * plane + i3]);
+                } else if constexpr (XM == X_SMEM) {
+                    xv = reinterpret_cast<const uint4 *>(xs + cs)[v];
                 } else {
-                    for (uint64_t j = c0 + lane; j < c1; j += 32)
-                        acc.add(__ldcs(Ar + j), XS ? xsrc[j] : __ldg(xsrc + j), m);
+                    xv = __ldg(reinterpret_cast<const uint4 *>(x + c0) + v);
                 }
+                acc.add4(buf[u], xv, m);
             }
+        }
+    };
+
+    uint64_t pacc = 0;   // projection partial (sum of residues)
+    bool staged = XM == X_GLOBAL;
+    for (uint64_t rb = r_begin; rb < r_end; rb += window) {
+        const uint32_t rcount = (uint32_t)min(r_end - rb, (uint64_t)window);
+        const auto finish = [&](uint32_t i) {
             uint64_t s = acc.residue(m);
 #pragma unroll
             for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
             if (lane == 0) part[i * W + sgm] = reduce64(s, m);
+            acc.init(m, k);
+        };
+        if (vec) {
+            uint4 b0[U], b1[U];
+            RowPart cur, nxt;
+            uint32_t i = g, q = 0;
+            if (i < rcount) {
+                locate(rb + i, cur);
+                load(cur, 0, b0);
+            }
+            if (!staged) {   // the first loads are under way
+                for (uint64_t j = threadIdx.x; j < colsp; j += MV_THREADS)
+                    xs[XM == X_PLANES ? (j & 3) * plane + (j >> 2) : j] = (j < cols) ? x[j] : 0u;
+                __syncthreads();
+                staged = true;
+            }
+            // one batch: start the next, add this one up, end the row
+            const auto step = [&](uint4 (&bc)[U], uint4 (&bn)[U]) {
+                uint32_t ni = i, n = q + 1;
+                nxt = cur;
+                if (n == nq) {
+                    n = 0;
+                    ni += G;
+                    if (ni < rcount) locate(rb + ni, nxt);
+                }
+                if (ni < rcount) load(nxt, n, bn);
+                consume(cur, q, bc);
+                if (n == 0) {
+                    if (cur.ecol != ~0u) acc.add(cur.eval, xat(cur.ecol), m);
+                    finish(i);
+                }
+                cur = nxt;
+                i = ni;
+                q = n;
+            };
+            while (i < rcount) {
+                step(b0, b1);
+                if (i < rcount) step(b1, b0);
+            }
+        } else {
+            for (uint32_t i = g; i < rcount; i += G) {
+                const uint32_t *Ar = A + (rb + i) * lda;
+                constexpr int S = 8;
+                for (uint64_t j = c0 + lane; j < c1; j += 32 * S) {
+                    uint32_t v[S];
+#pragma unroll
+                    for (int u = 0; u < S; ++u) v[u] = j + u * 32 < c1 ? __ldcs(Ar + j + u * 32) : 0u;
+#pragma unroll
+                    for (int u = 0; u < S; ++u)
+                        if (j + u * 32 < c1) acc.add(v[u], __ldg(x + j + u * 32), m);
+                }
+                finish(i);
+            }
         }
         __syncthreads();
-        for (uint64_t i = threadIdx.x; i < rcount; i += blockDim.x) {
+        for (uint32_t i = threadIdx.x; i < rcount; i += MV_THREADS) {
             uint64_t s = 0;
             for (int q = 0; q < W; ++q) s += part[i * W + q];
             const uint32_t yi = reduce64(s, m);
@@ -149,32 +255,35 @@ __global__ void __launch_bounds__(MV_THREADS, 1)
     }
 }
 
-// Shared memory above which x is read through the L1/L2 path instead.
-constexpr size_t MV_XS_MAX = 200 * 1024;
+// Shared memory above which x is read through the L1/L2 path instead, and the
+// part kept for the segment residues of a window of rows.
+constexpr size_t MV_XS_MAX = 200 * 1024, MV_PART_MAX = 16 * 1024;
 
-template <class Acc, bool XS>
+template <class Acc, int XM>
 static cudaError_t mv_launch(const Mod &m, uint64_t k, uint64_t rows, uint64_t cols,
                              const uint32_t *A, uint64_t lda, const uint32_t *x, uint32_t *y,
                              int sm_count, cudaStream_t s, const MvProj &proj)
 {
-    constexpr int U = 4;
+    constexpr int U = MV_U;
     const int nw = MV_THREADS / 32;
-    // warps per row: enough that each warp streams >= U*32 vectors, at most nw
-    uint64_t nv = cols / 4;
+    const uint64_t grid = std::min<uint64_t>((uint64_t)sm_count, rows ? rows : 1);
+    const uint64_t per_cta = (rows + grid - 1) / grid;
+    // warps per row: as few as take a row in one batch of U vectors a lane (more
+    // warps would reduce more often for the same bytes), and more where a CTA's
+    // rows would leave half of its warps without one
+    const uint64_t nv = cols / 4;
     int W = 1;
-    while (W < nw && nv / (uint64_t)(2 * W) >= (uint64_t)U * 32) W *= 2;
+    while (W < nw && (nv > (uint64_t)W * U * 32 || (uint64_t)(nw / W) >= 2 * per_cta)) W *= 2;
     const size_t colsp = (cols + 3) & ~3ull;
-    const size_t smem = (XS ? colsp * 4 : 0) + (size_t)MV_RB * W * 4;
+    const uint32_t window = (uint32_t)std::min<uint64_t>(per_cta, MV_PART_MAX / (4 * W));
+    const size_t smem = (XM != X_GLOBAL ? colsp * 4 : 0) + (size_t)window * W * 4;
     static bool attr_set = false;
     if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_matvec<Acc, XS, U>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)(MV_XS_MAX + MV_RB * nw * 4));
+        cudaError_t e = cudaFuncSetAttribute(k_matvec<Acc, XM, U>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)(MV_XS_MAX + MV_PART_MAX));
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
-    uint64_t grid = (uint64_t)sm_count;
-    if (grid > rows) grid = rows ? rows : 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(MV_THREADS);
@@ -185,8 +294,8 @@ static cudaError_t mv_launch(const Mod &m, uint64_t k, uint64_t rows, uint64_t c
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_matvec<Acc, XS, U>, m, k, rows, cols, A, lda, x,
-                                             y, W, proj);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_matvec<Acc, XM, U>, m, k, rows, cols, A, lda, x,
+                                             y, W, window, proj);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -195,9 +304,12 @@ static cudaError_t mv_dispatch(const Mod &m, uint64_t k, uint64_t rows, uint64_t
                                const uint32_t *A, uint64_t lda, const uint32_t *x, uint32_t *y,
                                int sm_count, cudaStream_t s, const MvProj &proj)
 {
-    if (((cols + 3) & ~3ull) * 4 <= MV_XS_MAX)
-        return mv_launch<Acc, true>(m, k, rows, cols, A, lda, x, y, sm_count, s, proj);
-    return mv_launch<Acc, false>(m, k, rows, cols, A, lda, x, y, sm_count, s, proj);
+    if (((cols + 3) & ~3ull) * 4 > MV_XS_MAX)
+        return mv_launch<Acc, X_GLOBAL>(m, k, rows, cols, A, lda, x, y, sm_count, s, proj);
+    // rows that 16-byte loads take as they are, or not
+    if ((((uintptr_t)A) & 15u) == 0 && lda % 4 == 0)
+        return mv_launch<Acc, X_SMEM>(m, k, rows, cols, A, lda, x, y, sm_count, s, proj);
+    return mv_launch<Acc, X_PLANES>(m, k, rows, cols, A, lda, x, y, sm_count, s, proj);
 }
 
 cudaError_t launch_matvec(Repr r, const Mod &m, uint64_t k, uint64_t rows, uint64_t cols,
