@@ -196,6 +196,19 @@ def _check(st: int, where: str):
         raise GfpError(st, where)
 
 
+_torch = None      # set by the first call that needs it (the host-only functions work without torch)
+_stream_ready = False
+_U32 = _U16 = ()   # the tensor types taken as uint32, as uint16 codes
+
+
+def _import_torch():
+    global _torch, _U32, _U16
+    import torch
+    _U32, _U16 = (torch.int32, torch.uint32), (torch.int16, torch.uint16)
+    _torch = torch
+    return torch
+
+
 def _ptr(t) -> int:
     """Device (or host) address of a tensor / numpy array / int."""
     if t is None:
@@ -210,19 +223,28 @@ def _ptr(t) -> int:
 
 
 def _stream(stream) -> int:
+    """The raw handle of `stream`, of the current device's current stream when
+    none is given (asked for as a handle: a torch.cuda.Stream object built on
+    every call cost more than the launch of a small product)."""
+    global _stream_ready
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        if not _stream_ready:   # the first time through torch's own call, which initialises CUDA
+            s = (_torch or _import_torch()).cuda.current_stream().cuda_stream
+            _stream_ready = True
+            return s
+        c = _torch._C
+        return c._cuda_getCurrentRawStream(c._cuda_getDevice())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
 
 
-def _check_u32(t, n: int, name: str):
-    import torch
+def _addr32(t, n: int, name: str) -> int:
+    """Address of a contiguous CUDA tensor of at least n 32-bit elements."""
+    torch = _torch or _import_torch()
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name} must be a torch tensor")
-    if t.dtype not in (torch.uint32, torch.int32):
+    if t.dtype not in _U32:
         raise TypeError(f"{name} must be uint32 (or int32 bit-identical), got {t.dtype}")
     if not t.is_cuda:
         raise ValueError(f"{name} must be on a CUDA device")
@@ -230,6 +252,7 @@ def _check_u32(t, n: int, name: str):
         raise ValueError(f"{name} must be contiguous")
     if t.numel() < n:
         raise ValueError(f"{name} has {t.numel()} elements, needs {n}")
+    return t.data_ptr()
 
 
 # ---- host-only functions ----
@@ -319,11 +342,10 @@ def gfp_launch_count(ctx: Context) -> int:
 def gfp_dot(ctx: Context, p: int, x, y, out, stream=None, n: int | None = None):
     """out[0] = dot(x[:n], y[:n]) mod p (device tensors)."""
     n = x.numel() if n is None else n
-    _check_u32(x, n, "x")
-    _check_u32(y, n, "y")
-    _check_u32(out, 1, "out")
-    _check(load().gfp_dot(ctx.handle, p, n, _ptr(x), _ptr(y), _ptr(out), _stream(stream)),
-           "gfp_dot")
+    ax, ay, ao = _addr32(x, n, "x"), _addr32(y, n, "y"), _addr32(out, 1, "out")
+    st = (_lib or load()).gfp_dot(ctx.handle, p, n, ax, ay, ao, _stream(stream))
+    if st:
+        _check(st, "gfp_dot")
     return out
 
 
@@ -346,7 +368,7 @@ def _descs(pairs):
 def gfp_dot_batched(ctx: Context, pairs, out, stream=None):
     arr, count = _descs(pairs)
     if count:
-        _check_u32(out, count, "out")
+        _addr32(out, count, "out")
     _check(load().gfp_dot_batched(ctx.handle, arr, count, _ptr(out), _stream(stream)),
            "gfp_dot_batched")
     return out
@@ -357,7 +379,7 @@ def gfp_dot_batched_noalloc(pairs, out, stream=None):
     (no allocation anywhere; at most 1024 pairs, see the header)."""
     arr, count = _descs(pairs)
     if count:
-        _check_u32(out, count, "out")
+        _addr32(out, count, "out")
     _check(load().gfp_dot_batched_noalloc(arr, count, _ptr(out), _stream(stream)),
            "gfp_dot_batched_noalloc")
     return out
@@ -376,9 +398,9 @@ class BatchPlan:
         self._keep = pairs  # keep operand tensors alive with the plan
 
     def exec(self, out, stream=None):
-        _check_u32(out, self.count, "out")
-        _check(load().gfp_batch_plan_exec(self.handle, _ptr(out), _stream(stream)),
-               "gfp_batch_plan_exec")
+        st = (_lib or load()).gfp_batch_plan_exec(self.handle, _addr32(out, self.count, "out"), _stream(stream))
+        if st:
+            _check(st, "gfp_batch_plan_exec")
         return out
 
     def info(self):
@@ -432,10 +454,10 @@ def gfp_matvec(ctx: Context, p: int, A, x, y, stream=None, lda: int | None = Non
     rows = A.shape[0] if rows is None else rows
     cols = A.shape[1] if cols is None else cols
     lda = A.stride(0) if lda is None else lda
-    _check_u32(x, cols, "x")
-    _check_u32(y, rows, "y")
-    _check(load().gfp_matvec(ctx.handle, p, rows, cols, _ptr(A), lda, _ptr(x), _ptr(y),
-                             _stream(stream)), "gfp_matvec")
+    ax, ay = _addr32(x, cols, "x"), _addr32(y, rows, "y")
+    st = (_lib or load()).gfp_matvec(ctx.handle, p, rows, cols, _ptr(A), lda, ax, ay, _stream(stream))
+    if st:
+        _check(st, "gfp_matvec")
     return y
 
 
@@ -443,8 +465,8 @@ def gfp_matvec_iterate(ctx: Context, p: int, A, x0, Y, iters: int, stream=None,
                        lda: int | None = None):
     n = A.shape[0]
     lda = A.stride(0) if lda is None else lda
-    _check_u32(x0, n, "x0")
-    _check_u32(Y, n * iters, "Y")
+    _addr32(x0, n, "x0")
+    _addr32(Y, n * iters, "Y")
     _check(load().gfp_matvec_iterate(ctx.handle, p, n, _ptr(A), lda, _ptr(x0), _ptr(Y), iters,
                                      _stream(stream)), "gfp_matvec_iterate")
     return Y
@@ -455,11 +477,11 @@ def gfp_matvec_sequence(ctx: Context, p: int, A, x0, u, seq, iters: int, Y=None,
     """seq[t] = u^T A^t x0 mod p, t = 0..iters (device tensors)."""
     n = A.shape[0]
     lda = A.stride(0) if lda is None else lda
-    _check_u32(x0, n, "x0")
-    _check_u32(u, n, "u")
-    _check_u32(seq, iters + 1, "seq")
+    _addr32(x0, n, "x0")
+    _addr32(u, n, "u")
+    _addr32(seq, iters + 1, "seq")
     if Y is not None:
-        _check_u32(Y, n * iters, "Y")
+        _addr32(Y, n * iters, "Y")
     _check(load().gfp_matvec_sequence(ctx.handle, p, n, _ptr(A), lda, _ptr(x0), _ptr(u), iters,
                                       _ptr(seq), _ptr(Y), _stream(stream)), "gfp_matvec_sequence")
     return seq
@@ -590,7 +612,7 @@ def gfp_plan_size(ctx: Context) -> int:
 def gfp_fill_uniform(p: int, seed: int, stream_id: int, out, n: int | None = None,
                      offset: int = 0, stream=None):
     n = out.numel() if n is None else n
-    _check_u32(out, n, "out")
+    _addr32(out, n, "out")
     _check(load().gfp_fill_uniform(p, seed, stream_id, offset, n, _ptr(out), _stream(stream)),
            "gfp_fill_uniform")
     return out
@@ -605,14 +627,16 @@ def gfp_gfq_find_primitive(p: int, k: int):
     return f
 
 
-def _check_u16(t, n: int, name: str):
-    import torch
+def _addr16(t, n: int, name: str) -> int:
+    """Address of a contiguous CUDA tensor of at least n 16-bit codes."""
+    torch = _torch or _import_torch()
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name} must be a torch tensor")
-    if t.dtype not in (torch.uint16, torch.int16):
+    if t.dtype not in _U16:
         raise TypeError(f"{name} must be uint16 (or int16 bit-identical), got {t.dtype}")
     if not t.is_cuda or not t.is_contiguous() or t.numel() < n:
         raise ValueError(f"{name} must be a contiguous CUDA tensor of >= {n} elements")
+    return t.data_ptr()
 
 
 class Field:
@@ -649,27 +673,26 @@ class Field:
 
     def to_log(self, values, codes, n: int | None = None, stream=None):
         n = values.numel() if n is None else n
-        _check_u32(values, n, "values")
-        _check_u16(codes, n, "codes")
+        _addr32(values, n, "values")
+        _addr16(codes, n, "codes")
         _check(load().gfp_gfq_to_log(self.handle, n, _ptr(values), _ptr(codes), _stream(stream)),
                "gfp_gfq_to_log")
         return codes
 
     def from_log(self, codes, values, n: int | None = None, stream=None):
         n = codes.numel() if n is None else n
-        _check_u16(codes, n, "codes")
-        _check_u32(values, n, "values")
+        _addr16(codes, n, "codes")
+        _addr32(values, n, "values")
         _check(load().gfp_gfq_from_log(self.handle, n, _ptr(codes), _ptr(values), _stream(stream)),
                "gfp_gfq_from_log")
         return values
 
     def dot(self, x, y, out, n: int | None = None, stream=None):
         n = x.numel() if n is None else n
-        _check_u16(x, n, "x")
-        _check_u16(y, n, "y")
-        _check_u16(out, 1, "out")
-        _check(load().gfp_gfq_dot(self.handle, n, _ptr(x), _ptr(y), _ptr(out), _stream(stream)),
-               "gfp_gfq_dot")
+        ax, ay, ao = _addr16(x, n, "x"), _addr16(y, n, "y"), _addr16(out, 1, "out")
+        st = (_lib or load()).gfp_gfq_dot(self.handle, n, ax, ay, ao, _stream(stream))
+        if st:
+            _check(st, "gfp_gfq_dot")
         return out
 
     def check(self) -> int:
