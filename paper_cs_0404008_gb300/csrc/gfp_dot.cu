@@ -6,10 +6,12 @@
 // residues, a per-thread unreduced accumulator (Section 3 of the paper),
 // one reduction per thread, a warp-shuffle plus shared-memory combine of the
 // thread residues, one 64-bit atomic add per CTA into the output's slot, and a
-// single final reduction by the last CTA to finish (found by a ticket counter
-// in the batched kernel, by a CTA count packed into the slot itself in the
-// single-dot kernel).  The last CTA returns slots and tickets to zero, so the
-// scratch is reusable by the next launch without a memset.
+// single final reduction by the last CTA to finish (found by a CTA count packed
+// into the slot itself, or by a ticket counter above 65535 units of one pair).
+// The last CTA returns slots and tickets to zero, so the scratch is reusable by
+// the next launch without a memset.
+#include <algorithm>
+
 #include "gfp_internal.h"
 
 namespace gfp {
@@ -56,7 +58,18 @@ __device__ __forceinline__ void accumulate_range(Acc &acc, const Mod &m, const u
 #pragma unroll
             for (int u = 0; u < U; ++u) acc.add4(a[u], c[u], m);
         }
-        for (; v < nv; v += T) acc.add4(ld_stream4(xv + v), ld_stream4(yv + v), m);
+        // at most U - 1 vectors left: one batch, so one memory latency
+        if (v < nv) {
+            uint4 a[U - 1], c[U - 1];
+#pragma unroll
+            for (int u = 0; u < U - 1; ++u) {
+                const bool in = v + u * T < nv;
+                a[u] = in ? ld_stream4(xv + v + u * T) : make_uint4(0u, 0u, 0u, 0u);
+                c[u] = in ? ld_stream4(yv + v + u * T) : make_uint4(0u, 0u, 0u, 0u);
+            }
+#pragma unroll
+            for (int u = 0; u < U - 1; ++u) acc.add4(a[u], c[u], m);
+        }
         const uint64_t i = b + (nv << 2) + t;   // fewer than 4 tail elements, T >= 4
         if (i < e) acc.add(ld_stream1(x + i), ld_stream1(y + i), m);
     } else {
@@ -113,7 +126,7 @@ __device__ __forceinline__ void combine_and_finish(uint64_t cta_total, const Mod
     }
 }
 
-// Single-dot combine in one atomic: each CTA adds its residue (below 2^32)
+// Combine in one atomic: each CTA adds its residue (below 2^32)
 // plus 2^48 to a 64-bit slot, so the low 48 bits collect the residue sum and
 // the high 16 bits count the CTAs (a grid of at most 2^16 - 1 CTAs keeps the
 // sum below 2^48).  The CTA whose add returns a count of grid - 1 holds every
@@ -159,20 +172,32 @@ __device__ __forceinline__ uint32_t unit_residue(const DevPair &pr, const DevUni
     return acc.residue(pr.m);
 }
 
-// Persistent batched kernel: CTAs pull work units from a global counter until
-// the list is exhausted; the representation is chosen per pair.  The last CTA
-// to leave returns both counters to zero.
-__global__ void __launch_bounds__(DOT_THREADS)
+// Persistent batched kernel; the representation is chosen per pair.  A CTA's
+// first unit is the one of its index (the grid is no larger than the list), the
+// others it pulls from a global counter, asking for the next one before it
+// streams the current one; the last CTA to leave returns both counters to zero.
+// A pair of one unit is written at once; the units of another meet in one
+// 64-bit atomic each (combine_packed), or, above the 65535 that its count holds,
+// through a slot and a ticket.  For a list of short pairs these round trips are
+// the time: 64 pairs of 2^6 to 2^13 terms 7.8 -> 2.9 us a launch, 1024 of 2^8 to
+// 2^14 14.5 -> 8.0 us against a counter for every unit, a slot, a fence and a
+// ticket for every pair and no early launch; 4096 pairs of 2^8 to 2^20 terms 606
+// -> 575 us (7.4 TB/s).  Three CTAs per SM: with four (64 registers) the long list
+// took 572 us, the short ones 5.2 and 8.4 against 4.3 (256 pairs) and 8.0 us.
+__global__ void __launch_bounds__(DOT_THREADS, 3)
     k_dot_batched(const DevPair *__restrict__ pairs, const DevPairAux *__restrict__ aux,
                   const DevUnit *__restrict__ units, uint32_t n_units, BatchScratch sc,
                   uint32_t *__restrict__ out)
 {
     __shared__ uint32_t s_u;
-    for (;;) {
-        if (threadIdx.x == 0) s_u = atomicAdd(&sc.ctr[0], 1u);
-        __syncthreads();
-        const uint32_t u = s_u;
-        if (u >= n_units) break;
+    // programmatic dependent launch, as in k_dot_single
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const bool more = n_units > gridDim.x;   // CTAs take further units
+    uint32_t u = blockIdx.x;
+    while (u < n_units) {
+        uint32_t nxt = 0;
+        if (more && threadIdx.x == 0) nxt = gridDim.x + atomicAdd(&sc.ctr[0], 1u);
         const DevUnit un = units[u];
         const DevPair pr = pairs[un.pair];
         const DevPairAux ax = aux[un.pair];
@@ -186,10 +211,19 @@ __global__ void __launch_bounds__(DOT_THREADS)
         case MONTGOMERY: r = unit_residue<AccMontgomery>(pr, un); break;
         default: r = unit_residue<AccPerTerm>(pr, un); break;
         }
-        const uint64_t s = cta_sum(r);   // its barriers also order the reuse of s_u
-        if (threadIdx.x == 0)
-            combine_and_finish(s, pr.m, sc.slots + un.pair, sc.tickets + un.pair, ax.units,
-                               out + un.pair);
+        if (threadIdx.x == 0) s_u = nxt;
+        const uint64_t s = cta_sum(r);   // its barriers also order s_u
+        if (threadIdx.x == 0) {
+            if (ax.units == 1)
+                out[un.pair] = reduce64(s, pr.m);
+            else if (ax.units <= 65535u)
+                combine_packed(s, pr.m, sc.slots + un.pair, ax.units, out + un.pair);
+            else
+                combine_and_finish(s, pr.m, sc.slots + un.pair, sc.tickets + un.pair, ax.units, out + un.pair);
+        }
+        if (!more) return;
+        u = s_u;
+        __syncthreads();   // every thread has read s_u before it is written again
     }
     if (threadIdx.x == 0) {
         __threadfence();
@@ -324,8 +358,17 @@ cudaError_t launch_dot_batched(const DevPair *pairs, const DevPairAux *aux, cons
                                uint32_t n_units, BatchScratch sc, uint32_t *out, int grid,
                                cudaStream_t s)
 {
-    k_dot_batched<<<grid, DOT_THREADS, 0, s>>>(pairs, aux, units, n_units, sc, out);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)std::max<uint32_t>(1, std::min<uint32_t>((uint32_t)grid, n_units)));
+    cfg.blockDim = dim3(DOT_THREADS);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_dot_batched, pairs, aux, units, n_units, sc, out);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 static uint64_t fill_key(uint64_t seed, uint64_t stream_id)
