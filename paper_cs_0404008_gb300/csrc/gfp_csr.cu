@@ -107,6 +107,14 @@ __global__ void __launch_bounds__(256)
 // are staged in shared memory so that a lane fetches its four pairs with two
 // 16-byte loads; the two halves' residues are added modulo p at the end.
 //
+// SPLIT, where rows are too few to give every second warp of the chip one: S
+// warps of a CTA share a row, each taking a run of its nonzeros, and their
+// residues meet in shared memory behind one barrier of the group.  A row is a
+// chain of L2 latencies, so its length over S is the time: 300 rows of 819
+// nonzeros x 64 columns 33 -> 10.3 us, 1000 of 328 17 -> 12.4 us a product (calls
+// back to back).  With rows enough for every warp the meetings cost more than the
+// evener split gives: 16384 rows of 164, 44 us unsplit, 58 us with S = 2.
+//
 // PLAIN (blocked representation, lambda >= 16): plain 64-bit sums with no
 // per-term bookkeeping.  A half adds at most 16 products per chunk of 32
 // nonzeros, so reducing the sums after every floor(lambda / 16) chunks keeps
@@ -162,9 +170,9 @@ __device__ __forceinline__ void csr_row_quads(uint32_t q0, uint32_t q1, uint64_t
     }
 }
 
-template <class Acc, bool PLAIN>
+template <class Acc, bool PLAIN, bool SPLIT>
 __global__ void __launch_bounds__(256, PLAIN ? 4 : 3)
-    k_block_csr_wide(Mod mod, uint64_t kbound, uint32_t segc, uint64_t m, uint64_t k, uint64_t nb,
+    k_block_csr_wide(Mod mod, uint64_t kbound, uint32_t segc, int S, uint64_t m, uint64_t k, uint64_t nb,
                      const uint32_t *__restrict__ row_ptr, const uint32_t *__restrict__ col,
                      const uint32_t *__restrict__ val, const uint32_t *__restrict__ B,
                      uint32_t ldb_bytes, uint32_t *__restrict__ C, uint64_t ldc)
@@ -172,12 +180,23 @@ __global__ void __launch_bounds__(256, PLAIN ? 4 : 3)
     __shared__ __align__(16) uint2 stage[8][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int half = lane >> 4, hl = lane & 15;
+    // residues of a row's warps, in two buffers by turns: a warp writes one again
+    // only after a barrier that the reader of its last contents has passed too
+    __shared__ uint4 meet[2][SPLIT ? 8 : 1][16];
+    uint32_t turn = 0;
     uint2 *st = stage[w];
-    const uint64_t warps = (uint64_t)gridDim.x * 8;
+    const int groups = SPLIT ? 8 / S : 8, group = SPLIT ? w / S : w, sub = SPLIT ? w % S : 0;
+    const uint64_t stride = (uint64_t)gridDim.x * groups;
     const bool cvec = ((((uintptr_t)C) & 15u) == 0) && (ldc % 4 == 0);
-    for (uint64_t row = (uint64_t)blockIdx.x * 8 + w; row < m; row += warps) {
-        const uint32_t q0 = __ldg(row_ptr + row), q1 = __ldg(row_ptr + row + 1);
+    for (uint64_t row = (uint64_t)blockIdx.x * groups + group; row < m; row += stride) {
+        uint32_t q0 = __ldg(row_ptr + row), q1 = __ldg(row_ptr + row + 1);
         GFP_DCHECK(g_csr_check, q0 <= q1, DCHECK_CSR_ROW_PTR);
+        if constexpr (SPLIT) {   // one of S equal runs, rounded up to steps of eight
+            const uint32_t n = q1 > q0 ? q1 - q0 : 0u, part = ((n + 8 * S - 1) / (8 * S)) * 8;
+            const uint32_t b = min(part * sub, n), e = min(b + part, n);
+            q1 = q0 + e;
+            q0 += b;
+        }
         for (uint64_t c0 = 0; c0 < nb; c0 += 64) {
             const uint64_t ca = c0 + 4 * (uint64_t)hl;
             const bool va = ca < nb;   // nb % 4 == 0: the whole quad is valid
@@ -232,7 +251,23 @@ __global__ void __launch_bounds__(256, PLAIN ? 4 : 3)
                 const uint64_t t = (uint64_t)r[j] + __shfl_xor_sync(0xffffffffu, r[j], 16);
                 r[j] = (uint32_t)(t >= mod.p ? t - mod.p : t);
             }
-            if (half == 0 && va) {
+            if constexpr (SPLIT) {
+                if (half == 0) meet[turn][w][hl] = make_uint4(r[0], r[1], r[2], r[3]);
+                asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "r"(32 * S) : "memory");
+                if (sub == 0 && half == 0) {
+                    for (int o = 1; o < S; ++o) {
+                        const uint4 t = meet[turn][w + o][hl];
+                        const uint32_t a4[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const uint64_t u = (uint64_t)r[j] + a4[j];
+                            r[j] = (uint32_t)(u >= mod.p ? u - mod.p : u);
+                        }
+                    }
+                }
+                turn ^= 1u;
+            }
+            if (half == 0 && sub == 0 && va) {
                 uint32_t *out = C + row * ldc + ca;
                 if (cvec) {
                     *reinterpret_cast<uint4 *>(out) = make_uint4(r[0], r[1], r[2], r[3]);
@@ -253,7 +288,7 @@ static int csr_wide_blocks_per_sm()
     static int cached = 0;
     if (!cached) {
         int b = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_block_csr_wide<Acc, PLAIN>, 256, 0) !=
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_block_csr_wide<Acc, PLAIN, false>, 256, 0) !=
                 cudaSuccess ||
             b < 1)
             b = 1;
@@ -269,12 +304,17 @@ static cudaError_t csr_wide_launch(const Mod &mod, uint64_t kbound, uint32_t seg
                                    uint64_t ldb, uint32_t *C, uint64_t ldc, int sm_count,
                                    cudaStream_t s)
 {
-    uint64_t blocks = (m + 7) / 8;
     const uint64_t cap = (uint64_t)sm_count * csr_wide_blocks_per_sm<Acc, PLAIN>();
-    if (blocks > cap) blocks = cap;
-    if (blocks < 1) blocks = 1;
-    k_block_csr_wide<Acc, PLAIN><<<(unsigned)blocks, 256, 0, s>>>(
-        mod, kbound, segc, m, k, nb, row_ptr, col, val, B, (uint32_t)(ldb * 4), C, ldc);
+    // warps per row: as many as leave every warp of the chip at most one part
+    int S = 1;
+    while (S < 8 && m * (uint64_t)(2 * S) <= cap * 8) S *= 2;
+    const uint64_t blocks = std::max<uint64_t>(1, std::min((m * S + 7) / 8, cap));
+    if (S > 1)
+        k_block_csr_wide<Acc, PLAIN, true><<<(unsigned)blocks, 256, 0, s>>>(
+            mod, kbound, segc, S, m, k, nb, row_ptr, col, val, B, (uint32_t)(ldb * 4), C, ldc);
+    else
+        k_block_csr_wide<Acc, PLAIN, false><<<(unsigned)blocks, 256, 0, s>>>(
+            mod, kbound, segc, 1, m, k, nb, row_ptr, col, val, B, (uint32_t)(ldb * 4), C, ldc);
     return cudaGetLastError();
 }
 
