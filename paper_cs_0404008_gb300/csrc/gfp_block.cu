@@ -131,8 +131,9 @@ struct Args {
     const uint8_t *Bimg;      // [n_tiles][kblocks] tiles of B_TILE_BYTES
     uint32_t *C;
     uint64_t ldc;
-    uint32_t *Cacc;           // (n_tiles*NT) x m u32 partial residue sums, column-major: the
-                              // entry of row i, column j at j*m + i (zero outside calls)
+    uint32_t *Cacc;           // (n_tiles*NT) x m u32 partial residue sums, by pairs of columns:
+                              // row i of columns 2 j and 2 j + 1 at 2 (j m + i) and the next
+                              // word (zero outside calls)
     uint32_t *err;            // bit 0: a bounded wait expired
     uint32_t p, half;         // half = (p-1)/2
     uint32_t magic;           // floor(2^32 / p)
@@ -665,8 +666,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_block_tc(const __grid_constant__
             const uint64_t col0 = (uint64_t)w.nt * NT + c_first;
             // columns of this warp's 32 that exist (none for a row outside)
             const int ncols = grow < a.m && col0 < a.nb ? (int)min(a.nb - col0, (uint64_t)32) : 0;
-            uint32_t *dst = a.direct ? a.C + grow * a.ldc + col0 : a.Cacc + col0 * a.m + grow;
-            const uint64_t step = a.direct ? 1 : a.m;
+            uint32_t *dst = a.direct ? a.C + grow * a.ldc + col0 : a.Cacc + col0 * a.m + 2 * grow;
 #pragma unroll 1
             for (int g = 0; g < 32; g += 8) {
                 uint32_t hh[8], md[8], ll[8];
@@ -701,12 +701,16 @@ __global__ void __launch_bounds__(THREADS, 1) k_block_tc(const __grid_constant__
                     for (int j = 0; j < 8; ++j)
                         if (g + j < ncols) dst[g + j] = min(hh[j], hh[j] - a.p);
                 } else {
-                    // column-major partial sums: the 32 lanes of a warp
-                    // (consecutive rows) add to 128 consecutive bytes
+                    // two columns in one 64-bit addition (neither sum reaches
+                    // 2^32, so nothing carries between them; columns past the
+                    // last add their zero), the 32 lanes of a warp, consecutive
+                    // rows, to 256 consecutive bytes
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        if (g + j < ncols) atomicAdd(dst, hh[j]);
-                        dst += step;
+                    for (int j = 0; j < 8; j += 2) {
+                        if (g + j < ncols)
+                            atomicAdd(reinterpret_cast<unsigned long long *>(dst),
+                                      (unsigned long long)hh[j] | (unsigned long long)hh[j + 1] << 32);
+                        dst += 2 * a.m;
                     }
                 }
             }
@@ -799,18 +803,22 @@ __global__ void __launch_bounds__(FIN_THREADS)
     // all of a thread's loads are issued before any is used or cleared (one
     // memory latency, not one per element); consecutive threads take
     // consecutive rows of one column
-    uint32_t v[PER];
+    constexpr int PAIRS = PER / 2;
+    uint2 v[PAIRS];
+    uint2 *acc = reinterpret_cast<uint2 *>(Cacc);
 #pragma unroll
-    for (int e = 0; e < PER; ++e) {
-        const int i = threadIdx.x + e * FIN_THREADS, c = i / BM, r = i % BM;
-        v[e] = (r0 + r < m && c0 + c < nb) ? __ldcg(&Cacc[(c0 + c) * m + r0 + r]) : 0u;
+    for (int e = 0; e < PAIRS; ++e) {
+        const int i = threadIdx.x + e * FIN_THREADS, c = i / BM * 2, r = i % BM;
+        v[e] = (r0 + r < m && c0 + c < nb) ? __ldcg(&acc[(c0 + c) / 2 * m + r0 + r]) : make_uint2(0u, 0u);
     }
 #pragma unroll
-    for (int e = 0; e < PER; ++e) {
-        const int i = threadIdx.x + e * FIN_THREADS, c = i / BM, r = i % BM;
-        v[e] = reduce_small(v[e], p, magic);   // the sums are below 2^32
-        if (r0 + r < m && c0 + c < nb) __stcg(&Cacc[(c0 + c) * m + r0 + r], C ? 0u : v[e]);
-        t[c][r] = v[e];
+    for (int e = 0; e < PAIRS; ++e) {
+        const int i = threadIdx.x + e * FIN_THREADS, c = i / BM * 2, r = i % BM;
+        v[e].x = reduce_small(v[e].x, p, magic);   // the sums are below 2^32
+        v[e].y = reduce_small(v[e].y, p, magic);
+        if (r0 + r < m && c0 + c < nb) __stcg(&acc[(c0 + c) / 2 * m + r0 + r], C ? make_uint2(0u, 0u) : v[e]);
+        t[c][r] = v[e].x;
+        t[c + 1][r] = v[e].y;
     }
     if (!C) return;
     __syncthreads();
