@@ -258,14 +258,18 @@ GFP_API gfp_status gfp_matvec_sequence(gfp_ctx *ctx, uint32_t p, uint64_t n, con
 /* C[i*ldc + j] = (sum_t A[i*lda + t] * B[t*ldb + j]) mod p, 0 <= i < m,
  * 0 <= j < nb.  A (m x k), B (k x nb), C (m x nb): device, row-major,
  * lda >= k, ldb >= nb, ldc >= nb; C must not overlap A or B.
- * Path: with GFP_REPR_AUTO or GFP_REPR_F16TC, A 16-byte aligned and lda a
- * multiple of 4, the tensor cores: for p <= 65791 the digit kernel directly
+ * Path: with GFP_REPR_AUTO, or with GFP_REPR_F16TC, A 16-byte aligned and lda
+ * a multiple of 4, the tensor cores: for p <= 65791 the digit kernel directly
  * (three launches: B digit split, the persistent product, the reduction of
- * its partial sums into C); for larger p
+ * its partial sums into C; two where K is at most 512 and the row and column
+ * tiles fill the GPU); for larger p
  * one such pass per modulus of a residue number system (the L <= 6 largest
  * primes <= 65536 whose product exceeds k (p-1)^2, each pass reducing the
- * inputs modulo its prime) and one launch recombining the residues with
- * Garner's method modulo p.  Otherwise the CUDA-core kernel with the
+ * inputs modulo its prime; B's digits for all of them in one launch) and one
+ * launch recombining the residues with
+ * Garner's method modulo p, where that is expected to be faster than the
+ * CUDA cores.  Rows of A at other alignments take the same kernel with 4-byte
+ * loads.  Otherwise the CUDA-core kernel with the
  * representation forced on the context, else the built-in rule for p (tuned
  * plans time the dot-product kernels and do not apply here; forcing F16TC
  * where the tensor cores are not eligible gives GFP_ERR_UNSUPPORTED).  The tensor-core path
@@ -283,7 +287,7 @@ GFP_API gfp_status gfp_matmul_block(gfp_ctx *ctx, uint32_t p, uint64_t m, uint64
  * representative of each residue taken in [-32896, 32639] so that both
  * digits fit a byte), stored as two 8-bit digit planes per tile, 2 bytes per
  * entry of A: each product reads half the bytes of the uint32 A and only
- * widens the digits to fp16 in shared memory.  For p <= 65536 one image; for
+ * widens the digits to fp16.  For p <= 65536 one image; for
  * larger p one image per residue-pass modulus (A reduced modulo each, 2 bytes
  * per entry each; gfp_block_prep_info gives the bytes and the pass count).
  *   A: device, m x k row-major, lda >= k, canonical residues; not referenced
@@ -297,7 +301,8 @@ GFP_API gfp_status gfp_block_prepare(gfp_ctx *ctx, uint32_t p, uint64_t m, uint6
 /* C = A B mod p for the prepared A (m x k): B device k x nb (ldb >= nb),
  * C device m x nb (ldc >= nb); the same result as gfp_matmul_block on the
  * original A.  Three launches (B's digits, the product, its partial sums
- * into C), or three per residue pass plus one recombination.  Uses the
+ * into C), or for residue passes B's digits once, two a pass and one
+ * recombination.  Uses the
  * context's block workspace (grown on first use of a shape: make that call
  * outside stream capture); calls sharing one context must not run
  * concurrently on different streams. */

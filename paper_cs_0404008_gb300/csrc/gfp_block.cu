@@ -32,18 +32,33 @@
 //     warp 25      bulk-copies B's digit tiles, split once by a small kernel
 //                  before this one, each as soon as the MMAs of the K range
 //                  before have read its place for the last time
-//   Each output meets the partial sums of its K ranges in a column-major u32
-//   workspace (coalesced atomics, one transaction per column and warp), and a
-//   small kernel behind this one reduces the sums mod p, writes C through a
-//   shared-memory transpose and clears the workspace; a product with a single
-//   K range writes C directly.
+//   The residues of a unit are added to a u32 workspace, two columns in one
+//   64-bit addition, and a small kernel behind this one reduces the sums mod p,
+//   writes C through a shared-memory transpose and clears the workspace; a product
+//   with a single K range writes C directly.
+//
+//   What bounds it (16384 x 16384 x 64 over GF(65521), calls back to back, before
+//   -> now; before: A through in-place shared-memory slots, B's tiles re-read for
+//   every row tile):  uint32 A 215 -> 176 us, HBM at 6.1 TB/s of the 6.5-7.0 that
+//   loads in this pattern reach alone; prepared A 172 -> 117 us, the hand-over of
+//   TMEM slots between converters and MMAs (0.45 us per k-block against 0.265 us of
+//   MMAs and 0.37 us of HBM).  In the order they were taken, with a flushed L2
+//   (uint32 / prepared): digits in shared-memory slots beside the resident B
+//   366 / 304 us (28 KiB of L1 left: the loads in flight did not fit), digits in
+//   TMEM 253 / 206, fewer instructions per k-block 213 / 177, B's tiles split by a
+//   kernel of its own instead of by each CTA 201 / 156, MMAs issued from a converged
+//   warp 196 / 135, two converter groups 184 / 114, 64-bit additions 185 / 111.
+//   Not kept: half-k-block hand-overs (125 prepared), a look ahead at the next
+//   slot's barrier (116), L2 prefetch of the next unit (197 uint32), 32-byte loads
+//   (186), more half k-blocks in registers (199 / 121), remainders of the drain in
+//   fp32 (117 prepared).
 //
 // Larger moduli on the tensor cores (p > 65791): the exact integer products
 // sum_t A[i][t] B[t][j] are below k (p-1)^2, so they are fixed by their
 // residues modulo a few small primes p' <= 65536 whose product exceeds that
 // bound (a residue number system).  Each pass runs the tensor-core kernel
 // above modulo one p', reducing every input a < 2^32 to a mod p' while it is
-// split into digits; a last kernel recombines the residues with Garner's
+// split into digits (B's digits for all passes are made by one launch); a last kernel recombines the residues with Garner's
 // mixed-radix method and evaluates the integer modulo p.
 //
 // CUDA-core path (any p <= 2^32-1): shared-memory tiled product with the

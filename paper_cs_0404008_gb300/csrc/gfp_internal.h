@@ -218,7 +218,7 @@ struct gfp_ctx {
     uint32_t *stage_out = nullptr;
     size_t stage_out_elems = 0;
 
-    // block-product buffer: error flag and column-major partial sums at its
+    // block-product buffer: error flag and partial sums (by pairs of columns) at its
     // start, zero outside calls; B's digit tiles and the residue matrices of the
     // passes of a large modulus at its end; grown on demand
     void *blk_ws = nullptr;
