@@ -218,11 +218,11 @@ struct gfp_ctx {
     uint32_t *stage_out = nullptr;
     size_t stage_out_elems = 0;
 
-    // block-product buffer: error flag and partial sums (by pairs of columns) at its
-    // start, zero outside calls; B's digit tiles and the residue matrices of the
-    // passes of a large modulus at its end; grown on demand
+    // block-product buffer: error flag and partial sums (by pairs of columns),
+    // zero outside calls; behind them B's digit tiles and the residue matrices of
+    // the passes of a large modulus; grown on demand
     void *blk_ws = nullptr;
-    size_t blk_ws_bytes = 0, blk_zero = 0;   // size, length of the prefix known to be zero
+    size_t blk_ws_bytes = 0, blk_tail_bytes = 0;   // sizes of the two parts
 
     // tuned plan: (p, lg_n) -> entry
     std::map<std::pair<uint32_t, uint32_t>, gfp_plan_entry> plan;

@@ -771,34 +771,36 @@ static int block_sms(const gfp_ctx *ctx)
 }
 
 // Block-product buffer of the context for an m x k by k x nb product with n_mod
-// moduli, one allocation grown on demand: the workspace at its start, B's digit
-// tiles and (where there are several moduli) the residue matrices at its end.
-// Only [0, blk_zero) is known to be zero; the caller holds ctx->mu.
+// moduli: the workspace (zero outside calls), then B's digit tiles and, where
+// there are several moduli, the residue matrices.  One allocation, grown on
+// demand to the largest of either part, so that no shape's tiles reach into
+// another's workspace; the caller holds ctx->mu.
 static gfp_status ensure_block_ws(gfp_ctx *ctx, uint64_t m, uint64_t k, uint64_t nb, int n_mod, cudaStream_t s,
                                   BlockScratch *sc, uint32_t **res)
 {
     const size_t ws = align256(block_tc_workspace_bytes(m, nb)), img = align256(block_tc_bimg_bytes(k, nb, n_mod));
-    const size_t rb = n_mod > 1 ? align256((size_t)n_mod * m * nb * 4) : 0, need = ws + img + rb;
-    if (need > ctx->blk_ws_bytes) {
+    const size_t tail = img + (n_mod > 1 ? align256((size_t)n_mod * m * nb * 4) : 0);
+    if (ws > ctx->blk_ws_bytes || tail > ctx->blk_tail_bytes) {
         GFP_CUDA_TRY(cudaDeviceSynchronize());   // work in flight may still use the old one
+        size_t w = std::max(ws, ctx->blk_ws_bytes), t = std::max(tail, ctx->blk_tail_bytes);
         if (ctx->blk_ws) cudaFree(ctx->blk_ws);
         ctx->blk_ws = nullptr;
-        ctx->blk_ws_bytes = ctx->blk_zero = 0;
-        if (cudaMalloc(&ctx->blk_ws, need) != cudaSuccess) {
-            ctx->blk_ws = nullptr;
-            return GFP_ERR_NOMEM;
+        ctx->blk_ws_bytes = ctx->blk_tail_bytes = 0;
+        if (cudaMalloc(&ctx->blk_ws, w + t) != cudaSuccess) {
+            w = ws;   // no room for both largest parts: this product's alone
+            t = tail;
+            if (cudaMalloc(&ctx->blk_ws, w + t) != cudaSuccess) {
+                ctx->blk_ws = nullptr;
+                return GFP_ERR_NOMEM;
+            }
         }
-        ctx->blk_ws_bytes = need;
+        GFP_CUDA_TRY(cudaMemsetAsync(ctx->blk_ws, 0, w, s));
+        ctx->blk_ws_bytes = w;
+        ctx->blk_tail_bytes = t;
     }
-    uint8_t *base = (uint8_t *)ctx->blk_ws, *tail = base + (ctx->blk_ws_bytes - img - rb) / 256 * 256;
-    if (ws > ctx->blk_zero) {
-        GFP_CUDA_TRY(cudaMemsetAsync(base + ctx->blk_zero, 0, ws - ctx->blk_zero, s));
-        ctx->blk_zero = ws;
-    }
-    ctx->blk_zero = std::min<size_t>(ctx->blk_zero, (size_t)(tail - base));   // the rest is written below
-    sc->ws = base;
-    sc->bimg = tail;
-    *res = (uint32_t *)(tail + img);
+    sc->ws = ctx->blk_ws;
+    sc->bimg = (uint8_t *)ctx->blk_ws + ctx->blk_ws_bytes;
+    *res = (uint32_t *)(sc->bimg + img);
     return GFP_OK;
 }
 
@@ -1032,7 +1034,6 @@ GFP_API gfp_status gfp_context_check(gfp_ctx *ctx)
     GFP_CUDA_TRY(cudaMemcpy(&h, ctx->blk_ws, 4, cudaMemcpyDeviceToHost));   // the error flag
     if (h) {
         GFP_CUDA_TRY(cudaMemset(ctx->blk_ws, 0, ctx->blk_ws_bytes));
-        ctx->blk_zero = ctx->blk_ws_bytes;
         return GFP_ERR_TIMEOUT;
     }
     return dbits ? GFP_ERR_INVALID : GFP_OK;

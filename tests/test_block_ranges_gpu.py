@@ -98,3 +98,30 @@ def test_block_k_beyond_one_launch(lib, p):
         assert np.array_equal(host(C), oracle.block(p, A, B))
     finally:
         c.close()
+
+
+def test_block_graph_replay_after_another_shape(lib):
+    """A captured product replays exactly after the context ran products of
+    other shapes (their operands never reach the captured one's partial sums)."""
+    c = lib.Context(0)
+    try:
+        p, m, k, nb = 65521, 3000, 1300, 64
+        A, B = gi.uniform(p, m * k, 96, 0).reshape(m, k), gi.uniform(p, k * nb, 96, 1).reshape(k, nb)
+        want = oracle.block(p, A, B)
+        check(lib, c, p, 200, 20000, 64)          # larger tiles of B, smaller result
+        Ad, Bd, C = dev2(A), dev2(B), torch.zeros((m, nb), dtype=torch.int32, device="cuda")
+        lib.gfp_matmul_block(c, p, Ad, Bd, C)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        s = torch.cuda.Stream()
+        with torch.cuda.graph(g, stream=s):
+            lib.gfp_matmul_block(c, p, Ad, Bd, C)
+        for m2, k2 in ((200, 20000), (64, 15000), (2500, 900)):
+            check(lib, c, p, m2, k2, 64)
+            C.fill_(-1)
+            g.replay()
+            torch.cuda.synchronize()
+            assert np.array_equal(host(C), want), (m2, k2)
+        del g
+    finally:
+        c.close()
