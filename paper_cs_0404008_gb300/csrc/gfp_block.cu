@@ -17,8 +17,8 @@
 //   terms (eight 64-deep k-blocks) of one 64-column tile of B.  Units are
 //   ordered with the row tiles innermost and split evenly over one persistent
 //   CTA per SM, so a CTA works through many row tiles against the same K
-//   range: that range's B digits (128 KiB) stay in shared memory and are made
-//   once per range, and A alone streams.  A's digits go to TMEM, from where
+//   range: that range's B digits (128 KiB) are copied to shared memory once and
+//   stay, and A alone streams.  A's digits go to TMEM, from where
 //   the MMAs read them: shared memory sees only B, and the rest of its 256 KiB
 //   per SM stays L1, which is where loads in flight land.  Roles per CTA:
 //     warps 0-15   load A with 16-byte loads (64 KiB in flight per SM), centre
@@ -58,8 +58,9 @@
 // residues modulo a few small primes p' <= 65536 whose product exceeds that
 // bound (a residue number system).  Each pass runs the tensor-core kernel
 // above modulo one p', reducing every input a < 2^32 to a mod p' while it is
-// split into digits (B's digits for all passes are made by one launch); a last kernel recombines the residues with Garner's
-// mixed-radix method and evaluates the integer modulo p.
+// split into digits (B's digits for all passes are made by one launch); a last
+// kernel recombines the residues with Garner's mixed-radix method and evaluates
+// the integer modulo p.
 //
 // CUDA-core path (any p <= 2^32-1): shared-memory tiled product with the
 // per-thread unreduced accumulators of the dot-product kernels.
@@ -993,11 +994,6 @@ __global__ void __launch_bounds__(CC_THREADS)
 bool block_tc_layout_ok(const uint32_t *A, uint64_t lda)
 {
     return ((((uintptr_t)A) & 15u) == 0) && (lda % 4 == 0);
-}
-
-bool block_tc_eligible(uint32_t p, const uint32_t *A, uint64_t lda)
-{
-    return p >= 2 && p <= BLOCK_TC_MAX_P && block_tc_layout_ok(A, lda);
 }
 
 static uint32_t pow_mod_small(uint64_t b, uint64_t e, uint32_t m)

@@ -125,7 +125,6 @@ constexpr uint32_t BLOCK_TC_MAX_P = 65791;
 // Moduli of the residue passes, and of prepared operands taken directly: at
 // most 65536, so that every residue has two 8-bit balanced digits.
 constexpr uint32_t RNS_PRIME_MAX = 65536;
-bool block_tc_eligible(uint32_t p, const uint32_t *A, uint64_t lda);
 // A's layout suits 16-byte loads (16-byte base, rows a multiple of 16 bytes apart)
 bool block_tc_layout_ok(const uint32_t *A, uint64_t lda);
 
