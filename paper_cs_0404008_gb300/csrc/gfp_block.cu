@@ -40,9 +40,9 @@
 //   What bounds it (16384 x 16384 x 64 over GF(65521), calls back to back, before
 //   -> now; before: A through in-place shared-memory slots, B's tiles re-read for
 //   every row tile):  uint32 A 215 -> 176 us, HBM at 6.1 TB/s of the 6.5-7.0 that
-//   loads in this pattern reach alone; prepared A 172 -> 117 us, the hand-over of
-//   TMEM slots between converters and MMAs (0.45 us per k-block against 0.265 us of
-//   MMAs and 0.37 us of HBM).  In the order they were taken, with a flushed L2
+//   loads in this pattern reach alone; prepared A 172 -> 128 us, the hand-over of
+//   TMEM slots between converters and MMAs (0.5 us per k-block against 0.37 us of
+//   HBM).  In the order they were taken, with a flushed L2
 //   (uint32 / prepared): digits in shared-memory slots beside the resident B
 //   366 / 304 us (28 KiB of L1 left: the loads in flight did not fit), digits in
 //   TMEM 253 / 206, fewer instructions per k-block 213 / 177, B's tiles split by a
@@ -79,9 +79,9 @@ namespace blk {
 constexpr int BM = 128;            // rows per tile (MMA M)
 constexpr int BK = 64;             // K per k-block: one 128-byte swizzle row of fp16
 constexpr int NT = 64;             // output columns per n-tile
-constexpr int MMA_N = 2 * NT;      // low and high digits of B stacked along N
+constexpr int B_ROWS = 2 * NT;     // low and high digits of B, one below the other
 constexpr int RK = 8;              // k-blocks per K range at most: 512 terms, the exact chunk
-constexpr int B_TILE_BYTES = MMA_N * BK * 2;                  // 16 KiB
+constexpr int B_TILE_BYTES = B_ROWS * BK * 2;                 // 16 KiB
 // A's digits live in TMEM: two slots of one k-block each
 constexpr int SLOTS = 2;
 constexpr uint32_t SLOT_COLS = 64;                            // 32 columns per digit
@@ -101,8 +101,14 @@ static_assert(W_EPI0 % 4 == 0, "an epilogue warp reads the TMEM lanes of its ind
 constexpr uint32_t TMEM_COLS = 512;
 static_assert(A_COL0 + SLOTS * SLOT_COLS == TMEM_COLS, "accumulators and A digits fill TMEM");
 constexpr uint64_t WAIT_NS = 2000000000ull;   // bounded waits: 2 s
-constexpr uint32_t IDESC = ptx::idesc_f16_f32(BM, MMA_N);
-constexpr uint32_t IDESC_HALF = ptx::idesc_f16_f32(BM, NT);
+// Every MMA is 128 x 64 x 16 and adds into one of three accumulators that do not
+// overlap: MMAs in flight are ordered among themselves only where accumulator and
+// shape are the same, and the middle sum takes two MMAs per 16 K.  (One 128-wide
+// MMA for each digit of A, over ll | middle and middle | hh, took 108.6 us for the
+// prepared 16384 x 16384 x 64 against 122.5 us, the same for uint32 A; its middle
+// sum would rest on an order that nothing promises.)
+constexpr uint32_t IDESC = ptx::idesc_f16_f32(BM, NT);
+constexpr uint64_t B_HIGH = (NT * 128) >> 4;   // from a tile's low to its high digits, in descriptor units
 // terms of one launch: 2^24 / 512 partial sums below p <= 65791, and one more
 // (the sums of earlier launches, folded below p), stay below 2^32
 constexpr uint64_t SLAB_K = 1ull << 24;
@@ -583,8 +589,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_block_tc(const __grid_constant__
             // the accumulator set was drained by the unit before the last
             if (!wait_bar_warp(ptx::smem_u32(&bars->acc_empty[b]), bph, abort, a.err)) break;
             ptx::tc_fence_after();
-            const uint32_t d_lo = tmem + b * ACC_COLS;   // A low digit x [B lo | B hi]: ll, lh
-            const uint32_t d_hi = d_lo + NT;             // A high digit x [B lo | B hi]: hl, hh
+            const uint32_t d_ll = tmem + b * ACC_COLS, d_md = d_ll + NT, d_hh = d_md + NT;
             const bool final = w.last_of_range(a);
             uint32_t t = bset * a.bset_tiles;
             uint64_t db = ptx::sdesc_k_sw128(ptx::smem_u32(btiles + t * B_TILE_BYTES));
@@ -597,20 +602,20 @@ __global__ void __launch_bounds__(THREADS, 1) k_block_tc(const __grid_constant__
                 if (!ok) break;
                 ptx::tc_fence_after();
                 const uint32_t ah = tmem + A_COL0 + s * SLOT_COLS, al = ah + SLOT_COLS / 2;
-                // 16 K: eight TMEM columns of A, 32 bytes of B inside the swizzle atom
-                if (j == 0) {
-                    // the middle columns then hold lh; hh starts from zero
-                    ptx::mma_f16_ts(lead, d_lo, al, db, IDESC, 0u);
-                    ptx::mma_f16_ts(lead, d_hi, ah, db, IDESC_HALF, 1u);
-                    ptx::mma_f16_ts(lead, d_hi + NT, ah, db + ((64 * 128) >> 4), IDESC_HALF, 0u);
-                } else {
-                    ptx::mma_f16_ts(lead, d_lo, al, db, IDESC, 1u);
-                    ptx::mma_f16_ts(lead, d_hi, ah, db, IDESC, 1u);
-                }
+                // 16 K: eight TMEM columns of A, 32 bytes of B inside the swizzle atom.
+                // Two such steps an accumulator at a time: 122.5 us for the prepared
+                // 16384 x 16384 x 64, one at a time 125.3, four 141.2
 #pragma unroll
-                for (uint32_t kk = 1; kk < 4; ++kk) {
-                    ptx::mma_f16_ts(lead, d_lo, al + 8 * kk, db + 2 * kk, IDESC, 1u);
-                    ptx::mma_f16_ts(lead, d_hi, ah + 8 * kk, db + 2 * kk, IDESC, 1u);
+                for (uint32_t kk = 0; kk < 4; kk += 2) {
+                    const uint32_t more = kk || j ? 1u : 0u;
+                    const auto two = [&](uint32_t d, uint32_t at, uint64_t bd, uint32_t accumulate) {
+                        ptx::mma_f16_ts(lead, d, at + 8 * kk, bd + 2 * kk, IDESC, accumulate);
+                        ptx::mma_f16_ts(lead, d, at + 8 * kk + 8, bd + 2 * kk + 2, IDESC, 1u);
+                    };
+                    two(d_ll, al, db, more);
+                    two(d_md, al, db + B_HIGH, more);
+                    two(d_md, ah, db, 1u);
+                    two(d_hh, ah, db + B_HIGH, more);
                 }
                 ptx::mma_commit(lead, ptx::smem_u32(&bars->a_empty[s]));
                 if (final) ptx::mma_commit(lead, ptx::smem_u32(&bars->b_empty[t]));
