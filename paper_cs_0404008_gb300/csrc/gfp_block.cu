@@ -97,6 +97,7 @@ static_assert(REGS_LAUNCH * THREADS ==
                   32 * (REGS_CONV * CONV_GROUPS * CONV_WARPS + REGS_EPI * EPI_WARPS + REGS_MMA * 4),
               "the roles' registers are exactly those the block is launched with");
 static_assert(REGS_LAUNCH * THREADS <= 65536, "one CTA per SM");
+static_assert(W_EPI0 % 4 == 0 && W_MMA % 4 == 0, "the shares go to whole warpgroups");
 static_assert(W_EPI0 % 4 == 0, "an epilogue warp reads the TMEM lanes of its index modulo 4");
 constexpr uint32_t TMEM_COLS = 512;
 static_assert(A_COL0 + SLOTS * SLOT_COLS == TMEM_COLS, "accumulators and A digits fill TMEM");
@@ -508,6 +509,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_block_tc(const __grid_constant__
     ptx::tc_fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);   // uniform, as above
     volatile uint32_t *abort = &bars->abort;
+    // registers by role, each share by one instruction for all warps of a
+    // warpgroup (the .aligned form wants that), so ahead of the roles: the last
+    // warpgroup holds several
+    if (warp < W_EPI0) ptx::regs_inc<REGS_CONV>();
+    else if (warp < W_MMA) ptx::regs_dec<REGS_EPI>();
+    else ptx::regs_dec<REGS_MMA>();
     // Programmatic dependent launch: this grid may be placed while the previous
     // kernel of the stream, the one that makes B's digits or reduces the partial
     // sums of the pass before, is still running.  What came before that kernel
@@ -516,7 +523,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_block_tc(const __grid_constant__
 
     if (warp < W_EPI0) {
         // ---------------- converters: A to fp16 digits ----------------
-        ptx::regs_inc<REGS_CONV>();
         // each group takes every second k-block: while one waits for its slot's
         // MMAs the other converts
         const int group = warp / CONV_WARPS, gw = warp % CONV_WARPS;
@@ -579,7 +585,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_block_tc(const __grid_constant__
         // the loop every operand of every MMA was moved there first, and the
         // eight MMAs of a k-block took 750-1000 cycles to issue against the 503
         // they need
-        ptx::regs_dec<REGS_MMA>();
         const uint32_t lead = ptx::elect_one();
         Walk w;
         w.start(a, u0, u1);
@@ -637,7 +642,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_block_tc(const __grid_constant__
         __syncwarp();
     } else if (warp > W_MMA) {
         // ---------------- B digit tiles, once per K range (bulk copies) ----------------
-        ptx::regs_dec<REGS_MMA>();
         if (warp == W_BPROD && lane == 0) {
             asm volatile("griddepcontrol.wait;" ::: "memory");
             Walk w;
@@ -673,7 +677,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_block_tc(const __grid_constant__
         }
     } else {
         // ---------------- epilogue: TMEM -> residues ----------------
-        ptx::regs_dec<REGS_EPI>();
         asm volatile("griddepcontrol.wait;" ::: "memory");
         const int quarter = warp & 3;               // TMEM lanes 32*quarter .. +31
         const uint32_t c_first = (uint32_t)((warp - W_EPI0) >> 2) * 32u;   // this warp's 32 columns
