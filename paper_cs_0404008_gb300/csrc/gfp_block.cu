@@ -1131,6 +1131,11 @@ cudaError_t launch_block_tc(const uint32_t *mods, int n_mod, uint64_t m, uint64_
             // the rest of the 256 KiB stays L1: the loads in flight land there
             if (e == cudaSuccess)
                 e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 58);
+            // a warpgroup that asks for more registers than the block was launched
+            // with waits forever: nothing but the planned number is launched
+            cudaFuncAttributes fa;
+            if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, f);
+            if (e == cudaSuccess && fa.numRegs != REGS_LAUNCH) e = cudaErrorInvalidDeviceFunction;
             if (e != cudaSuccess) return e;
         }
         attr = true;
