@@ -515,11 +515,14 @@ __global__ void __launch_bounds__(THREADS, 1) k_block_tc(const __grid_constant__
     if (warp < W_EPI0) ptx::regs_inc<REGS_CONV>();
     else if (warp < W_MMA) ptx::regs_dec<REGS_EPI>();
     else ptx::regs_dec<REGS_MMA>();
-    // Programmatic dependent launch: this grid may be placed while the previous
-    // kernel of the stream, the one that makes B's digits or reduces the partial
-    // sums of the pass before, is still running.  What came before that kernel
-    // is complete (it waited for it), so A may be read at once; the roles that
-    // touch B's digits or the partial sums wait for it.
+    // Programmatic dependent launch: this grid may be placed, and sets itself up,
+    // while the previous kernel of the stream, the one that makes B's digits or
+    // reduces the partial sums of the pass before, is still running.  What it and
+    // the kernels before it wrote is visible behind griddepcontrol.wait only, so
+    // every role that touches global memory starts with it.  (Converters that load
+    // A ahead of it, on the ground that A's writer completed before the previous
+    // kernel went on, gained 0.6 of 174 us and nothing of 20 us; one wait ahead of
+    // the roles made the compiler spill, 750 us.)
 
     if (warp < W_EPI0) {
         // ---------------- converters: A to fp16 digits ----------------
@@ -536,6 +539,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_block_tc(const __grid_constant__
         ld.locate(a, gw, lane);
         if (group) ld.advance(a, gw, lane, 1);
         uint32_t loaded = 0;
+        asm volatile("griddepcontrol.wait;" ::: "memory");
 #pragma unroll
         for (int d = 0; d < D; ++d) {
             if (!ld.end) {
