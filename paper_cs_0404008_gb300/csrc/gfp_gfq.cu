@@ -609,7 +609,7 @@ GFP_API gfp_status gfp_gfq_create(int device, uint32_t p, uint32_t k, const uint
     fq->mode = p == 2 ? 2 : (k == 1 ? 1 : (small_ext ? 3 : 0));
     cudaError_t e = cudaSuccess;
     auto alloc = [&](void **ptr, size_t bytes) {
-        if (e == cudaSuccess) e = cudaMalloc(ptr, bytes);
+        if (e == cudaSuccess) e = dev_malloc(ptr, bytes);
     };
     alloc((void **)&fq->d_zech, gfq::SMEM);
     alloc((void **)&fq->d_log, (size_t)q * 4);

@@ -75,6 +75,23 @@ struct DevUnit {
     uint32_t pad;
 };
 
+// cudaMalloc whose failure stays with the caller: the runtime keeps a failed call's
+// error until it is asked for, and the next launch's check would take it for its own.
+inline cudaError_t dev_malloc(void **p, size_t bytes)
+{
+    const cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess) {
+        *p = nullptr;
+        (void)cudaGetLastError();
+    }
+    return e;
+}
+template <class T>
+cudaError_t dev_malloc(T **p, size_t bytes)
+{
+    return dev_malloc((void **)p, bytes);
+}
+
 // Records a CUDA error for gfp_last_cuda_error (entry points in other units).
 void note_cuda_error(cudaError_t e);
 

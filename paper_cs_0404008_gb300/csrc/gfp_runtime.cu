@@ -416,7 +416,7 @@ GFP_API gfp_status gfp_context_create(int device, gfp_ctx **out)
     }
     const size_t ring_bytes = (size_t)c->ring_size * sizeof(unsigned long long);
     void *mem = nullptr;
-    if (cudaMalloc(&mem, ring_bytes + 256) != cudaSuccess) {
+    if (dev_malloc(&mem, ring_bytes + 256) != cudaSuccess) {
         delete c;
         return GFP_ERR_NOMEM;
     }
@@ -513,7 +513,7 @@ GFP_API gfp_status gfp_batch_plan_create(gfp_ctx *ctx, const gfp_dot_desc *d, ui
     BatchLayout L(count, hb.units.size());
     gfp_batch_plan *pl = new (std::nothrow) gfp_batch_plan();
     if (!pl) return GFP_ERR_NOMEM;
-    if (cudaMalloc(&pl->mem, L.total) != cudaSuccess) {
+    if (dev_malloc(&pl->mem, L.total) != cudaSuccess) {
         delete pl;
         return GFP_ERR_NOMEM;
     }
@@ -591,7 +591,7 @@ static gfp_status batched_oneshot(gfp_ctx *ctx, const gfp_dot_desc *d, uint64_t 
             ctx->bw_bytes = 0;
         }
         const size_t want = std::max<size_t>(L.total, (size_t)1 << 20);
-        if (cudaMalloc(&ctx->bw, want) != cudaSuccess) return GFP_ERR_NOMEM;
+        if (dev_malloc(&ctx->bw, want) != cudaSuccess) return GFP_ERR_NOMEM;
         ctx->bw_bytes = want;
         fresh = true;
     }
@@ -645,7 +645,7 @@ GFP_API gfp_status gfp_dot_batched_host(gfp_ctx *ctx, uint64_t count, const uint
         if (ctx->stage) cudaFree(ctx->stage);
         ctx->stage = nullptr;
         ctx->stage_elems = 0;
-        if (cudaMalloc(&ctx->stage, need * 4) != cudaSuccess) return GFP_ERR_NOMEM;
+        if (dev_malloc(&ctx->stage, need * 4) != cudaSuccess) return GFP_ERR_NOMEM;
         ctx->stage_elems = need;
     }
     if (count > ctx->stage_out_elems) {
@@ -653,7 +653,7 @@ GFP_API gfp_status gfp_dot_batched_host(gfp_ctx *ctx, uint64_t count, const uint
         if (ctx->stage_out) cudaFree(ctx->stage_out);
         ctx->stage_out = nullptr;
         ctx->stage_out_elems = 0;
-        if (cudaMalloc(&ctx->stage_out, count * 4) != cudaSuccess) return GFP_ERR_NOMEM;
+        if (dev_malloc(&ctx->stage_out, count * 4) != cudaSuccess) return GFP_ERR_NOMEM;
         ctx->stage_out_elems = count;
     }
     uint32_t *dx = ctx->stage, *dy = ctx->stage + (total ? total : 1);
@@ -786,10 +786,10 @@ static gfp_status ensure_block_ws(gfp_ctx *ctx, uint64_t m, uint64_t k, uint64_t
         if (ctx->blk_ws) cudaFree(ctx->blk_ws);
         ctx->blk_ws = nullptr;
         ctx->blk_ws_bytes = ctx->blk_tail_bytes = 0;
-        if (cudaMalloc(&ctx->blk_ws, w + t) != cudaSuccess) {
+        if (dev_malloc(&ctx->blk_ws, w + t) != cudaSuccess) {
             w = ws;   // no room for both largest parts: this product's alone
             t = tail;
-            if (cudaMalloc(&ctx->blk_ws, w + t) != cudaSuccess) {
+            if (dev_malloc(&ctx->blk_ws, w + t) != cudaSuccess) {
                 ctx->blk_ws = nullptr;
                 return GFP_ERR_NOMEM;
             }
@@ -919,7 +919,7 @@ GFP_API gfp_status gfp_block_prepare(gfp_ctx *ctx, uint32_t p, uint64_t m, uint6
     gfp_block_prep *pp = new (std::nothrow) gfp_block_prep();
     if (!pp) return GFP_ERR_NOMEM;
     pp->per = block_prep_a_bytes(m, k);
-    if (cudaMalloc(&pp->mem, pp->per * passes) != cudaSuccess) {
+    if (dev_malloc(&pp->mem, pp->per * passes) != cudaSuccess) {
         delete pp;
         return GFP_ERR_NOMEM;
     }
@@ -1073,7 +1073,7 @@ GFP_API gfp_status gfp_matvec_sequence(gfp_ctx *ctx, uint32_t p, uint64_t n, con
         ctx->seq_cap = 0;
         const uint32_t cap = std::max<uint32_t>(iters + 1, 256);
         void *mem = nullptr;
-        if (cudaMalloc(&mem, (size_t)cap * 12) != cudaSuccess) return GFP_ERR_NOMEM;
+        if (dev_malloc(&mem, (size_t)cap * 12) != cudaSuccess) return GFP_ERR_NOMEM;
         GFP_CUDA_TRY(cudaMemset(mem, 0, (size_t)cap * 12));
         ctx->seq_slots = (unsigned long long *)mem;
         ctx->seq_tickets = (uint32_t *)((char *)mem + (size_t)cap * 8);
@@ -1084,7 +1084,7 @@ GFP_API gfp_status gfp_matvec_sequence(gfp_ctx *ctx, uint32_t p, uint64_t n, con
         if (ctx->pingpong) cudaFree(ctx->pingpong);
         ctx->pingpong = nullptr;
         ctx->pingpong_n = 0;
-        if (cudaMalloc(&ctx->pingpong, 2 * n * 4) != cudaSuccess) return GFP_ERR_NOMEM;
+        if (dev_malloc(&ctx->pingpong, 2 * n * 4) != cudaSuccess) return GFP_ERR_NOMEM;
         ctx->pingpong_n = 2 * n;
     }
     gfp_ctx::SeqKey key{p, n, A, lda, x0, u, seq, Y, iters, (int)r};

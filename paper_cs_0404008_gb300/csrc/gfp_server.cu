@@ -504,7 +504,7 @@ GFP_API gfp_status gfp_server_create(const gfp_server_cfg *cfg, gfp_server **out
     if (!s->cfg.simulate) {
         gfp_status stt = GFP_OK;
         if (cudaSetDevice(s->cfg.device) != cudaSuccess) stt = GFP_ERR_CUDA;
-        if (stt == GFP_OK && cudaMalloc(&s->base, s->cfg.mem_budget) != cudaSuccess) {
+        if (stt == GFP_OK && gfp::dev_malloc(&s->base, s->cfg.mem_budget) != cudaSuccess) {
             s->base = nullptr;
             stt = GFP_ERR_NOMEM;
         }
@@ -610,7 +610,7 @@ GFP_API gfp_status gfp_register_matrix(gfp_server *s, uint32_t p, uint64_t rows,
         M.ld = (cols + 3) / 4 * 4;
         void *mem = nullptr;
         if (cudaSetDevice(s->cfg.device) != cudaSuccess) return GFP_ERR_CUDA;
-        if (cudaMalloc(&mem, 4 * rows * M.ld) != cudaSuccess) return GFP_ERR_NOMEM;
+        if (gfp::dev_malloc(&mem, 4 * rows * M.ld) != cudaSuccess) return GFP_ERR_NOMEM;
         if (gfp::launch_fill_uniform_2d(p, seed, 0, rows, cols, M.ld, (uint32_t *)mem, nullptr) != cudaSuccess ||
             cudaDeviceSynchronize() != cudaSuccess) {
             cudaFree(mem);

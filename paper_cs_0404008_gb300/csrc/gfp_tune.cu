@@ -111,9 +111,9 @@ GFP_API gfp_status gfp_tune(gfp_ctx *ctx, const uint32_t *primes, uint32_t nprim
     // operand pool: 2 x 2^28 bytes (larger than L2, so each timing run is cold)
     const uint64_t pool_elems = 1ull << 26;
     DevBuf xb, yb, ob;
-    if (cudaMalloc(&xb.p, pool_elems * 4) != cudaSuccess) return GFP_ERR_NOMEM;
-    if (cudaMalloc(&yb.p, pool_elems * 4) != cudaSuccess) return GFP_ERR_NOMEM;
-    if (cudaMalloc(&ob.p, 1 << 20) != cudaSuccess) return GFP_ERR_NOMEM;
+    if (dev_malloc(&xb.p, pool_elems * 4) != cudaSuccess) return GFP_ERR_NOMEM;
+    if (dev_malloc(&yb.p, pool_elems * 4) != cudaSuccess) return GFP_ERR_NOMEM;
+    if (dev_malloc(&ob.p, 1 << 20) != cudaSuccess) return GFP_ERR_NOMEM;
     cudaStream_t s;
     if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) return GFP_ERR_CUDA;
     cudaEvent_t e0, e1;
