@@ -764,7 +764,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_block_tc(const __grid_constant__
 // low digits of output columns nt*64 + r, rows 64..127 the high digits.  One
 // pass over B serves every residue pass.
 struct PrepB {
-    uint32_t n;                        // moduli; one: B's entries are already below it
+    uint32_t n;                        // moduli
+    uint32_t reduce;                   // B's entries are not below them yet
     uint32_t p[RNS_MAX], magic[RNS_MAX];
 };
 constexpr int PREPB_THREADS = 256;
@@ -797,7 +798,7 @@ __global__ void __launch_bounds__(PREPB_THREADS)
             uint32_t u[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
-                const uint32_t b = pb.n > 1 ? reduce_small(v[i][e], p, pb.magic[l]) : v[i][e];
+                const uint32_t b = pb.reduce ? reduce_small(v[i][e], p, pb.magic[l]) : v[i][e];
                 u[e] = b + (b > half ? U_BIAS - p : U_BIAS);
             }
             uint4 h, lo;
@@ -1065,12 +1066,19 @@ size_t block_tc_workspace_bytes(uint64_t m, uint64_t nb)
     return 256 /* error flag */ + ((m * n_tiles * blk::NT * 4 + 255) & ~(size_t)255);
 }
 
-size_t block_tc_bimg_bytes(uint64_t k, uint64_t nb, int n_mod)
+size_t block_tc_bimg_bytes(uint64_t k, uint64_t nb, int at_once)
 {
-    const bool cut = k > blk::SLAB_K;   // residue passes then make their tiles one after the other
     const uint64_t kblocks = (std::min<uint64_t>(k, blk::SLAB_K) + blk::BK - 1) / blk::BK;
     const uint64_t n_tiles = (nb + blk::NT - 1) / blk::NT;
-    return n_tiles * kblocks * (uint64_t)blk::B_TILE_BYTES * (cut ? (n_mod > 1 ? 2 : 1) : n_mod);
+    return n_tiles * kblocks * (uint64_t)blk::B_TILE_BYTES * at_once;
+}
+
+// One launch for all of them saves the others' (4.7 us each) and their reads of B,
+// next to nothing once B is large; what B's tiles may take is bounded by it.
+int block_tc_moduli_at_once(uint64_t k, uint64_t nb, int n_mod)
+{
+    constexpr size_t TILES_MAX = (size_t)1 << 30;
+    return k <= blk::SLAB_K && block_tc_bimg_bytes(k, nb, n_mod) <= TILES_MAX ? n_mod : 1;
 }
 
 size_t block_prep_a_bytes(uint64_t m, uint64_t k)
@@ -1175,9 +1183,8 @@ cudaError_t launch_block_tc(const uint32_t *mods, int n_mod, uint64_t m, uint64_
     bcfg.numAttrs = cfg.numAttrs = fcfg.numAttrs = 1;
     PrepB pb;
     memset(&pb, 0, sizeof pb);
-    for (int l0 = 0; l0 < n_mod; l0 += k > SLAB_K ? 1 : n_mod) {
-        // all moduli of a product in one launch set; one at a time where K is cut
-        const int l1 = k > SLAB_K ? l0 + 1 : n_mod;
+    for (int l0 = 0; l0 < n_mod; l0 += sc.at_once) {
+        const int l1 = std::min(n_mod, l0 + sc.at_once);
         for (uint64_t k0 = 0; k0 < k; k0 += SLAB_K) {
             a.k = std::min<uint64_t>(SLAB_K, k - k0);
             const bool last = k - k0 <= SLAB_K;
@@ -1194,14 +1201,10 @@ cudaError_t launch_block_tc(const uint32_t *mods, int n_mod, uint64_t m, uint64_
             a.direct = a.ranges == 1 && k <= SLAB_K ? 1 : 0;
             const uint32_t btiles = a.n_tiles * a.kblocks;
             pb.n = (uint32_t)(l1 - l0);
+            pb.reduce = reduce ? 1 : 0;
             for (int l = l0; l < l1; ++l) {
                 pb.p[l - l0] = mods[l];
                 pb.magic[l - l0] = (uint32_t)((1ull << 32) / mods[l]);
-            }
-            if (reduce && pb.n == 1) {   // the tiles of one residue modulus still need the reduction
-                pb.n = 2;
-                pb.p[1] = pb.p[0];
-                pb.magic[1] = pb.magic[0];
             }
             bcfg.gridDim = dim3(btiles);
             cudaError_t e = cudaLaunchKernelEx(&bcfg, k_block_prep_b, B + k0 * ldb, ldb, a.k, nb, a.kblocks, pb,

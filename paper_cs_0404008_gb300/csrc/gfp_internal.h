@@ -164,10 +164,15 @@ cudaError_t launch_block_crt(const uint32_t *R, uint64_t m, uint64_t nb, uint32_
                              const RnsConst &rc, int sm_count, cudaStream_t s);
 // error flag and partial sums; all zero at launch, and again after it
 size_t block_tc_workspace_bytes(uint64_t m, uint64_t nb);
-size_t block_tc_bimg_bytes(uint64_t k, uint64_t nb, int n_mod);
+// B's digit tiles for at_once moduli
+size_t block_tc_bimg_bytes(uint64_t k, uint64_t nb, int at_once);
+// Moduli whose tiles of B are made by one launch: all, or one where K is cut into
+// several launches or the tiles of all would be too large.
+int block_tc_moduli_at_once(uint64_t k, uint64_t nb, int n_mod);
 struct BlockScratch {
     void *ws;        // block_tc_workspace_bytes, zero; the error flag is its first word
     uint8_t *bimg;   // block_tc_bimg_bytes: B's digit tiles
+    int at_once;     // moduli whose tiles bimg holds: as many as above, or one
 };
 // n_mod = 1: C = A B mod mods[0].  More: the residue passes, A and B reduced
 // modulo each; pass l writes the dense m x nb matrix C + l m nb (ldc = nb).

@@ -770,37 +770,60 @@ static int block_sms(const gfp_ctx *ctx)
     return (ctx->blk_sms > 0 && ctx->blk_sms < ctx->sm_count) ? ctx->blk_sms : ctx->sm_count;
 }
 
-// Block-product buffer of the context for an m x k by k x nb product with n_mod
-// moduli: the workspace (zero outside calls), then B's digit tiles and, where
-// there are several moduli, the residue matrices.  One allocation, grown on
-// demand to the largest of either part, so that no shape's tiles reach into
-// another's workspace; the caller holds ctx->mu.
+// Sizes of the two parts of a block product's scratch: the workspace, and behind
+// it B's digit tiles for at_once moduli with, where there are several moduli, the
+// residue matrices.
+struct BlockParts {
+    size_t ws, img, tail;
+    BlockParts(uint64_t m, uint64_t k, uint64_t nb, int n_mod, int at_once)
+    {
+        ws = align256(block_tc_workspace_bytes(m, nb));
+        img = align256(block_tc_bimg_bytes(k, nb, at_once));
+        tail = img + (n_mod > 1 ? align256((size_t)n_mod * m * nb * 4) : 0);
+    }
+    bool fit(size_t w, size_t t) const { return ws <= w && tail <= t; }
+};
+
+// Block-product buffer of the context: the workspace (zero outside calls), then
+// the rest.  One allocation, grown on demand to the largest of either part, so
+// that no shape's tiles reach into another's workspace; to this product's own
+// parts, and its tiles for one modulus, where there is no room for more.  The caller
+// holds ctx->mu.
 static gfp_status ensure_block_ws(gfp_ctx *ctx, uint64_t m, uint64_t k, uint64_t nb, int n_mod, cudaStream_t s,
                                   BlockScratch *sc, uint32_t **res)
 {
-    const size_t ws = align256(block_tc_workspace_bytes(m, nb)), img = align256(block_tc_bimg_bytes(k, nb, n_mod));
-    const size_t tail = img + (n_mod > 1 ? align256((size_t)n_mod * m * nb * 4) : 0);
-    if (ws > ctx->blk_ws_bytes || tail > ctx->blk_tail_bytes) {
+    sc->at_once = block_tc_moduli_at_once(k, nb, n_mod);
+    BlockParts need(m, k, nb, n_mod, sc->at_once);
+    const BlockParts least(m, k, nb, n_mod, 1);
+    if (!need.fit(ctx->blk_ws_bytes, ctx->blk_tail_bytes) && least.fit(ctx->blk_ws_bytes, ctx->blk_tail_bytes)) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        GFP_CUDA_TRY(cudaStreamIsCapturing(s, &cap));
+        if (cap != cudaStreamCaptureStatusNone) {   // nothing can grow now
+            sc->at_once = 1;
+            need = least;
+        }
+    }
+    if (!need.fit(ctx->blk_ws_bytes, ctx->blk_tail_bytes)) {
         GFP_CUDA_TRY(cudaDeviceSynchronize());   // work in flight may still use the old one
-        size_t w = std::max(ws, ctx->blk_ws_bytes), t = std::max(tail, ctx->blk_tail_bytes);
+        size_t w = std::max(need.ws, ctx->blk_ws_bytes), t = std::max(need.tail, ctx->blk_tail_bytes);
         if (ctx->blk_ws) cudaFree(ctx->blk_ws);
         ctx->blk_ws = nullptr;
         ctx->blk_ws_bytes = ctx->blk_tail_bytes = 0;
-        if (dev_malloc(&ctx->blk_ws, w + t) != cudaSuccess) {
-            w = ws;   // no room for both largest parts: this product's alone
-            t = tail;
-            if (dev_malloc(&ctx->blk_ws, w + t) != cudaSuccess) {
-                ctx->blk_ws = nullptr;
-                return GFP_ERR_NOMEM;
-            }
+        cudaError_t e = dev_malloc(&ctx->blk_ws, w + t);
+        if (e != cudaSuccess) e = dev_malloc(&ctx->blk_ws, (w = need.ws) + (t = need.tail));
+        if (e != cudaSuccess && sc->at_once > 1) {
+            sc->at_once = 1;
+            need = least;
+            e = dev_malloc(&ctx->blk_ws, (w = need.ws) + (t = need.tail));
         }
+        if (e != cudaSuccess) return GFP_ERR_NOMEM;
         GFP_CUDA_TRY(cudaMemsetAsync(ctx->blk_ws, 0, w, s));
         ctx->blk_ws_bytes = w;
         ctx->blk_tail_bytes = t;
     }
     sc->ws = ctx->blk_ws;
     sc->bimg = (uint8_t *)ctx->blk_ws + ctx->blk_ws_bytes;
-    *res = (uint32_t *)(sc->bimg + img);
+    *res = (uint32_t *)(sc->bimg + need.img);
     return GFP_OK;
 }
 

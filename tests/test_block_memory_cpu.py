@@ -11,7 +11,7 @@ def test_smaller_buffer_after_a_failed_allocation(lib):
 c = context()
 assert block(c, {p}, 64, 4194304, 64) == 0                  # large tiles of B
 assert F.fake_used() > 1 << 30
-F.fake_room(F.fake_used() + (64 << 20))
+F.fake_room(F.fake_used() + (900 << 20))
 F.fake_events()
 assert block(c, {p}, 1 << 22, 1024, 8) == 0                 # large workspace: the two together do not fit
 ks = kernels()
@@ -33,4 +33,43 @@ for _ in range(2):
     assert L.gfp_block_prepare(c, 65521, 1 << 20, 512, A, 512, ctypes.byref(out)) == g.GFP_ERR_NOMEM
     assert L.gfp_dot(c, 65521, 1024, A, B, C, 0) == 0
     assert L.gfp_matvec(c, 65521, 1024, 1024, A, 1024, B, C, 0) == 0
+""")
+
+
+def test_tiles_of_b_for_one_modulus_where_all_would_be_too_large(lib):
+    """The digit tiles of B take 4 bytes an entry and modulus: those of all moduli
+    are made at once up to 1 GiB, and one modulus at a time above that or where
+    there is no room."""
+    fake_cuda.run("""
+p = 2147483647
+c = context()
+base = F.fake_used()
+# small: one launch for all moduli
+assert block(c, p, 512, 8192, 64) == 0
+ks = kernels()
+passes = count(ks, "k_block_tc")
+assert passes >= 5 and count(ks, "k_block_prep_b") == 1 and count(ks, "k_block_crt") == 1
+# 16384 x 8192: 512 MiB a modulus
+assert block(c, p, 512, 16384, 8192) == 0
+ks = kernels()
+assert count(ks, "k_block_tc") == count(ks, "k_block_prep_b") == passes, ks
+tiles, sums = 4 * 16384 * 8192, 4 * 512 * 8192
+assert F.fake_used() - base < 1.01 * (tiles + (passes + 1) * sums)
+# no room for the tiles of all: the product still runs
+assert L.gfp_context_destroy(c) == 0
+c = context()
+tiles, sums = 4 * 16384 * 1024, 4 * 512 * 1024
+F.fake_room(F.fake_used() + int(1.01 * (tiles + (passes + 1) * sums)))
+F.fake_events()
+assert block(c, p, 512, 16384, 1024) == 0
+ks = kernels()
+assert count(ks, "k_block_tc") == count(ks, "k_block_prep_b") == passes and ks[-1].startswith("k_block_crt"), ks
+# under capture the tiles that fit are used, nothing is allocated
+F.fake_room(1 << 40)
+F.fake_capture(1)
+assert block(c, p, 512, 16384, 1024, stream=CAPTURING) == 0
+assert count(kernels(), "k_block_prep_b") == passes
+F.fake_capture(0)
+assert block(c, p, 512, 16384, 1024) == 0                   # room again: all at once
+assert count(kernels(), "k_block_prep_b") == 1
 """)
