@@ -272,10 +272,17 @@ GFP_API gfp_status gfp_matvec_sequence(gfp_ctx *ctx, uint32_t p, uint64_t n, con
  * loads.  Otherwise the CUDA-core kernel with the
  * representation forced on the context, else the built-in rule for p (tuned
  * plans time the dot-product kernels and do not apply here; forcing F16TC
- * where the tensor cores are not eligible gives GFP_ERR_UNSUPPORTED).  The tensor-core path
+ * where the tensor cores are not eligible gives GFP_ERR_UNSUPPORTED).
+ * Scratch: the tensor-core path
  * uses the context's workspace (grown on demand, so call once outside stream
  * capture for the largest shape) and must not run concurrently with another
- * block product of the same context.  k == 0 writes zeros. */
+ * block product of the same context.  Exempt from this, with GFP_REPR_AUTO, are rows
+ * of A at other alignments, and products over p > 65791 with m k nb / 4.5e12 <=
+ * L (25e-6 + m k / 1e12): they take their scratch from a stream-ordered pool, may
+ * run on several streams of one context at once and be captured without a call
+ * before; captured, and where the pool has no memory, they run on the CUDA cores,
+ * which need none (and are far slower: pad the rows of A to 16 bytes for the tensor
+ * cores in a graph).  k == 0 writes zeros. */
 GFP_API gfp_status gfp_matmul_block(gfp_ctx *ctx, uint32_t p, uint64_t m, uint64_t k, uint64_t nb,
                                     const uint32_t *A, uint64_t lda, const uint32_t *B,
                                     uint64_t ldb, uint32_t *C, uint64_t ldc, void *stream);

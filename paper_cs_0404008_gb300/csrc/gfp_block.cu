@@ -767,6 +767,8 @@ struct PrepB {
     uint32_t n;                        // moduli
     uint32_t reduce;                   // B's entries are not below them yet
     uint32_t p[RNS_MAX], magic[RNS_MAX];
+    uint4 *clear;                      // scratch that is to be zero for the product (or none)
+    uint64_t clear_n;
 };
 constexpr int PREPB_THREADS = 256;
 __global__ void __launch_bounds__(PREPB_THREADS)
@@ -789,6 +791,9 @@ __global__ void __launch_bounds__(PREPB_THREADS)
 #pragma unroll
         for (int e = 0; e < 8; ++e) v[i][e] = (col < nb && k0 + e < k) ? __ldg(B + (k0 + e) * ldb + col) : 0u;
     }
+    for (uint64_t i = (uint64_t)blockIdx.x * PREPB_THREADS + threadIdx.x; i < pb.clear_n;
+         i += (uint64_t)gridDim.x * PREPB_THREADS)
+        pb.clear[i] = make_uint4(0u, 0u, 0u, 0u);
     for (uint32_t l = 0; l < pb.n; ++l) {
         const uint32_t p = pb.p[l], half = (p - 1) / 2;
         uint8_t *out = img + ((uint64_t)l * gridDim.x + tile) * B_TILE_BYTES;
@@ -1063,7 +1068,7 @@ bool block_rns_plan(uint32_t p, uint64_t k, RnsConst *rc)
 size_t block_tc_workspace_bytes(uint64_t m, uint64_t nb)
 {
     const uint64_t n_tiles = (nb + blk::NT - 1) / blk::NT;
-    return 256 /* error flag */ + ((m * n_tiles * blk::NT * 4 + 255) & ~(size_t)255);
+    return (m * n_tiles * blk::NT * 4 + 255) & ~(size_t)255;
 }
 
 size_t block_tc_bimg_bytes(uint64_t k, uint64_t nb, int at_once)
@@ -1156,15 +1161,16 @@ cudaError_t launch_block_tc(const uint32_t *mods, int n_mod, uint64_t m, uint64_
     // prepared digits: 16-byte aligned tiles of a device allocation
     if (Aimg && (((uintptr_t)Aimg) & 15u)) return cudaErrorInvalidValue;
     const Kernel kernel = Aimg ? kernels[4] : kernels[(block_tc_layout_ok(A, lda) ? 0 : 2) + (reduce ? 1 : 0)];
-    if ((nb + NT - 1) / NT > 65535) return cudaErrorInvalidValue;   // grid y of the finishing kernel
+    static_assert(BLOCK_TC_MAX_NB == 65535ull * NT, "grid y of the finishing kernel");
+    if (nb > BLOCK_TC_MAX_NB) return cudaErrorInvalidValue;
     Args a;
     memset(&a, 0, sizeof a);
     a.m = m;
     a.nb = nb;
     a.lda = lda;
     a.img_kblocks = (uint32_t)((k + BK - 1) / BK);
-    a.err = (uint32_t *)sc.ws;
-    a.Cacc = (uint32_t *)((uint8_t *)sc.ws + 256);
+    a.err = sc.err;
+    a.Cacc = (uint32_t *)sc.ws;
     a.n_tiles = (uint32_t)((nb + NT - 1) / NT);
     a.m_tiles = (uint32_t)((m + BM - 1) / BM);
     a.edge_m = m % BM ? a.m_tiles - 1 : ~0u;
@@ -1183,6 +1189,7 @@ cudaError_t launch_block_tc(const uint32_t *mods, int n_mod, uint64_t m, uint64_
     bcfg.numAttrs = cfg.numAttrs = fcfg.numAttrs = 1;
     PrepB pb;
     memset(&pb, 0, sizeof pb);
+    bool dirty = sc.dirty;
     for (int l0 = 0; l0 < n_mod; l0 += sc.at_once) {
         const int l1 = std::min(n_mod, l0 + sc.at_once);
         for (uint64_t k0 = 0; k0 < k; k0 += SLAB_K) {
@@ -1206,6 +1213,9 @@ cudaError_t launch_block_tc(const uint32_t *mods, int n_mod, uint64_t m, uint64_
                 pb.p[l - l0] = mods[l];
                 pb.magic[l - l0] = (uint32_t)((1ull << 32) / mods[l]);
             }
+            pb.clear = dirty && !a.direct ? (uint4 *)sc.ws : nullptr;
+            pb.clear_n = pb.clear ? block_tc_workspace_bytes(m, nb) / 16 : 0;
+            dirty = false;
             bcfg.gridDim = dim3(btiles);
             cudaError_t e = cudaLaunchKernelEx(&bcfg, k_block_prep_b, B + k0 * ldb, ldb, a.k, nb, a.kblocks, pb,
                                                sc.bimg);

@@ -139,6 +139,8 @@ cudaError_t launch_matvec(Repr r, const Mod &m, uint64_t k, uint64_t rows, uint6
 // Block product (gfp_block.cu).  The tensor-core path needs the centred
 // residues to fit two balanced 8-bit digits: (p-1)/2 <= 32895.
 constexpr uint32_t BLOCK_TC_MAX_P = 65791;
+// Columns of a tensor-core product at most (grid y of the finishing kernel).
+constexpr uint64_t BLOCK_TC_MAX_NB = 65535ull * 64;
 // Moduli of the residue passes, and of prepared operands taken directly: at
 // most 65536, so that every residue has two 8-bit balanced digits.
 constexpr uint32_t RNS_PRIME_MAX = 65536;
@@ -162,7 +164,7 @@ struct RnsConst {
 bool block_rns_plan(uint32_t p, uint64_t k, RnsConst *rc);
 cudaError_t launch_block_crt(const uint32_t *R, uint64_t m, uint64_t nb, uint32_t *C, uint64_t ldc,
                              const RnsConst &rc, int sm_count, cudaStream_t s);
-// error flag and partial sums; all zero at launch, and again after it
+// partial sums; all zero at launch, and again after it
 size_t block_tc_workspace_bytes(uint64_t m, uint64_t nb);
 // B's digit tiles for at_once moduli
 size_t block_tc_bimg_bytes(uint64_t k, uint64_t nb, int at_once);
@@ -170,7 +172,9 @@ size_t block_tc_bimg_bytes(uint64_t k, uint64_t nb, int at_once);
 // several launches or the tiles of all would be too large.
 int block_tc_moduli_at_once(uint64_t k, uint64_t nb, int n_mod);
 struct BlockScratch {
-    void *ws;        // block_tc_workspace_bytes, zero; the error flag is its first word
+    uint32_t *err;   // bit 0: a bounded wait expired
+    void *ws;        // block_tc_workspace_bytes
+    bool dirty;      // ws is not zero yet: the first kernel clears it
     uint8_t *bimg;   // block_tc_bimg_bytes: B's digit tiles
     int at_once;     // moduli whose tiles bimg holds: as many as above, or one
 };
@@ -239,11 +243,15 @@ struct gfp_ctx {
     uint32_t *stage_out = nullptr;
     size_t stage_out_elems = 0;
 
-    // block-product buffer: error flag and partial sums (by pairs of columns),
-    // zero outside calls; behind them B's digit tiles and the residue matrices of
-    // the passes of a large modulus; grown on demand
+    // block-product buffer: partial sums (by pairs of columns), zero outside calls;
+    // behind them B's digit tiles and the residue matrices of the passes of a large
+    // modulus; grown on demand
     void *blk_ws = nullptr;
     size_t blk_ws_bytes = 0, blk_tail_bytes = 0;   // sizes of the two parts
+    uint32_t *blk_err = nullptr;                   // error word of all block products
+    // stream-ordered scratch of the block products that keep none in the context
+    cudaMemPool_t blk_pool = nullptr;
+    bool blk_pool_tried = false;
 
     // tuned plan: (p, lg_n) -> entry
     std::map<std::pair<uint32_t, uint32_t>, gfp_plan_entry> plan;

@@ -423,6 +423,7 @@ GFP_API gfp_status gfp_context_create(int device, gfp_ctx **out)
     cudaMemset(mem, 0, ring_bytes + 256);
     c->ring_slots = (unsigned long long *)mem;
     c->d_flag = (uint32_t *)((char *)mem + ring_bytes);
+    c->blk_err = (uint32_t *)((char *)mem + ring_bytes + 128);
     if (cudaDeviceSynchronize() != cudaSuccess) {
         cudaFree(mem);
         delete c;
@@ -457,6 +458,7 @@ GFP_API gfp_status gfp_context_destroy(gfp_ctx *ctx)
     if (ctx->stage) cudaFree(ctx->stage);
     if (ctx->stage_out) cudaFree(ctx->stage_out);
     if (ctx->blk_ws) cudaFree(ctx->blk_ws);
+    if (ctx->blk_pool) cudaMemPoolDestroy(ctx->blk_pool);
     delete ctx;
     return GFP_OK;
 }
@@ -784,6 +786,17 @@ struct BlockParts {
     bool fit(size_t w, size_t t) const { return ws <= w && tail <= t; }
 };
 
+// The stream is being captured, or cannot be asked because another one is.
+static bool is_capturing(cudaStream_t s)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return true;
+    }
+    return cap != cudaStreamCaptureStatusNone;
+}
+
 // Block-product buffer of the context: the workspace (zero outside calls), then
 // the rest.  One allocation, grown on demand to the largest of either part, so
 // that no shape's tiles reach into another's workspace; to this product's own
@@ -796,9 +809,7 @@ static gfp_status ensure_block_ws(gfp_ctx *ctx, uint64_t m, uint64_t k, uint64_t
     BlockParts need(m, k, nb, n_mod, sc->at_once);
     const BlockParts least(m, k, nb, n_mod, 1);
     if (!need.fit(ctx->blk_ws_bytes, ctx->blk_tail_bytes) && least.fit(ctx->blk_ws_bytes, ctx->blk_tail_bytes)) {
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        GFP_CUDA_TRY(cudaStreamIsCapturing(s, &cap));
-        if (cap != cudaStreamCaptureStatusNone) {   // nothing can grow now
+        if (is_capturing(s)) {   // nothing can grow now
             sc->at_once = 1;
             need = least;
         }
@@ -821,33 +832,118 @@ static gfp_status ensure_block_ws(gfp_ctx *ctx, uint64_t m, uint64_t k, uint64_t
         ctx->blk_ws_bytes = w;
         ctx->blk_tail_bytes = t;
     }
+    sc->err = ctx->blk_err;
     sc->ws = ctx->blk_ws;
+    sc->dirty = false;
     sc->bimg = (uint8_t *)ctx->blk_ws + ctx->blk_ws_bytes;
     *res = (uint32_t *)(sc->bimg + need.img);
     return GFP_OK;
 }
 
-// The tensor-core product through the context's buffers: one modulus directly,
-// several as residue passes recombined modulo rc.p.
-static gfp_status run_block_tc(gfp_ctx *ctx, uint32_t p, const RnsConst *rc, uint64_t m, uint64_t k, uint64_t nb,
-                               const uint32_t *A, uint64_t lda, const uint32_t *B, uint64_t ldb, uint32_t *C,
-                               uint64_t ldc, const uint8_t *Aimg, size_t img_bytes, cudaStream_t s)
+// One tensor-core product.
+struct BlockCall {
+    uint32_t p;
+    const RnsConst *rc;      // several residue passes recombined modulo p, or null: p directly
+    uint64_t m, k, nb;
+    const uint32_t *A;
+    uint64_t lda;
+    const uint32_t *B;
+    uint64_t ldb;
+    uint32_t *C;
+    uint64_t ldc;
+    const uint8_t *Aimg;     // prepared A (A and lda then unused)
+    size_t img_bytes;
+    int n_mod() const { return rc ? rc->L : 1; }
+};
+
+// Products over a large modulus small enough to be among the calls that need
+// nothing of the context: by the rule, L residue passes at 25 us and 4 TB/s would
+// not be faster than CUDA cores at 4.5e12 terms a second.
+static bool block_small_large_modulus(int L, uint64_t m, uint64_t k, uint64_t nb)
 {
-    std::lock_guard<std::mutex> g(ctx->mu);
-    const int n_mod = rc ? rc->L : 1;
-    BlockScratch sc;
-    uint32_t *R;
-    const gfp_status st = ensure_block_ws(ctx, m, k, nb, n_mod, s, &sc, &R);
-    if (st != GFP_OK) return st;
+    const double mk = (double)m * (double)k;
+    return mk * (double)nb / 4.5e12 <= L * (25e-6 + 4.0 * mk / 4.0e12);
+}
+
+static gfp_status launch_block(gfp_ctx *ctx, const BlockCall &q, const BlockScratch &sc, uint32_t *R, cudaStream_t s)
+{
+    const bool many = q.n_mod() > 1;
     int launches = 0;
-    GFP_CUDA_TRY(launch_block_tc(rc ? rc->mod : &p, n_mod, m, k, nb, A, lda, B, ldb, n_mod > 1 ? R : C,
-                                 n_mod > 1 ? nb : ldc, sc, block_sms(ctx), s, &launches, Aimg, img_bytes));
-    if (n_mod > 1) {
-        GFP_CUDA_TRY(launch_block_crt(R, m, nb, C, ldc, *rc, ctx->sm_count, s));
+    GFP_CUDA_TRY(launch_block_tc(q.rc ? q.rc->mod : &q.p, q.n_mod(), q.m, q.k, q.nb, q.A, q.lda, q.B, q.ldb,
+                                 many ? R : q.C, many ? q.nb : q.ldc, sc, block_sms(ctx), s, &launches, q.Aimg,
+                                 q.img_bytes));
+    if (many) {
+        GFP_CUDA_TRY(launch_block_crt(R, q.m, q.nb, q.C, q.ldc, *q.rc, ctx->sm_count, s));
         ++launches;
     }
     ctx->launches += launches;
     return GFP_OK;
+}
+
+// The product through the context's buffer.
+static gfp_status run_block_tc(gfp_ctx *ctx, const BlockCall &q, cudaStream_t s)
+{
+    std::lock_guard<std::mutex> g(ctx->mu);
+    BlockScratch sc;
+    uint32_t *R;
+    const gfp_status st = ensure_block_ws(ctx, q.m, q.k, q.nb, q.n_mod(), s, &sc, &R);
+    return st == GFP_OK ? launch_block(ctx, q, sc, R, s) : st;
+}
+
+// Pool of the stream-ordered scratch: keeps up to 256 MiB between calls, makes no
+// stream wait for another.  Null where it cannot be had.
+static cudaMemPool_t block_pool(gfp_ctx *ctx)
+{
+    std::lock_guard<std::mutex> g(ctx->mu);
+    if (ctx->blk_pool_tried) return ctx->blk_pool;
+    ctx->blk_pool_tried = true;
+    int has = 0;
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = ctx->device;
+    cudaMemPool_t pool = nullptr;
+    if (cudaDeviceGetAttribute(&has, cudaDevAttrMemoryPoolsSupported, ctx->device) != cudaSuccess || !has ||
+        cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return nullptr;
+    }
+    uint64_t keep = 256ull << 20;
+    int no = 0;
+    if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess ||
+        cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowInternalDependencies, &no) != cudaSuccess) {
+        (void)cudaGetLastError();
+        cudaMemPoolDestroy(pool);
+        return nullptr;
+    }
+    return ctx->blk_pool = pool;
+}
+
+// The product with scratch of its own, allocated and freed in stream order: calls
+// on several streams do not meet.  GFP_ERR_NOMEM, with nothing launched, where there
+// is none.
+static gfp_status run_block_tc_pool(gfp_ctx *ctx, const BlockCall &q, cudaStream_t s)
+{
+    const cudaMemPool_t pool = block_pool(ctx);
+    if (!pool) return GFP_ERR_NOMEM;
+    BlockScratch sc;
+    sc.at_once = block_tc_moduli_at_once(q.k, q.nb, q.n_mod());
+    void *mem = nullptr;
+    for (;;) {
+        const BlockParts need(q.m, q.k, q.nb, q.n_mod(), sc.at_once);
+        if (cudaMallocFromPoolAsync(&mem, need.ws + need.tail, pool, s) == cudaSuccess) {
+            sc.err = ctx->blk_err;
+            sc.ws = mem;
+            sc.dirty = true;
+            sc.bimg = (uint8_t *)mem + need.ws;
+            const gfp_status st = launch_block(ctx, q, sc, (uint32_t *)(sc.bimg + need.img), s);
+            GFP_CUDA_TRY(cudaFreeAsync(mem, s));
+            return st;
+        }
+        (void)cudaGetLastError();
+        if (sc.at_once == 1) return GFP_ERR_NOMEM;
+        sc.at_once = 1;
+    }
 }
 
 GFP_API gfp_status gfp_matmul_block(gfp_ctx *ctx, uint32_t p, uint64_t m, uint64_t k, uint64_t nb,
@@ -868,7 +964,11 @@ GFP_API gfp_status gfp_matmul_block(gfp_ctx *ctx, uint32_t p, uint64_t m, uint64
     // primes (one pass each, then a Garner recombination) above that.  Forcing
     // them asks for a layout that 16-byte loads take; the automatic choice also
     // uses them for other layouts, with 4-byte loads
-    const bool layout_ok = ctx->forced == GFP_REPR_AUTO || block_tc_layout_ok(A, lda);
+    const bool vec_ok = block_tc_layout_ok(A, lda);
+    // A call that promises its caller to need nothing of the context (header):
+    // several streams may be in it at once, and it may be captured at any time
+    bool own_scratch = ctx->forced == GFP_REPR_AUTO && !vec_ok;
+    const bool layout_ok = ctx->forced == GFP_REPR_AUTO || vec_ok;
     RnsConst rc;
     const bool direct_ok = layout_ok && p <= BLOCK_TC_MAX_P;
     bool rns_ok = layout_ok && p > BLOCK_TC_MAX_P && block_rns_plan(p, k, &rc);
@@ -884,15 +984,15 @@ GFP_API gfp_status gfp_matmul_block(gfp_ctx *ctx, uint32_t p, uint64_t m, uint64
         const double t_rns = 5e-6 + rc.L * (10e-6 + (4.0 * (double)m * (double)k + 16.0 * (double)m * (double)nb) / 4.5e12);
         const double t_cc = 7e-6 + (double)k * 0.134e-6 * std::max(1.0, ctas / ctx->sm_count);
         if (t_cc <= t_rns) rns_ok = false;
+        if (block_small_large_modulus(rc.L, m, k, nb)) own_scratch = true;
     }
-    const bool tc_ok = direct_ok || rns_ok;
-    bool use_tc = false;
+    // such a call takes the tensor cores with scratch from a pool, else (a captured
+    // one must not share scratch with the calls beside its replays; no memory) the
+    // CUDA cores, which need none: 3001 x 5003 x 40 24 and 2236 us
+    const bool tc_ok = (direct_ok || rns_ok) && !(own_scratch && (nb > BLOCK_TC_MAX_NB || is_capturing(s)));
     Repr r = U64_CARRY;
     if (ctx->forced == GFP_REPR_F16TC) {
         if (!tc_ok) return GFP_ERR_UNSUPPORTED;
-        use_tc = true;
-    } else if (ctx->forced == GFP_REPR_AUTO && tc_ok) {
-        use_tc = true;
     } else if (!resolve_repr_untuned(ctx, p, &r)) {
         return GFP_ERR_UNSUPPORTED;
     }
@@ -901,13 +1001,16 @@ GFP_API gfp_status gfp_matmul_block(gfp_ctx *ctx, uint32_t p, uint64_t m, uint64
         if (st == GFP_OK) st = check_range_rows(ctx, B, k, nb, ldb, p, s);
         if (st != GFP_OK) return st;
     }
-    const Mod mod = make_mod(p);
-    if (!use_tc) {
-        GFP_CUDA_TRY(launch_block_cc(r, mod, k_for(r, p), m, k, nb, A, lda, B, ldb, C, ldc, s));
-        ctx->launches++;
-        return GFP_OK;
+    if (tc_ok && (ctx->forced == GFP_REPR_F16TC || ctx->forced == GFP_REPR_AUTO)) {
+        const BlockCall q{p, rns_ok ? &rc : nullptr, m, k, nb, A, lda, B, ldb, C, ldc, nullptr, 0};
+        if (!own_scratch) return run_block_tc(ctx, q, s);
+        const gfp_status st = run_block_tc_pool(ctx, q, s);
+        if (st != GFP_ERR_NOMEM) return st;
     }
-    return run_block_tc(ctx, p, rns_ok ? &rc : nullptr, m, k, nb, A, lda, B, ldb, C, ldc, nullptr, 0, s);
+    const Mod mod = make_mod(p);
+    GFP_CUDA_TRY(launch_block_cc(r, mod, k_for(r, p), m, k, nb, A, lda, B, ldb, C, ldc, s));
+    ctx->launches++;
+    return GFP_OK;
 }
 
 // A prepared once for repeated block products: its tensor-core digit
@@ -1000,8 +1103,8 @@ GFP_API gfp_status gfp_matmul_block_prepared(gfp_ctx *ctx, const gfp_block_prep 
         const gfp_status st = check_range_rows(ctx, B, k, nb, ldb, pp->p, s);
         if (st != GFP_OK) return st;
     }
-    return run_block_tc(ctx, pp->p, pp->passes > 1 ? &pp->rc : nullptr, m, k, nb, nullptr, 0, B, ldb, C, ldc,
-                        (const uint8_t *)pp->mem, pp->per, s);
+    return run_block_tc(ctx, BlockCall{pp->p, pp->passes > 1 ? &pp->rc : nullptr, m, k, nb, nullptr, 0, B, ldb, C, ldc,
+                                       (const uint8_t *)pp->mem, pp->per}, s);
 }
 
 GFP_API gfp_status gfp_matmul_block_csr(gfp_ctx *ctx, uint32_t p, uint64_t m, uint64_t k,
@@ -1052,11 +1155,11 @@ GFP_API gfp_status gfp_context_check(gfp_ctx *ctx)
     if (cudaDeviceSynchronize() != cudaSuccess) return GFP_ERR_CUDA;
     // device-side checks (GFP_DEVICE_CHECKS builds; always 0 otherwise)
     const uint32_t dbits = csr_check_bits() | dot_check_bits();
-    if (!ctx->blk_ws) return dbits ? GFP_ERR_INVALID : GFP_OK;
     uint32_t h = 0;
-    GFP_CUDA_TRY(cudaMemcpy(&h, ctx->blk_ws, 4, cudaMemcpyDeviceToHost));   // the error flag
+    GFP_CUDA_TRY(cudaMemcpy(&h, ctx->blk_err, 4, cudaMemcpyDeviceToHost));
     if (h) {
-        GFP_CUDA_TRY(cudaMemset(ctx->blk_ws, 0, ctx->blk_ws_bytes));
+        GFP_CUDA_TRY(cudaMemset(ctx->blk_err, 0, 4));
+        if (ctx->blk_ws) GFP_CUDA_TRY(cudaMemset(ctx->blk_ws, 0, ctx->blk_ws_bytes));
         return GFP_ERR_TIMEOUT;
     }
     return dbits ? GFP_ERR_INVALID : GFP_OK;

@@ -9,6 +9,7 @@ def test_smaller_buffer_after_a_failed_allocation(lib):
     for p, last in ((65521, "k_block_finish"), (2147483647, "k_block_crt")):
         fake_cuda.run(f"""
 c = context()
+assert L.gfp_set_repr(c, g.GFP_REPR_F16TC) == 0             # the context's buffer for all of them
 assert block(c, {p}, 64, 4194304, 64) == 0                  # large tiles of B
 assert F.fake_used() > 1 << 30
 F.fake_room(F.fake_used() + (900 << 20))
@@ -72,4 +73,74 @@ assert count(kernels(), "k_block_prep_b") == passes
 F.fake_capture(0)
 assert block(c, p, 512, 16384, 1024) == 0                   # room again: all at once
 assert count(kernels(), "k_block_prep_b") == 1
+""")
+
+
+# rows of A that 16-byte loads cannot take (both widths of modulus), and a small
+# product over a large modulus: calls that need nothing of the context
+FREE = [(65521, 3001, 5003, 40), (2147483647, 3001, 5003, 40), (2147483647, 1024, 1024, 64)]
+
+
+def test_free_calls_run_under_capture_without_a_call_before(lib):
+    fake_cuda.run(f"""
+c = context()
+base = F.fake_used()
+F.fake_capture(1)
+for p, m, k, nb in {FREE}:
+    F.fake_events()
+    assert block(c, p, m, k, nb, stream=CAPTURING) == 0, (p, m, k, nb)
+    ks = kernels()
+    assert len(ks) == 1 and ks[0].startswith("k_block_cc"), ks
+assert F.fake_used() == base
+""")
+
+
+def test_free_calls_share_no_scratch(lib):
+    """Each takes its scratch from the pool on its own stream and gives it back;
+    the context's buffer is neither used nor grown."""
+    fake_cuda.run(f"""
+c = context()
+base = F.fake_used()
+for p, m, k, nb in {FREE}:
+    for stream in (0, 16, 32):
+        assert block(c, p, m, k, nb, stream=stream) == 0
+        ks = kernels()
+        assert count(ks, "k_block_tc") >= 1 and count(ks, "k_block_cc") == 0, ks
+        assert F.fake_used() == base
+assert L.gfp_context_destroy(c) == 0
+assert "pool destroyed" in F.fake_events().decode()
+""")
+
+
+def test_free_calls_without_memory_take_the_cuda_cores(lib):
+    fake_cuda.run(f"""
+for pools in (1, 0):
+    F.fake_room(280 << 30)
+    F.fake_pools(pools)
+    c = context()
+    if pools:
+        F.fake_room(F.fake_used() + 65536)
+    for p, m, k, nb in {FREE}:
+        assert block(c, p, m, k, nb) == 0, (p, m, k, nb)
+        ks = kernels()
+        assert len(ks) == 1 and ks[0].startswith("k_block_cc"), ks
+        assert L.gfp_dot(c, 65521, 1024, A, B, C, 0) == 0
+        F.fake_events()
+""")
+
+
+def test_wide_free_calls_and_the_other_calls(lib):
+    """More columns than the tensor-core launches take; and the calls whose rule is
+    the context's workspace still use that and fail to grow it under capture."""
+    fake_cuda.run("""
+c = context()
+assert block(c, 65521, 7, 9, 65535 * 64 + 1) == 0
+assert count(kernels(), "k_block_cc") == 1
+base = F.fake_used()
+assert block(c, 65521, 4096, 4096, 64) == 0 and F.fake_used() > base
+F.fake_events()
+F.fake_capture(1)
+assert block(c, 65521, 4096, 4096, 64, stream=CAPTURING) == 0
+assert count(kernels(), "k_block_tc") == 1
+assert block(c, 65521, 8192, 4096, 64, stream=CAPTURING) == g.GFP_ERR_CUDA
 """)

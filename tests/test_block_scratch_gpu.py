@@ -1,5 +1,6 @@
 """Block products by the scratch they have: B's tiles for one residue modulus at a
-time where those of all would be too large."""
+time where those of all would be too large; and calls that need nothing of the
+context, on several streams at once and captured without a call before."""
 import numpy as np
 import pytest
 import torch
@@ -29,5 +30,69 @@ def test_tiles_of_b_for_one_modulus_at_a_time(lib):
             assert lib.gfp_launch_count(c) - n0 == 3 * 5 + 1
             assert lib.gfp_context_check(c) == lib.GFP_OK
             assert np.array_equal(host(C)[:, cols], oracle.block(p, A, np.ascontiguousarray(B[:, cols])))
+    finally:
+        c.close()
+
+
+# rows of A that 16-byte loads cannot take, and a small product over a large modulus
+FREE = [(65521, 700, 2999, 64), (65789, 3001, 5003, 40), (2147483647, 513, 1031, 64), (2147483647, 1024, 1024, 64),
+        (65521, 129, 301, 33)]
+
+
+def operands(p, m, k, nb, n):
+    A = [gi.uniform(p, m * k, 99 + i, 0).reshape(m, k) for i in range(n)]
+    B = [gi.uniform(p, k * nb, 99 + i, 1).reshape(k, nb) for i in range(n)]
+    want = [oracle.block(p, a, b) for a, b in zip(A, B)]
+    C = [torch.full((m, nb), -1, dtype=torch.int32, device="cuda") for _ in range(n)]
+    return [dev2(a) for a in A], [dev2(b) for b in B], C, want
+
+
+@pytest.mark.parametrize("p,m,k,nb", FREE)
+def test_streams_of_one_context_at_once(lib, p, m, k, nb):
+    """The same context on three streams, nothing ordering them, several products on
+    each behind one another; one more stream runs products through the context's
+    buffer."""
+    n = 3
+    A, B, C, want = operands(p, m, k, nb, n)
+    A4, B4, C4, want4 = operands(65521, 1000, 2000, 64, 1)
+    c = lib.Context(0)
+    try:
+        streams = [torch.cuda.Stream() for _ in range(n + 1)]
+        torch.cuda.synchronize()
+        for _ in range(4):
+            for x in C + C4:
+                x.fill_(-1)
+            torch.cuda.synchronize()
+            for _ in range(6):
+                for i in range(n):
+                    lib.gfp_matmul_block(c, p, A[i], B[i], C[i], stream=streams[i])
+                lib.gfp_matmul_block(c, 65521, A4[0], B4[0], C4[0], stream=streams[n])
+            torch.cuda.synchronize()
+            for i in range(n):
+                assert np.array_equal(host(C[i]), want[i]), i
+            assert np.array_equal(host(C4[0]), want4[0])
+        assert lib.gfp_context_check(c) == lib.GFP_OK
+    finally:
+        c.close()
+
+
+@pytest.mark.parametrize("p,m,k,nb", FREE)
+def test_captured_without_a_call_before(lib, p, m, k, nb):
+    A, B, C, want = operands(p, m, k, nb, 2)
+    c = lib.Context(0)
+    try:
+        g, s = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+        with torch.cuda.graph(g, stream=s):
+            lib.gfp_matmul_block(c, p, A[0], B[0], C[0])
+        C[0].fill_(-1)
+        other = torch.cuda.Stream()
+        torch.cuda.synchronize()
+        for _ in range(3):      # replays beside calls of the same context
+            g.replay()
+            for _ in range(3):
+                lib.gfp_matmul_block(c, p, A[1], B[1], C[1], stream=other)
+        torch.cuda.synchronize()
+        assert np.array_equal(host(C[0]), want[0]) and np.array_equal(host(C[1]), want[1])
+        del g
     finally:
         c.close()
