@@ -106,12 +106,18 @@ static thread_local cudaError_t g_last_cuda_error = cudaSuccess;
     do {                                                     \
         cudaError_t e_ = (expr);                             \
         if (e_ != cudaSuccess) {                             \
-            g_last_cuda_error = e_;                          \
+            gfp::note_cuda_error(e_);                        \
             return GFP_ERR_CUDA;                             \
         }                                                    \
     } while (0)
 
-void gfp::note_cuda_error(cudaError_t e) { g_last_cuda_error = e; }
+// The status reports the error: it does not also stay with the runtime, where the
+// next launch's check would find it.
+void gfp::note_cuda_error(cudaError_t e)
+{
+    g_last_cuda_error = e;
+    (void)cudaGetLastError();
+}
 
 static inline cudaStream_t as_stream(void *s) { return reinterpret_cast<cudaStream_t>(s); }
 

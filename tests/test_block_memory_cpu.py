@@ -144,3 +144,17 @@ assert block(c, 65521, 4096, 4096, 64, stream=CAPTURING) == 0
 assert count(kernels(), "k_block_tc") == 1
 assert block(c, 65521, 8192, 4096, 64, stream=CAPTURING) == g.GFP_ERR_CUDA
 """)
+
+
+def test_reported_error_is_not_reported_again(lib):
+    """A call that cannot grow its buffer under capture fails; the calls behind it
+    do not fail for it."""
+    fake_cuda.run("""
+c = context()
+for _ in range(2):
+    F.fake_capture(1)
+    assert block(c, 65521, 4096, 4096, 64, stream=CAPTURING) == g.GFP_ERR_CUDA
+    F.fake_capture(0)
+    assert L.gfp_dot(c, 65521, 1024, A, B, C, 0) == 0
+    assert L.gfp_matvec(c, 65521, 1024, 1024, A, 1024, B, C, 0) == 0
+""")
