@@ -260,9 +260,9 @@ struct gfp_ctx {
     void *blk_ws = nullptr;
     size_t blk_ws_bytes = 0, blk_tail_bytes = 0;   // sizes of the two parts
     uint32_t *blk_err = nullptr;                   // error word of all block products
-    // stream-ordered scratch of the block products that keep none in the context
+    // stream-ordered scratch of the block products that keep none in the buffer, or
+    // null; made with the context, for making it may be refused during a capture
     cudaMemPool_t blk_pool = nullptr;
-    bool blk_pool_tried = false;
 
     // tuned plan: (p, lg_n) -> entry
     std::map<std::pair<uint32_t, uint32_t>, gfp_plan_entry> plan;

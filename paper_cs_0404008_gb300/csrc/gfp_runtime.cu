@@ -403,6 +403,32 @@ GFP_API gfp_repr gfp_choose_repr(const gfp_ctx *ctx, uint32_t p, uint64_t n)
 
 GFP_API gfp_status gfp_plan_load(gfp_ctx *ctx, const char *path);   // gfp_tune.cu
 
+// Pool of stream-ordered scratch: keeps up to 256 MiB between calls, makes no
+// stream wait for another.  Null where it cannot be had.
+static cudaMemPool_t make_scratch_pool(int device)
+{
+    int has = 0;
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = device;
+    cudaMemPool_t pool = nullptr;
+    if (cudaDeviceGetAttribute(&has, cudaDevAttrMemoryPoolsSupported, device) != cudaSuccess || !has ||
+        cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return nullptr;
+    }
+    uint64_t keep = 256ull << 20;
+    int no = 0;
+    if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess ||
+        cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowInternalDependencies, &no) != cudaSuccess) {
+        (void)cudaGetLastError();
+        cudaMemPoolDestroy(pool);
+        return nullptr;
+    }
+    return pool;
+}
+
 GFP_API gfp_status gfp_context_create(int device, gfp_ctx **out)
 {
     GFP_TRACE();
@@ -430,7 +456,9 @@ GFP_API gfp_status gfp_context_create(int device, gfp_ctx **out)
     c->ring_slots = (unsigned long long *)mem;
     c->d_flag = (uint32_t *)((char *)mem + ring_bytes);
     c->blk_err = (uint32_t *)((char *)mem + ring_bytes + 128);
+    c->blk_pool = make_scratch_pool(device);
     if (cudaDeviceSynchronize() != cudaSuccess) {
+        if (c->blk_pool) cudaMemPoolDestroy(c->blk_pool);
         cudaFree(mem);
         delete c;
         return GFP_ERR_CUDA;
@@ -896,42 +924,25 @@ static gfp_status run_block_tc(gfp_ctx *ctx, const BlockCall &q, cudaStream_t s)
     return st == GFP_OK ? launch_block(ctx, q, sc, R, s) : st;
 }
 
-// Pool of the stream-ordered scratch: keeps up to 256 MiB between calls, makes no
-// stream wait for another.  Null where it cannot be had.
-static cudaMemPool_t block_pool(gfp_ctx *ctx)
-{
-    std::lock_guard<std::mutex> g(ctx->mu);
-    if (ctx->blk_pool_tried) return ctx->blk_pool;
-    ctx->blk_pool_tried = true;
-    int has = 0;
-    cudaMemPoolProps props = {};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = ctx->device;
-    cudaMemPool_t pool = nullptr;
-    if (cudaDeviceGetAttribute(&has, cudaDevAttrMemoryPoolsSupported, ctx->device) != cudaSuccess || !has ||
-        cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return nullptr;
-    }
-    uint64_t keep = 256ull << 20;
-    int no = 0;
-    if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess ||
-        cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowInternalDependencies, &no) != cudaSuccess) {
-        (void)cudaGetLastError();
-        cudaMemPoolDestroy(pool);
-        return nullptr;
-    }
-    return ctx->blk_pool = pool;
-}
+// Allocating and freeing in stream order is refused, and ends the capture, while a
+// stream of any thread is being captured in the mode that watches them all; it has
+// nothing to do with that capture, so this thread asks not to be watched.
+struct Unwatched {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    Unwatched() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~Unwatched() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    Unwatched(const Unwatched &) = delete;
+    Unwatched &operator=(const Unwatched &) = delete;
+};
 
 // The product with scratch of its own, allocated and freed in stream order: calls
 // on several streams do not meet.  GFP_ERR_NOMEM, with nothing launched, where there
 // is none.
 static gfp_status run_block_tc_pool(gfp_ctx *ctx, const BlockCall &q, cudaStream_t s)
 {
-    const cudaMemPool_t pool = block_pool(ctx);
+    const cudaMemPool_t pool = ctx->blk_pool;
     if (!pool) return GFP_ERR_NOMEM;
+    const Unwatched unwatched;
     BlockScratch sc;
     sc.at_once = block_tc_moduli_at_once(q.k, q.nb, q.n_mod());
     void *mem = nullptr;

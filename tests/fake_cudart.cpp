@@ -19,7 +19,8 @@ std::map<void *, size_t> blocks;
 std::string events;
 size_t room = (size_t)280 << 30, peak = 0, used = 0;
 int regs = 72, has_pools = 1;
-bool captured = false;    // some stream is being captured
+bool captured = false;    // some stream is being captured, in the mode that watches all threads
+cudaStreamCaptureMode mode = cudaStreamCaptureModeGlobal;   // this thread's
 cudaError_t last = cudaSuccess;
 
 cudaError_t err(cudaError_t e)
@@ -121,6 +122,7 @@ cudaError_t cudaMemPoolDestroy(cudaMemPool_t) { note("pool destroyed"); return c
 cudaError_t cudaMallocFromPoolAsync(void **p, size_t n, cudaMemPool_t, cudaStream_t s)
 {
     if (capturing(s)) note("allocation captured");
+    if (captured && mode != cudaStreamCaptureModeRelaxed) return err(cudaErrorStreamCaptureUnsupported);
     return take(p, n);
 }
 cudaError_t cudaFreeAsync(void *p, cudaStream_t) { return give(p); }
@@ -129,6 +131,13 @@ cudaError_t cudaFreeAsync(void *p, cudaStream_t) { return give(p); }
 cudaError_t cudaStreamIsCapturing(cudaStream_t s, cudaStreamCaptureStatus *st)
 {
     *st = capturing(s) ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+    return cudaSuccess;
+}
+cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode *m)
+{
+    const cudaStreamCaptureMode was = mode;
+    mode = *m;
+    *m = was;
     return cudaSuccess;
 }
 }

@@ -158,3 +158,20 @@ for _ in range(2):
     assert L.gfp_dot(c, 65521, 1024, A, B, C, 0) == 0
     assert L.gfp_matvec(c, 65521, 1024, 1024, A, 1024, B, C, 0) == 0
 """)
+
+
+def test_free_calls_beside_a_capture(lib):
+    """While another stream is being captured, the first such call of a context
+    and the later ones run on the tensor cores, and ask the runtime for nothing it
+    refuses then; the thread's capture mode is as before."""
+    fake_cuda.run(f"""
+c = context()
+F.fake_capture(1)
+for p, m, k, nb in {FREE}:
+    assert block(c, p, m, k, nb) == 0
+    assert count(kernels(), "k_block_tc") >= 1
+assert F.cudaDeviceSynchronize() != 0
+mode = ctypes.c_int(0)
+F.cudaThreadExchangeStreamCaptureMode(ctypes.byref(mode))
+assert mode.value == 0
+""")

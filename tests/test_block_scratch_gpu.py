@@ -96,3 +96,30 @@ def test_captured_without_a_call_before(lib, p, m, k, nb):
         del g
     finally:
         c.close()
+
+
+@pytest.mark.parametrize("p,m,k,nb", FREE[:3])
+def test_beside_a_capture(lib, p, m, k, nb):
+    """While another stream is being captured (in the mode that watches all
+    threads), such a call runs on a stream of its own, the first of a context too."""
+    A, B, C, want = operands(p, m, k, nb, 1)
+    c, c2 = lib.Context(0), lib.Context(0)
+    try:
+        g, s, other = torch.cuda.CUDAGraph(), torch.cuda.Stream(), torch.cuda.Stream()
+        x = torch.zeros(1000, dtype=torch.int32, device="cuda")
+        lib.gfp_matmul_block(c2, p, A[0], B[0], C[0])     # kernels loaded
+        C[0].fill_(-1)
+        torch.cuda.synchronize()
+        with torch.cuda.graph(g, stream=s, capture_error_mode="global"):
+            x.add_(1)
+            lib.gfp_matmul_block(c, p, A[0], B[0], C[0], stream=other)
+            x.add_(1)
+        torch.cuda.synchronize()
+        assert np.array_equal(host(C[0]), want[0])
+        g.replay()
+        torch.cuda.synchronize()
+        assert int(x[0]) == 2
+        del g
+    finally:
+        c.close()
+        c2.close()
