@@ -197,7 +197,7 @@ def _check(st: int, where: str):
 
 
 _torch = None      # set by the first call that needs it (the host-only functions work without torch)
-_stream_ready = False
+_raw_stream = _device = None   # set by the first call on torch's current stream
 _U32 = _U16 = ()   # the tensor types taken as uint32, as uint16 codes
 
 
@@ -222,18 +222,28 @@ def _ptr(t) -> int:
     raise TypeError(f"cannot take the address of {type(t)}")
 
 
+def _stream_functions(torch):
+    """(raw handle of a device's current stream, current device): torch's internal
+    functions where this version has them, else through the public call."""
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    device = getattr(torch._C, "_cuda_getDevice", None)
+    if raw is None or device is None:
+        return (lambda _: torch.cuda.current_stream().cuda_stream), (lambda: None)
+    return raw, device
+
+
 def _stream(stream) -> int:
     """The raw handle of `stream`, of the current device's current stream when
     none is given (asked for as a handle: a torch.cuda.Stream object built on
     every call cost more than the launch of a small product)."""
-    global _stream_ready
+    global _raw_stream, _device
     if stream is None:
-        if not _stream_ready:   # the first time through torch's own call, which initialises CUDA
-            s = (_torch or _import_torch()).cuda.current_stream().cuda_stream
-            _stream_ready = True
+        if _raw_stream is None:   # the first time through torch's own call, which initialises CUDA
+            torch = _torch or _import_torch()
+            s = torch.cuda.current_stream().cuda_stream
+            _raw_stream, _device = _stream_functions(torch)
             return s
-        c = _torch._C
-        return c._cuda_getCurrentRawStream(c._cuda_getDevice())
+        return _raw_stream(_device())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
