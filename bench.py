@@ -840,6 +840,10 @@ def measure_secondary(args, workload, g, torch, ctx, stream):
                                        ("u64_carry_cuda_core", g.GFP_REPR_U64_CARRY, 3)):
                     ctx.set_repr(rp)
                     large[name] = timed(lambda: g.gfp_matmul_block(ctx, pl, Al, Bl, C, stream), reps)
+            ctx.set_repr(g.GFP_REPR_F16TC)
+            n0 = g.gfp_launch_count(ctx)
+            g.gfp_matmul_block(ctx, p, A, B, C, stream)
+            launches = g.gfp_launch_count(ctx) - n0
             ctx.set_repr(0)
             # A prepared once (digit images in the layout the tensor cores read),
             # as for a resident matrix used by many products
@@ -879,7 +883,7 @@ def measure_secondary(args, workload, g, torch, ctx, stream):
                              "peak_kind": f"{peak_kind} hbm_gbs",
                              "tensor_tflops_fp16": tflops},
                 "same_gpu": {n: {"ms": v, "gmacs": macs / (v / 1e3) / 1e9} for n, v in res.items()},
-                "gpu_launches": 3 if passes == 1 else 2 * passes + 2,
+                "gpu_launches": launches,
             })
             ppasses = rns_passes(p, k, 65536)
             ptf = ppasses * 4 * 2 * macs / (t_prep / 1e3) / 1e12

@@ -261,11 +261,13 @@ GFP_API gfp_status gfp_matvec_sequence(gfp_ctx *ctx, uint32_t p, uint64_t n, con
  * Path: with GFP_REPR_AUTO, or with GFP_REPR_F16TC, A 16-byte aligned and lda
  * a multiple of 4, the tensor cores: for p <= 65791 the digit kernel directly
  * (three launches: B digit split, the persistent product, the reduction of
- * its partial sums into C; two where K is at most 512 and the row and column
- * tiles fill the GPU); for larger p
+ * its partial sums into C; two, the product writing C, where a tile of C is the work
+ * of one CTA: k at most 64, or at most 512 with tiles enough to fill the GPU); for
+ * larger p
  * one such pass per modulus of a residue number system (the L <= 6 largest
  * primes <= 65536 whose product exceeds k (p-1)^2, each pass reducing the
- * inputs modulo its prime; B's digits for all of them in one launch) and one
+ * inputs modulo its prime; B's digits for all of them in one launch while they
+ * take at most 1 GiB, else one modulus at a time) and one
  * launch recombining the residues with
  * Garner's method modulo p, where that is expected to be faster than the
  * CUDA cores.  Rows of A at other alignments take the same kernel with 4-byte
@@ -308,8 +310,8 @@ GFP_API gfp_status gfp_block_prepare(gfp_ctx *ctx, uint32_t p, uint64_t m, uint6
 /* C = A B mod p for the prepared A (m x k): B device k x nb (ldb >= nb),
  * C device m x nb (ldc >= nb); the same result as gfp_matmul_block on the
  * original A.  Three launches (B's digits, the product, its partial sums
- * into C), or for residue passes B's digits once, two a pass and one
- * recombination.  Uses the
+ * into C), or for residue passes B's digits, two a pass and one recombination;
+ * one fewer a product or pass where a tile of C is the work of one CTA.  Uses the
  * context's block workspace (grown on first use of a shape: make that call
  * outside stream capture); calls sharing one context must not run
  * concurrently on different streams. */

@@ -222,15 +222,6 @@ __global__ void k_wait_selftest(uint64_t limit_ns, uint32_t *err)
 
 __device__ uint32_t g_selftest_err;
 
-// warp-uniform bounded wait: lane 0 polls, the result is broadcast
-__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile uint32_t *abort,
-                                          uint32_t *err)
-{
-    bool ok = true;
-    if ((threadIdx.x & 31) == 0) ok = wait_bar(bar, parity, abort, err);
-    return __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-}
-
 // Walks a CTA's units in order (row tiles innermost, then K ranges, then
 // column tiles), or backwards.
 struct Walk {

@@ -179,10 +179,10 @@ __device__ __forceinline__ uint32_t unit_residue(const DevPair &pr, const DevUni
 // A pair of one unit is written at once; the units of another meet in one
 // 64-bit atomic each (combine_packed), or, above the 65535 that its count holds,
 // through a slot and a ticket.  For a list of short pairs these round trips are
-// the time: 64 pairs of 2^6 to 2^13 terms 7.8 -> 2.9 us a launch, 1024 of 2^8 to
+// the time: 64 pairs of 2^6 to 2^13 terms 8.2 -> 3.2 us a launch, 1024 of 2^8 to
 // 2^14 14.5 -> 8.0 us against a counter for every unit, a slot, a fence and a
-// ticket for every pair and no early launch; 4096 pairs of 2^8 to 2^20 terms 606
-// -> 575 us (7.4 TB/s).  Three CTAs per SM: with four (64 registers) the long list
+// ticket for every pair and no early launch; 4096 pairs of 2^8 to 2^20 terms 597
+// -> 576 us (7.3 TB/s).  Three CTAs per SM: with four (64 registers) the long list
 // took 572 us, the short ones 5.2 and 8.4 against 4.3 (256 pairs) and 8.0 us.
 __global__ void __launch_bounds__(DOT_THREADS, 3)
     k_dot_batched(const DevPair *__restrict__ pairs, const DevPairAux *__restrict__ aux,

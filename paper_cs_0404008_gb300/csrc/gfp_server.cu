@@ -606,7 +606,7 @@ GFP_API gfp_status gfp_register_matrix(gfp_server *s, uint32_t p, uint64_t rows,
     Matrix M{p, rows, cols, dev, nullptr, cols};
     if (!dev && !s->cfg.simulate) {
         // rows start on 16-byte boundaries so that the tensor-core block
-        // product (which copies A by TMA) can take the matrix
+        // product reads them with 16-byte loads
         M.ld = (cols + 3) / 4 * 4;
         void *mem = nullptr;
         if (cudaSetDevice(s->cfg.device) != cudaSuccess) return GFP_ERR_CUDA;
