@@ -328,8 +328,9 @@ GFP_API gfp_status gfp_block_prep_destroy(gfp_block_prep *prep);
  * into col[] and val[], column indices < k, values canonical residues), B is
  * k x nb dense.  C[i*ldc + j] = (sum_q val[q] * B[col[q]*ldb + j]) mod p for
  * row_ptr[i] <= q < row_ptr[i+1].  All arrays on the device; row_ptr must be
- * non-decreasing with row_ptr[0] = 0 (checked on the device only when
- * validation is enabled, together with col < k and the residues).  One launch;
+ * non-decreasing with row_ptr[0] = 0 and row_ptr[m] <= 2^32 - 32 (checked only
+ * when validation is enabled, together with col < k and the residues; nonzeros past
+ * 2^32 - 32 are not read).  One launch;
  * k == 0 writes zeros.  Representation: the one forced on the context, else
  * the built-in rule for p (tuned plans do not apply). */
 GFP_API gfp_status gfp_matmul_block_csr(gfp_ctx *ctx, uint32_t p, uint64_t m, uint64_t k,

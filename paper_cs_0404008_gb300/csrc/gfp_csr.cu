@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(256)
     const bool pair_ok = ((((uintptr_t)B) & 7u) == 0) && (ldb % 2 == 0);
     for (uint64_t row = (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); row < m;
          row += warps) {
-        const uint32_t q0 = __ldg(row_ptr + row), q1 = __ldg(row_ptr + row + 1);
+        const uint32_t q0 = __ldg(row_ptr + row), q1 = min(__ldg(row_ptr + row + 1), CSR_NNZ_MAX);
         GFP_DCHECK(g_csr_check, q0 <= q1, DCHECK_CSR_ROW_PTR);
         for (uint64_t c0 = 0; c0 < nb; c0 += 64) {
             const uint64_t ca = c0 + 2 * lane;             // this lane's columns ca, ca+1
@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(256)
             Acc a0, a1;
             a0.init(mod, kbound);
             a1.init(mod, kbound);
-            for (uint32_t q = q0; q < q1; q = csr_next(q, q1)) {
+            for (uint32_t q = q0; q < q1; q += 32) {
                 const uint32_t cnt = min(32u, q1 - q);
                 uint32_t mycol = 0, myval = 0;
                 if ((uint32_t)lane < cnt) {
@@ -139,7 +139,7 @@ __device__ __forceinline__ void csr_row_quads(uint32_t q0, uint32_t q1, uint64_t
         cn = __ldg(col + q0 + lane);
         vn = __ldg(val + q0 + lane);
     }
-    for (uint32_t q = q0; q < q1; q = csr_next(q, q1)) {
+    for (uint32_t q = q0; q < q1; q += 32) {
         const uint32_t cnt = min(32u, q1 - q);
         uint32_t c = cn, v = vn;
         cn = 0;
@@ -189,12 +189,13 @@ __global__ void __launch_bounds__(256, PLAIN ? 4 : 3)
     const uint64_t stride = (uint64_t)gridDim.x * groups;
     const bool cvec = ((((uintptr_t)C) & 15u) == 0) && (ldc % 4 == 0);
     for (uint64_t row = (uint64_t)blockIdx.x * groups + group; row < m; row += stride) {
-        uint32_t q0 = __ldg(row_ptr + row), q1 = __ldg(row_ptr + row + 1);
+        uint32_t q0 = __ldg(row_ptr + row), q1 = min(__ldg(row_ptr + row + 1), CSR_NNZ_MAX);
         GFP_DCHECK(g_csr_check, q0 <= q1, DCHECK_CSR_ROW_PTR);
         if constexpr (SPLIT) {
-            const uint2 run = csr_run(q1 > q0 ? q1 - q0 : 0u, S, sub);
-            q1 = q0 + run.y;
-            q0 += run.x;
+            uint32_t b, e;
+            csr_run(q1 > q0 ? q1 - q0 : 0u, S, sub, b, e);
+            q1 = q0 + e;
+            q0 += b;
         }
         for (uint64_t c0 = 0; c0 < nb; c0 += 64) {
             const uint64_t ca = c0 + 4 * (uint64_t)hl;

@@ -195,18 +195,21 @@ cudaError_t wait_selftest(uint64_t limit_ns, cudaStream_t s, uint32_t *status_bi
 cudaError_t launch_block_cc(Repr r, const Mod &mod, uint64_t kbound, uint64_t m, uint64_t k,
                             uint64_t nb, const uint32_t *A, uint64_t lda, const uint32_t *B,
                             uint64_t ldb, uint32_t *C, uint64_t ldc, cudaStream_t s);
-// Sparse-row block product (gfp_csr.cu).  Offsets into a row's nonzeros go up to
-// 2^32 - 1, so nothing here may pass 2^32 on the way.
+// Sparse-row block product (gfp_csr.cu).  Nonzeros at most, so that the 32-bit
+// offset of a chunk of 32 behind any of them does not pass 2^32 (a loop over
+// chunks whose end is tested otherwise took 3 to 7 % longer).
+constexpr uint32_t CSR_NNZ_MAX = 0xFFFFFFE0u;
 // Run `sub` of the S >= 2 equal runs, rounded up to steps of eight, of n nonzeros:
-// [x, y).
-GFP_HD uint2 csr_run(uint32_t n, uint32_t S, uint32_t sub)
+// from x up to y.  The last takes what is left, so that nothing passes 2^32 on the
+// way where n is within 64 of it (in 64 bits, or with the quotient rounded up by a
+// comparison, a product with split rows took up to 28 % longer).
+GFP_HD void csr_run(uint32_t n, int S, int sub, uint32_t &x, uint32_t &y)
 {
-    const uint32_t part = (n / (8 * S) + (n % (8 * S) ? 1u : 0u)) * 8;
-    const uint32_t b = part * sub < n ? part * sub : n;   // at most n - n / S + 8 (S - 1)
-    return make_uint2(b, n - b > part ? b + part : n);
+    const uint32_t top = 0xFFFFFFC0u, part = (((n < top ? n : top) + 8 * S - 1) / (8 * S)) * 8;
+    const uint32_t b = part * sub;
+    x = b < n ? b : n;
+    y = sub == S - 1 ? n : x + part < n ? x + part : n;
 }
-// The chunk of 32 nonzeros behind the one at q < q1, or q1.
-GFP_HD uint32_t csr_next(uint32_t q, uint32_t q1) { return q1 - q > 32u ? q + 32u : q1; }
 cudaError_t launch_block_csr(Repr r, const Mod &mod, uint64_t kbound, uint64_t m, uint64_t k,
                              uint64_t nb,
                              const uint32_t *row_ptr, const uint32_t *col, const uint32_t *val,

@@ -1148,6 +1148,7 @@ GFP_API gfp_status gfp_matmul_block_csr(gfp_ctx *ctx, uint32_t p, uint64_t m, ui
         for (uint64_t i = 0; i < m; ++i)
             if (rp[i + 1] < rp[i]) return GFP_ERR_INVALID;
         const uint64_t nnz = rp[m];
+        if (nnz > CSR_NNZ_MAX) return GFP_ERR_INVALID;
         if (nnz && (!col || !val)) return GFP_ERR_INVALID;
         gfp_status st = check_range(ctx, col, nnz, k ? (uint32_t)std::min<uint64_t>(k, 0xFFFFFFFFull) : 0u, s);
         if (st == GFP_ERR_RANGE) return GFP_ERR_INVALID;
