@@ -102,9 +102,8 @@ uint64_t centered_bound(uint32_t p);
 uint64_t montgomery_bound(uint32_t p);
 bool repr_eligible(Repr r, uint32_t p);
 
-// Launch configuration constants of the dot kernels.
+// Launch configuration of the dot kernels.
 constexpr int DOT_THREADS = 256;
-constexpr int MV_THREADS = 512;
 
 // Device scratch of one batched execution.
 struct BatchScratch {

@@ -18,19 +18,36 @@
 // 41.6 us (6.1 TB/s).  Batches of four or six vectors were slower (70 and 66
 // against 52 us for the latter with a flushed L2): more batches a row.
 //
+// Rows of at most 256 columns are bound by the latency of a row (load, add, reduce
+// by shuffles): twice the warps with batches of two vectors; 200000 x 64 over
+// GF(65521) 64.8 -> 36.5 us, 45 with one batch of four in flight.  Above 51200
+// columns x is read through L1 and L2 beside A, in 32 warps with one batch of four
+// in flight: two batches of eight in 16 warps took 82.2 against 55.9 us for
+// 700 x 100000 over GF(65521), and 286 against 87.1 where rows are not 16-byte
+// aligned.
+//
 // Rows need not be 16-byte aligned.  A row that starts r words past a 16-byte
 // boundary is read as the aligned vectors inside it; x is then kept in shared
 // memory as four planes of every fourth element, so that the four elements a
 // vector multiplies are one conflict-free read each (from a plain x the lanes'
 // words would lie four apart, a four-way bank conflict).  The fewer than four
-// elements before the first and after the last vector are added by themselves.
+// elements before the first and after the last vector are added by themselves.  Such
+// rows of at most 64 columns, a word or two a lane, are read word by word (200000 x
+// 16 over GF(65521): 44 against 55 us).
 #include <algorithm>
 
 #include "gfp_internal.h"
 
 namespace gfp {
 
-constexpr int MV_U = 8;     // vectors a lane loads at a time, two batches in flight
+// Threads and vectors a lane loads at a time, two batches in flight: for rows of
+// more than MV_SHORT columns, for shorter ones; and, one batch in flight, for rows whose
+// x is not in shared memory.
+constexpr int MV_THREADS = 512, MV_U = 8;
+constexpr int MV_SHORT_THREADS = 1024, MV_SHORT_U = 2;
+constexpr int MV_GLOBAL_THREADS = 1024, MV_GLOBAL_U = 4;
+constexpr uint64_t MV_SHORT = 256, MV_WORDS = 64;   // columns
+constexpr uint32_t MV_GLOBAL_WINDOW = 64;           // rows
 constexpr int MV_PREFETCH_ROWS = 4;   // rows of A requested into L2 before the dependency wait
 
 // Sum of one uint64 per thread over the CTA, valid in thread 0.
@@ -76,8 +93,8 @@ struct RowPart {
     uint32_t eval;     // that element
 };
 
-template <class Acc, int XM, int U>
-__global__ void __launch_bounds__(MV_THREADS, 1)
+template <class Acc, int XM, int U, int T>
+__global__ void __launch_bounds__(T, 1)
     k_matvec(Mod m, uint64_t k, uint64_t rows, uint64_t cols, const uint32_t *__restrict__ A,
              uint64_t lda, const uint32_t *__restrict__ x, uint32_t *__restrict__ y, int W, uint32_t window,
              MvProj proj)
@@ -104,8 +121,9 @@ __global__ void __launch_bounds__(MV_THREADS, 1)
     uint32_t *xs = smem;
     const uint32_t plane = (uint32_t)(colsp >> 2);   // words of a plane of x
     uint32_t *part = smem + (XM != X_GLOBAL ? colsp : 0);
-    const int nw = MV_THREADS / 32, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int G = nw / W, g = w / W, sgm = w % W;
+    const int nw = T / 32, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int G = nw / W, sgm = w % W;
+    const uint32_t g = w < G * W ? (uint32_t)(w / W) : ~0u;   // ~0: no group, where W does not divide the warps
 
     // column segment of this warp: [c0, c1), c0 a multiple of 4
     const uint64_t seg = ((cols + W - 1) / W + 3) & ~3ull;
@@ -113,15 +131,11 @@ __global__ void __launch_bounds__(MV_THREADS, 1)
     const uint64_t c1 = min(c0 + seg, cols);
     // batches that cover any row's part (at least one: it carries the elements outside the vectors)
     const uint32_t nq = max(1u, (uint32_t)((((c1 - c0) >> 2) + U * 32 - 1) / (U * 32)));
-    // rows that 16-byte loads take as they are (X_GLOBAL: else the plain loop below)
-    const bool vec = XM != X_GLOBAL ||
-                     ((((uintptr_t)A) | (uintptr_t)(lda * 4) | ((uintptr_t)x)) & 15u) == 0;
 
-    const uint32_t cs = XM != X_GLOBAL ? (uint32_t)c0 : 0u;   // c0, where x is in shared memory
+    const uint32_t cs = (uint32_t)c0;   // where x is in shared memory
     const auto xat = [&](uint32_t j) -> uint32_t {
         if constexpr (XM == X_PLANES) return xs[(j & 3) * plane + ((cs + j) >> 2)];   // c0 is a multiple of 4
-        else if constexpr (XM == X_SMEM) return xs[cs + j];
-        else return __ldg(x + c0 + j);
+        else return xs[cs + j];
     };
     const auto locate = [&](uint64_t row, RowPart &p) {
         const uint32_t *Ar = A + row * lda + c0;
@@ -157,10 +171,8 @@ __global__ void __launch_bounds__(MV_THREADS, 1)
                     const uint32_t i1 = i + (j > 2), i2 = i + (j > 1), i3 = i + (j > 0);
                     xv = make_uint4(xs[j * plane + i], xs[((j + 1) & 3) * plane + i1],
                                     xs[((j + 2) & 3) * plane + i2], xs[((j + 3) & 3) * plane + i3]);
-                } else if constexpr (XM == X_SMEM) {
-                    xv = reinterpret_cast<const uint4 *>(xs + cs)[v];
                 } else {
-                    xv = __ldg(reinterpret_cast<const uint4 *>(x + c0) + v);
+                    xv = reinterpret_cast<const uint4 *>(xs + cs)[v];
                 }
                 acc.add4(buf[u], xv, m);
             }
@@ -178,7 +190,7 @@ __global__ void __launch_bounds__(MV_THREADS, 1)
             if (lane == 0) part[i * W + sgm] = reduce64(s, m);
             acc.init(m, k);
         };
-        if (vec) {
+        if constexpr (XM != X_GLOBAL) {
             uint4 b0[U], b1[U];
             RowPart cur, nxt;
             uint32_t i = g, q = 0;
@@ -187,7 +199,7 @@ __global__ void __launch_bounds__(MV_THREADS, 1)
                 load(cur, 0, b0);
             }
             if (!staged) {   // the first loads are under way
-                for (uint64_t j = threadIdx.x; j < colsp; j += MV_THREADS)
+                for (uint64_t j = threadIdx.x; j < colsp; j += T)
                     xs[XM == X_PLANES ? (j & 3) * plane + (j >> 2) : j] = (j < cols) ? x[j] : 0u;
                 __syncthreads();
                 staged = true;
@@ -216,22 +228,33 @@ __global__ void __launch_bounds__(MV_THREADS, 1)
                 if (i < rcount) step(b1, b0);
             }
         } else {
+            // rows that 16-byte loads take as they are
+            const bool vec = ((((uintptr_t)A) | (uintptr_t)(lda * 4) | ((uintptr_t)x)) & 15u) == 0;
             for (uint32_t i = g; i < rcount; i += G) {
                 const uint32_t *Ar = A + (rb + i) * lda;
-                constexpr int S = 8;
-                for (uint64_t j = c0 + lane; j < c1; j += 32 * S) {
-                    uint32_t v[S];
+                if (vec) {
+                    const uint4 *av = reinterpret_cast<const uint4 *>(Ar + c0);
+                    const uint4 *xv = reinterpret_cast<const uint4 *>(x + c0);
+                    const uint64_t nv = (c1 - c0) >> 2;
+                    uint64_t v = lane;
+                    for (; v + (U - 1) * 32 < nv; v += U * 32) {
+                        uint4 a[U];
 #pragma unroll
-                    for (int u = 0; u < S; ++u) v[u] = j + u * 32 < c1 ? __ldcs(Ar + j + u * 32) : 0u;
+                        for (int u = 0; u < U; ++u) a[u] = __ldcs(av + v + u * 32);
 #pragma unroll
-                    for (int u = 0; u < S; ++u)
-                        if (j + u * 32 < c1) acc.add(v[u], __ldg(x + j + u * 32), m);
+                        for (int u = 0; u < U; ++u) acc.add4(a[u], __ldg(xv + v + u * 32), m);
+                    }
+                    for (; v < nv; v += 32) acc.add4(__ldcs(av + v), __ldg(xv + v), m);
+                    const uint64_t j = c0 + (nv << 2) + lane;
+                    if (j < c1) acc.add(__ldcs(Ar + j), __ldg(x + j), m);
+                } else {
+                    for (uint64_t j = c0 + lane; j < c1; j += 32) acc.add(__ldcs(Ar + j), __ldg(x + j), m);
                 }
                 finish(i);
             }
         }
         __syncthreads();
-        for (uint32_t i = threadIdx.x; i < rcount; i += MV_THREADS) {
+        for (uint32_t i = threadIdx.x; i < rcount; i += T) {
             uint64_t s = 0;
             for (int q = 0; q < W; ++q) s += part[i * W + q];
             const uint32_t yi = reduce64(s, m);
@@ -259,34 +282,48 @@ __global__ void __launch_bounds__(MV_THREADS, 1)
 // part kept for the segment residues of a window of rows.
 constexpr size_t MV_XS_MAX = 200 * 1024, MV_PART_MAX = 16 * 1024;
 
-template <class Acc, int XM>
+template <class Acc, int XM, int U, int T>
 static cudaError_t mv_launch(const Mod &m, uint64_t k, uint64_t rows, uint64_t cols,
                              const uint32_t *A, uint64_t lda, const uint32_t *x, uint32_t *y,
                              int sm_count, cudaStream_t s, const MvProj &proj)
 {
-    constexpr int U = MV_U;
-    const int nw = MV_THREADS / 32;
+    const int nw = T / 32;
     const uint64_t grid = std::min<uint64_t>((uint64_t)sm_count, rows ? rows : 1);
     const uint64_t per_cta = (rows + grid - 1) / grid;
-    // warps per row: as few as take a row in one batch of U vectors a lane (more
-    // warps would reduce more often for the same bytes), and more where a CTA's
-    // rows would leave half of its warps without one
     const uint64_t nv = cols / 4;
     int W = 1;
-    while (W < nw && (nv > (uint64_t)W * U * 32 || (uint64_t)(nw / W) >= 2 * per_cta)) W *= 2;
+    if constexpr (XM == X_GLOBAL) {
+        // at least one batch a warp
+        while (W < nw && nv / (uint64_t)(2 * W) >= (uint64_t)U * 32) W *= 2;
+    } else {
+        // warps per row: the power of two that takes a row in one batch of U vectors a
+        // lane (more would reduce more often for the same bytes), another number where
+        // its batches fill more of all lanes (a row of 1125 vectors: eight warps fill
+        // 55 % of them, three groups of five 82 %; 3000 x 4500 over GF(65521) 12.2 ->
+        // 10.2 us, 10.6 in eight warps with batches of four), and more where a CTA's
+        // rows would leave half of its warps without one
+        const auto filled = [&](int c) {
+            const uint64_t batch = (uint64_t)c * U * 32;
+            return (double)(nw / c * c) / nw * (double)nv / (double)((nv + batch - 1) / batch * batch);
+        };
+        while (W < nw && nv > (uint64_t)W * U * 32) W *= 2;
+        for (int c = 1; nv && c <= nw; ++c)
+            if (nv <= (uint64_t)c * U * 32 && filled(c) > 1.05 * filled(W)) W = c;
+        while (2 * W <= nw && (uint64_t)(nw / W) >= 2 * per_cta) W *= 2;
+    }
     const size_t colsp = (cols + 3) & ~3ull;
-    const uint32_t window = (uint32_t)std::min<uint64_t>(per_cta, MV_PART_MAX / (4 * W));
+    const uint32_t window = (uint32_t)std::min<uint64_t>(per_cta, XM == X_GLOBAL ? MV_GLOBAL_WINDOW : MV_PART_MAX / (4 * W));
     const size_t smem = (XM != X_GLOBAL ? colsp * 4 : 0) + (size_t)window * W * 4;
     static bool attr_set = false;
     if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_matvec<Acc, XM, U>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(k_matvec<Acc, XM, U, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)(MV_XS_MAX + MV_PART_MAX));
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(MV_THREADS);
+    cfg.blockDim = dim3(T);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
@@ -294,7 +331,7 @@ static cudaError_t mv_launch(const Mod &m, uint64_t k, uint64_t rows, uint64_t c
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_matvec<Acc, XM, U>, m, k, rows, cols, A, lda, x,
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_matvec<Acc, XM, U, T>, m, k, rows, cols, A, lda, x,
                                              y, W, window, proj);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -304,12 +341,19 @@ static cudaError_t mv_dispatch(const Mod &m, uint64_t k, uint64_t rows, uint64_t
                                const uint32_t *A, uint64_t lda, const uint32_t *x, uint32_t *y,
                                int sm_count, cudaStream_t s, const MvProj &proj)
 {
-    if (((cols + 3) & ~3ull) * 4 > MV_XS_MAX)
-        return mv_launch<Acc, X_GLOBAL>(m, k, rows, cols, A, lda, x, y, sm_count, s, proj);
     // rows that 16-byte loads take as they are, or not
-    if ((((uintptr_t)A) & 15u) == 0 && lda % 4 == 0)
-        return mv_launch<Acc, X_SMEM>(m, k, rows, cols, A, lda, x, y, sm_count, s, proj);
-    return mv_launch<Acc, X_PLANES>(m, k, rows, cols, A, lda, x, y, sm_count, s, proj);
+    const bool vec = (((uintptr_t)A) & 15u) == 0 && lda % 4 == 0;
+    const bool words = !vec && cols <= MV_WORDS;
+    if (words || ((cols + 3) & ~3ull) * 4 > MV_XS_MAX)
+        return mv_launch<Acc, X_GLOBAL, MV_GLOBAL_U, MV_GLOBAL_THREADS>(m, k, rows, cols, A, lda, x, y, sm_count, s,
+                                                                        proj);
+    if (cols <= MV_SHORT)
+        return vec ? mv_launch<Acc, X_SMEM, MV_SHORT_U, MV_SHORT_THREADS>(m, k, rows, cols, A, lda, x, y, sm_count, s,
+                                                                          proj)
+                   : mv_launch<Acc, X_PLANES, MV_SHORT_U, MV_SHORT_THREADS>(m, k, rows, cols, A, lda, x, y, sm_count,
+                                                                            s, proj);
+    return vec ? mv_launch<Acc, X_SMEM, MV_U, MV_THREADS>(m, k, rows, cols, A, lda, x, y, sm_count, s, proj)
+               : mv_launch<Acc, X_PLANES, MV_U, MV_THREADS>(m, k, rows, cols, A, lda, x, y, sm_count, s, proj);
 }
 
 cudaError_t launch_matvec(Repr r, const Mod &m, uint64_t k, uint64_t rows, uint64_t cols,
