@@ -271,7 +271,7 @@ GFP_API gfp_status gfp_matvec_sequence(gfp_ctx *ctx, uint32_t p, uint64_t n, con
  * launch recombining the residues with
  * Garner's method modulo p, where that is expected to be faster than the
  * CUDA cores.  Rows of A at other alignments take the same kernel with 4-byte
- * loads.  Otherwise the CUDA-core kernel with the
+ * loads where k exceeds 12.  Otherwise the CUDA-core kernel with the
  * representation forced on the context, else the built-in rule for p (tuned
  * plans time the dot-product kernels and do not apply here; forcing F16TC
  * where the tensor cores are not eligible gives GFP_ERR_UNSUPPORTED).

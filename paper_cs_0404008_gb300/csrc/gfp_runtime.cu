@@ -899,6 +899,25 @@ static bool block_small_large_modulus(int L, uint64_t m, uint64_t k, uint64_t nb
     return mk * (double)nb / 4.5e12 <= L * (25e-6 + 4.0 * mk / 4.0e12);
 }
 
+// Expected microseconds of the residue passes: a pass has two or three launches,
+// reads A once for each 64 columns (5.3 TB/s), drains 64 columns of every row for
+// each, and moves its results a few times (2.2 TB/s).
+static double block_rns_us(int L, uint64_t m, uint64_t k, uint64_t nb)
+{
+    const double tiles = (double)((nb + 63) / 64), rows = (double)m * 1e-6;
+    return 3.0 + L * (7.6 + rows * (0.75 * (double)k * tiles + 0.47 * 64.0 * tiles + 7.2 * (double)nb));
+}
+
+// Expected microseconds on the CUDA cores: a CTA takes 64 x 64 outputs; the time of
+// an SM's CTAs, or of one alone, in sums that count wraps or plain ones.
+static double block_cc_us(Repr r, uint64_t m, uint64_t k, uint64_t nb, int sm_count)
+{
+    const double ctas = (double)((m + 63) / 64) * (double)((nb + 63) / 64);
+    const bool plain = r == U64_BLOCK;
+    if (ctas <= sm_count) return 7.1 + (plain ? 0.39 : 0.118) * (double)k;
+    return 4.5 + std::ceil(ctas / sm_count) * (2.3 + (plain ? 0.195 : 0.102) * (double)k);
+}
+
 static gfp_status launch_block(gfp_ctx *ctx, const BlockCall &q, const BlockScratch &sc, uint32_t *R, cudaStream_t s)
 {
     const bool many = q.n_mod() > 1;
@@ -987,20 +1006,17 @@ GFP_API gfp_status gfp_matmul_block(gfp_ctx *ctx, uint32_t p, uint64_t m, uint64
     bool own_scratch = ctx->forced == GFP_REPR_AUTO && !vec_ok;
     const bool layout_ok = ctx->forced == GFP_REPR_AUTO || vec_ok;
     RnsConst rc;
-    const bool direct_ok = layout_ok && p <= BLOCK_TC_MAX_P;
+    // a dozen terms are soonest summed where they are read: unaligned 16384 x 8 x
+    // 200 28.5 us on the tensor cores, 18 on the CUDA cores, 16384 x 16 x 200 27 and 31
+    const bool direct_ok = layout_ok && p <= BLOCK_TC_MAX_P && (vec_ok || k > 12);
     bool rns_ok = layout_ok && p > BLOCK_TC_MAX_P && block_rns_plan(p, k, &rc);
     if (rns_ok && ctx->forced == GFP_REPR_AUTO) {
-        // A residue pass costs about 10 us before its traffic (its own launch, its
-        // finishing launch, a partly filled wave), then A once at about 4.5 TB/s
-        // and its result three times.  A CTA of the CUDA-core kernel takes 0.134 us
-        // per term for its 64 x 64 outputs, an SM as long for each CTA it holds.
-        // Measured (us, residues / CUDA cores): 256 x 256 x 64 over GF(2^26 - 5)
-        // 45 / 42, 512 x 512 x 64 45 / 76, 1024 x 1024 x 64 45 / 144,
-        // 256 x 16384 x 64 71 / 2172, 16384 x 256 x 64 70 / 66, 4096 x 64 x 64 46 / 17
-        const double ctas = (double)((m + 63) / 64) * (double)((nb + 63) / 64);
-        const double t_rns = 5e-6 + rc.L * (10e-6 + (4.0 * (double)m * (double)k + 16.0 * (double)m * (double)nb) / 4.5e12);
-        const double t_cc = 7e-6 + (double)k * 0.134e-6 * std::max(1.0, ctas / ctx->sm_count);
-        if (t_cc <= t_rns) rns_ok = false;
+        // the residue passes have to be expected a fifth faster: the estimates are
+        // within a tenth on average (a third at most) over 1216 shapes of 64 to 65536
+        // rows, 1 to 1024 terms and columns.  Measured (us, residues / CUDA cores) over
+        // GF(2^31 - 1): 500 x 200 x 64 49 / 29, 500 x 1024 x 64 49 / 126,
+        // 16384 x 200 x 200 242 / 158, 16384 x 1024 x 200 355 / 721
+        if (1.2 * block_rns_us(rc.L, m, k, nb) >= block_cc_us(default_repr(p), m, k, nb, ctx->sm_count)) rns_ok = false;
         if (block_small_large_modulus(rc.L, m, k, nb)) own_scratch = true;
     }
     // such a call takes the tensor cores with scratch from a pool, else (a captured

@@ -134,7 +134,9 @@ def test_wide_free_calls_and_the_other_calls(lib):
     the context's workspace still use that and fail to grow it under capture."""
     fake_cuda.run("""
 c = context()
-assert block(c, 65521, 7, 9, 65535 * 64 + 1) == 0
+assert block(c, 65521, 7, 21, 65535 * 64) == 0
+assert count(kernels(), "k_block_tc") == 1
+assert block(c, 65521, 7, 21, 65535 * 64 + 1) == 0
 assert count(kernels(), "k_block_cc") == 1
 base = F.fake_used()
 assert block(c, 65521, 4096, 4096, 64) == 0 and F.fake_used() > base
@@ -174,4 +176,23 @@ assert F.cudaDeviceSynchronize() != 0
 mode = ctypes.c_int(0)
 F.cudaThreadExchangeStreamCaptureMode(ctypes.byref(mode))
 assert mode.value == 0
+""")
+
+
+# (p, m, k, nb, rows of A padded by, tensor cores): each side of the rules that choose
+ROUTES = [(65521, 16384, 8, 200, 1, False), (65521, 16384, 12, 200, 1, False), (65521, 16384, 13, 200, 0, True),
+          (65521, 16384, 8, 200, 0, True), (65521, 16384, 1, 1, 0, False), (65521, 64, 64, 64, 1, True),
+          (2147483647, 500, 200, 64, 0, False), (2147483647, 500, 1024, 64, 0, True),
+          (2147483647, 16384, 200, 200, 1, False), (2147483647, 16384, 1024, 200, 1, True),
+          (2147483647, 8192, 8192, 64, 0, True), (67108859, 65536, 64, 512, 0, False),
+          (67108859, 256, 16384, 64, 1, True), (100003, 500, 200, 64, 0, True), (100003, 500, 32, 64, 0, False)]
+
+
+def test_routes_on_each_side_of_the_rules(lib):
+    fake_cuda.run(f"""
+c = context()
+for p, m, k, nb, pad, tc in {ROUTES}:
+    assert block(c, p, m, k, nb, lda=k + pad) == 0
+    ks = kernels()
+    assert (count(ks, "k_block_tc") > 0) == tc and (count(ks, "k_block_cc") == 0) == tc, (p, m, k, nb, pad, ks)
 """)
