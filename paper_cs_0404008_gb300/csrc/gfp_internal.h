@@ -262,8 +262,8 @@ struct gfp_ctx {
     void *blk_ws = nullptr;
     size_t blk_ws_bytes = 0, blk_tail_bytes = 0;   // sizes of the two parts
     uint32_t *blk_err = nullptr;                   // error word of all block products
-    // stream-ordered scratch of the block products that keep none in the buffer, or
-    // null; made with the context, for making it may be refused during a capture
+    // stream-ordered scratch of the block products that keep none in the buffer; made
+    // by the first of them (50 us)
     cudaMemPool_t blk_pool = nullptr;
 
     // tuned plan: (p, lg_n) -> entry

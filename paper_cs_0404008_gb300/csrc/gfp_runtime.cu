@@ -456,9 +456,7 @@ GFP_API gfp_status gfp_context_create(int device, gfp_ctx **out)
     c->ring_slots = (unsigned long long *)mem;
     c->d_flag = (uint32_t *)((char *)mem + ring_bytes);
     c->blk_err = (uint32_t *)((char *)mem + ring_bytes + 128);
-    c->blk_pool = make_scratch_pool(device);
     if (cudaDeviceSynchronize() != cudaSuccess) {
-        if (c->blk_pool) cudaMemPoolDestroy(c->blk_pool);
         cudaFree(mem);
         delete c;
         return GFP_ERR_CUDA;
@@ -943,9 +941,10 @@ static gfp_status run_block_tc(gfp_ctx *ctx, const BlockCall &q, cudaStream_t s)
     return st == GFP_OK ? launch_block(ctx, q, sc, R, s) : st;
 }
 
-// Allocating and freeing in stream order is refused, and ends the capture, while a
-// stream of any thread is being captured in the mode that watches them all; it has
-// nothing to do with that capture, so this thread asks not to be watched.
+// Making a pool, and allocating and freeing in stream order, is refused, and ends the
+// capture, while a stream of any thread is being captured in the mode that watches
+// them all; it has nothing to do with that capture, so this thread asks not to be
+// watched.
 struct Unwatched {
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     Unwatched() { cudaThreadExchangeStreamCaptureMode(&mode); }
@@ -959,9 +958,14 @@ struct Unwatched {
 // is none.
 static gfp_status run_block_tc_pool(gfp_ctx *ctx, const BlockCall &q, cudaStream_t s)
 {
-    const cudaMemPool_t pool = ctx->blk_pool;
-    if (!pool) return GFP_ERR_NOMEM;
     const Unwatched unwatched;
+    cudaMemPool_t pool;
+    {
+        std::lock_guard<std::mutex> g(ctx->mu);
+        if (!ctx->blk_pool) ctx->blk_pool = make_scratch_pool(ctx->device);
+        pool = ctx->blk_pool;
+    }
+    if (!pool) return GFP_ERR_NOMEM;
     BlockScratch sc;
     sc.at_once = block_tc_moduli_at_once(q.k, q.nb, q.n_mod());
     void *mem = nullptr;

@@ -116,7 +116,12 @@ cudaError_t cudaFree(void *p) { return give(p); }
 cudaError_t cudaMemset(void *, int, size_t) { return cudaSuccess; }
 cudaError_t cudaMemsetAsync(void *, int, size_t n, cudaStream_t) { note("memset " + std::to_string(n)); return cudaSuccess; }
 cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind) { memcpy(d, s, n); return cudaSuccess; }
-cudaError_t cudaMemPoolCreate(cudaMemPool_t *p, const cudaMemPoolProps *) { *p = (cudaMemPool_t)&blocks; return cudaSuccess; }
+cudaError_t cudaMemPoolCreate(cudaMemPool_t *p, const cudaMemPoolProps *)
+{
+    if (captured && mode != cudaStreamCaptureModeRelaxed) return err(cudaErrorStreamCaptureUnsupported);
+    *p = (cudaMemPool_t)&blocks;
+    return cudaSuccess;
+}
 cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void *) { return cudaSuccess; }
 cudaError_t cudaMemPoolDestroy(cudaMemPool_t) { note("pool destroyed"); return cudaSuccess; }
 cudaError_t cudaMallocFromPoolAsync(void **p, size_t n, cudaMemPool_t, cudaStream_t s)
