@@ -11,6 +11,7 @@
 // The last CTA returns slots and tickets to zero, so the scratch is reusable by
 // the next launch without a memset.
 #include <algorithm>
+#include <type_traits>
 
 #include "gfp_internal.h"
 
@@ -58,8 +59,12 @@ __device__ __forceinline__ void accumulate_range(Acc &acc, const Mod &m, const u
 #pragma unroll
             for (int u = 0; u < U; ++u) acc.add4(a[u], c[u], m);
         }
-        // at most U - 1 vectors left: one batch, so one memory latency
-        if (v < nv) {
+        // at most U - 1 vectors left: one batch, so one memory latency; where the
+        // arithmetic is the time, only the vectors that there are (3000 pairs of
+        // 1000 terms in FP64 43 us, 66 with a batch filled up by zeros)
+        if constexpr (std::is_same<Acc, AccF64>::value || std::is_same<Acc, AccPerTerm>::value) {
+            for (; v < nv; v += T) acc.add4(ld_stream4(xv + v), ld_stream4(yv + v), m);
+        } else if (v < nv) {
             uint4 a[U - 1], c[U - 1];
 #pragma unroll
             for (int u = 0; u < U - 1; ++u) {
