@@ -33,18 +33,22 @@
 // words would lie four apart, a four-way bank conflict).  The fewer than four
 // elements before the first and after the last vector are added by themselves.  Such
 // rows of at most 64 columns, a word or two a lane, are read word by word (200000 x
-// 16 over GF(65521): 44 against 55 us).
+// 16 over GF(65521): 44 against 55 us), in FP64, where each pass over the lanes
+// costs, up to 256 (200000 x 200: 360 against 408 us).
 #include <algorithm>
+#include <type_traits>
 
 #include "gfp_internal.h"
 
 namespace gfp {
 
 // Threads and vectors a lane loads at a time, two batches in flight: for rows of
-// more than MV_SHORT columns, for shorter ones; and, one batch in flight, for rows whose
-// x is not in shared memory.
+// more than MV_SHORT columns, for shorter ones, for a remainder at every term (which
+// bounds the time: 32 warps, 3000 x 5000 23.4 us, 30.4 in 16); and, one batch in
+// flight, for rows whose x is not in shared memory.
 constexpr int MV_THREADS = 512, MV_U = 8;
 constexpr int MV_SHORT_THREADS = 1024, MV_SHORT_U = 2;
+constexpr int MV_TERM_THREADS = 1024, MV_TERM_U = 4;
 constexpr int MV_GLOBAL_THREADS = 1024, MV_GLOBAL_U = 4;
 constexpr uint64_t MV_SHORT = 256, MV_WORDS = 64;   // columns
 constexpr uint32_t MV_GLOBAL_WINDOW = 64;           // rows
@@ -343,17 +347,23 @@ static cudaError_t mv_dispatch(const Mod &m, uint64_t k, uint64_t rows, uint64_t
 {
     // rows that 16-byte loads take as they are, or not
     const bool vec = (((uintptr_t)A) & 15u) == 0 && lda % 4 == 0;
-    const bool words = !vec && cols <= MV_WORDS;
+    const bool words = !vec && cols <= (std::is_same<Acc, AccF64>::value ? MV_SHORT : MV_WORDS);
     if (words || ((cols + 3) & ~3ull) * 4 > MV_XS_MAX)
         return mv_launch<Acc, X_GLOBAL, MV_GLOBAL_U, MV_GLOBAL_THREADS>(m, k, rows, cols, A, lda, x, y, sm_count, s,
                                                                         proj);
-    if (cols <= MV_SHORT)
+    if constexpr (std::is_same<Acc, AccPerTerm>::value)
+        return vec ? mv_launch<Acc, X_SMEM, MV_TERM_U, MV_TERM_THREADS>(m, k, rows, cols, A, lda, x, y, sm_count, s,
+                                                                        proj)
+                   : mv_launch<Acc, X_PLANES, MV_TERM_U, MV_TERM_THREADS>(m, k, rows, cols, A, lda, x, y, sm_count, s,
+                                                                          proj);
+    else if (cols <= MV_SHORT)
         return vec ? mv_launch<Acc, X_SMEM, MV_SHORT_U, MV_SHORT_THREADS>(m, k, rows, cols, A, lda, x, y, sm_count, s,
                                                                           proj)
                    : mv_launch<Acc, X_PLANES, MV_SHORT_U, MV_SHORT_THREADS>(m, k, rows, cols, A, lda, x, y, sm_count,
                                                                             s, proj);
-    return vec ? mv_launch<Acc, X_SMEM, MV_U, MV_THREADS>(m, k, rows, cols, A, lda, x, y, sm_count, s, proj)
-               : mv_launch<Acc, X_PLANES, MV_U, MV_THREADS>(m, k, rows, cols, A, lda, x, y, sm_count, s, proj);
+    else
+        return vec ? mv_launch<Acc, X_SMEM, MV_U, MV_THREADS>(m, k, rows, cols, A, lda, x, y, sm_count, s, proj)
+                   : mv_launch<Acc, X_PLANES, MV_U, MV_THREADS>(m, k, rows, cols, A, lda, x, y, sm_count, s, proj);
 }
 
 cudaError_t launch_matvec(Repr r, const Mod &m, uint64_t k, uint64_t rows, uint64_t cols,
