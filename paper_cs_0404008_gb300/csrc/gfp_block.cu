@@ -67,6 +67,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 #include <mutex>
 
@@ -1131,7 +1132,7 @@ cudaError_t launch_block_tc(const uint32_t *mods, int n_mod, uint64_t m, uint64_
     static const Kernel kernels[5] = {k_block_tc<A_VEC, false>, k_block_tc<A_VEC, true>,
                                       k_block_tc<A_ANY, false>, k_block_tc<A_ANY, true>,
                                       k_block_tc<A_PREP, false>};
-    static bool attr = false;
+    static std::atomic<bool> attr{false};   // products of several threads may be the first
     if (!attr) {
         for (Kernel f : kernels) {
             cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -1,6 +1,8 @@
 """Block products by the scratch they have: B's tiles for one residue modulus at a
 time where those of all would be too large; and calls that need nothing of the
 context, on several streams at once and captured without a call before."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -74,6 +76,37 @@ def test_streams_of_one_context_at_once(lib, p, m, k, nb):
         assert lib.gfp_context_check(c) == lib.GFP_OK
     finally:
         c.close()
+
+
+@pytest.mark.parametrize("p,m,k,nb", FREE[:4])
+def test_threads_of_one_context_at_once(lib, p, m, k, nb):
+    """Two threads with a stream each and no order between them, and two on one
+    stream."""
+    for streams in ([torch.cuda.Stream(), torch.cuda.Stream()], [torch.cuda.Stream()] * 2):
+        A, B, C, want = operands(p, m, k, nb, 2)
+        c = lib.Context(0)
+        try:
+            torch.cuda.synchronize()
+            errors = []
+
+            def work(i):
+                try:
+                    for _ in range(20):
+                        lib.gfp_matmul_block(c, p, A[i], B[i], C[i], stream=streams[i])
+                except Exception as e:
+                    errors.append(e)
+
+            threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+            for t in threads:
+                t.start()
+            for t in threads:
+                t.join()
+            torch.cuda.synchronize()
+            assert not errors
+            assert all(np.array_equal(host(C[i]), want[i]) for i in range(2))
+            assert lib.gfp_context_check(c) == lib.GFP_OK
+        finally:
+            c.close()
 
 
 @pytest.mark.parametrize("p,m,k,nb", FREE)
